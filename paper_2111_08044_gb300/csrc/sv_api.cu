@@ -19,6 +19,7 @@
 #include "sv_block.h"
 #include "sv_internal.h"
 #include "sv_kernels.h"
+#include "sv_tile.h"
 
 using fsv::cd;
 
@@ -61,6 +62,16 @@ struct sv_ctx {
   fsv::BlockPlan* block = nullptr;  // block-mode plan and buffers
   std::vector<fsv::MultiArgs> mg;   // multi-gate passes of a period
   int* d_mg = nullptr;              // their gate indices and tile bits
+  // plain mode: the period's tile passes (none on chains too short for them,
+  // which take one launch per gate)
+  struct TileLaunch {
+    fsv::TileArgs ta;
+    int grid = 0;
+    std::unique_ptr<fsv::TileTab<fsv::kTileMaxGates>> tab;  // complex64, fixed gates
+  };
+  std::vector<TileLaunch> tiles;
+  bool tile_single = false;  // one tile holds the chain: whole periods in one launch
+  long long part_pairs = 0;  // partial pairs of a period
 
   cudaGraphExec_t graph = nullptr;       // one period
   cudaGraphExec_t graph_exit = nullptr;  // an evolution's last period (block plans
@@ -143,6 +154,8 @@ void free_build(sv_ctx* ctx) {
   cudaFree(ctx->d_mg);
   ctx->d_mg = nullptr;
   ctx->mg.clear();
+  ctx->tiles.clear();
+  ctx->tile_single = false;
   if (ctx->block) {
     fsv::block_free(ctx->block);
     ctx->block = nullptr;
@@ -196,9 +209,40 @@ int enqueue_multigate_period(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev) {
   return SV_OK;
 }
 
+// `periods` periods of a chain that one tile holds, in one launch.
+int enqueue_tile_run(sv_ctx* ctx, int64_t periods, cudaStream_t s) {
+  fsv::TileArgs ta = ctx->tiles[0].ta;
+  ta.periods = (int)periods;
+  SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, ta, ctx->tiles[0].tab.get(), 1, s), "tile launch");
+  return SV_OK;
+}
+
+// One period in tile passes; ev (nullable): one event before each launch and
+// one after the last.
+int enqueue_tile_period(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev) {
+  size_t k = 0;
+  if (ctx->tile_single) {
+    if (ev) SV_CUDA(cudaEventRecord(ev[k++], s), "event record");
+    int rc = enqueue_tile_run(ctx, 1, s);
+    if (rc) return rc;
+  } else {
+    for (const auto& t : ctx->tiles) {
+      if (ev) SV_CUDA(cudaEventRecord(ev[k++], s), "event record");
+      SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, t.ta, t.tab.get(), t.grid, s), "tile launch");
+    }
+    if (ev) SV_CUDA(cudaEventRecord(ev[k++], s), "event record");
+    SV_CUDA(fsv::launch_period_reduce(ctx->d_part_evolve, ctx->part_pairs, ctx->L, ctx->d_ring,
+                                      kRing, ctx->d_counter, 1, s),
+            "period reduce launch");
+  }
+  if (ev) SV_CUDA(cudaEventRecord(ev[k], s), "event record");
+  return SV_OK;
+}
+
 // Enqueue one plain-mode period on stream s.
 int enqueue_plain_period(sv_ctx* ctx, cudaStream_t s) {
   if (ctx->params.mode == SV_MODE_MULTIGATE) return enqueue_multigate_period(ctx, s, nullptr);
+  if (!ctx->tiles.empty()) return enqueue_tile_period(ctx, s, nullptr);
   const int ng = (int)ctx->gates.size();
   const size_t cbytes = amp_bytes(ctx->precision);
   const long long stride = ctx->n_period_params > 0 ? (long long)ng * fsv::kGateEntries : 0;
@@ -252,6 +296,7 @@ int capture_period(sv_ctx* ctx, bool last, cudaGraphExec_t* out) {
 }
 
 int ensure_graph(sv_ctx* ctx) {
+  if (ctx->tile_single) return SV_OK;  // launched directly
   if (!ctx->graph) {
     int rc = capture_period(ctx, false, &ctx->graph);
     if (rc) return rc;
@@ -266,6 +311,12 @@ int ensure_graph(sv_ctx* ctx) {
 int launch_periods(sv_ctx* ctx, int64_t count, bool last) {
   const bool off = off_natural(ctx);
   if (count <= 0) return SV_OK;
+  if (ctx->tile_single) {
+    int rc = enqueue_tile_run(ctx, count, ctx->stream);
+    if (rc) return rc;
+    ctx->counter += count;
+    return SV_OK;
+  }
   if (off && !ctx->in_period_layout) {
     cudaError_t e = fsv::block_enqueue_entry(ctx->block, ctx->state, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "relabel launch");
@@ -310,8 +361,12 @@ int ctx_capture_run(sv_ctx* ctx, int64_t periods, cudaGraph_t* out) {
     cudaError_t e = fsv::block_enqueue_entry(ctx->block, ctx->state, ctx->cap_stream);
     if (e != cudaSuccess) rc = cuda_fail(ctx, e, "relabel launch");
   }
-  for (int64_t k = 0; k < periods && rc == SV_OK; ++k)
-    rc = enqueue_period(ctx, ctx->cap_stream, k + 1 == periods);
+  if (ctx->tile_single) {
+    if (periods > 0) rc = enqueue_tile_run(ctx, periods, ctx->cap_stream);
+  } else {
+    for (int64_t k = 0; k < periods && rc == SV_OK; ++k)
+      rc = enqueue_period(ctx, ctx->cap_stream, k + 1 == periods);
+  }
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(ctx->cap_stream, &g);
   if (rc != SV_OK) {
@@ -619,6 +674,7 @@ int enqueue_period_profiled(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev, bool l
     return SV_OK;
   }
   if (ctx->params.mode == SV_MODE_MULTIGATE) return enqueue_multigate_period(ctx, s, ev);
+  if (!ctx->tiles.empty()) return enqueue_tile_period(ctx, s, ev);
   const int ng = (int)ctx->gates.size();
   const size_t cbytes = amp_bytes(ctx->precision);
   const long long stride = ctx->n_period_params > 0 ? (long long)ng * fsv::kGateEntries : 0;
@@ -714,6 +770,116 @@ int build_multigate(sv_ctx* ctx, const std::vector<fsv::MultiPass>& plan) {
   return SV_OK;
 }
 
+// The tile passes of a plain-mode period (none on chains too short for them):
+// their rounds on the device, the launch arguments, the partial pairs.
+// host_tab: the first period's complex64 tables.
+int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab) {
+  const int L = ctx->L, ng = (int)ctx->gates.size();
+  const int tb = fsv::tile_bits(L, ctx->gates, ctx->precision, ctx->cfg.num_sms);
+  if (tb == 0) return SV_OK;
+  const auto plan = fsv::tile_plan(L, ctx->gates, ctx->precision, tb);
+  if (plan.empty()) return SV_OK;
+  std::vector<fsv::TileRound> rounds;
+  for (const auto& p : plan) rounds.insert(rounds.end(), p.rounds.begin(), p.rounds.end());
+  ctx->tile_single = plan.size() == 1 && tb == L;
+  const size_t cb = amp_bytes(ctx->precision);
+  size_t round_at = 0;
+  ctx->part_pairs = 0;
+  for (const auto& p : plan) {
+    sv_ctx::TileLaunch t;
+    fsv::TileArgs& ta = t.ta;
+    ta.L = L;
+    ta.tb = tb;
+    ta.ngates = (int)p.gates.size();
+    ta.nrounds = (int)p.rounds.size();
+    ta.direct_out = p.direct_out ? 1 : 0;
+    ta.first = round_at == 0 ? 1 : 0;
+    int nr = 0;
+    for (int q = 0; q < tb; ++nr) {  // the tile's bits, in runs of consecutive state bits
+      int len = 1;
+      while (q + len < tb && p.bits[q + len] == p.bits[q] + len) ++len;
+      if (nr == fsv::kTileRuns) return fail(ctx, SV_EINVAL, "tile of too many runs");
+      ta.erun_m[nr] = (uint16_t)(((1u << len) - 1) << q);
+      ta.erun_s[nr] = (uint8_t)(p.bits[q] - q);
+      q += len;
+    }
+    // the other state bits, in runs of consecutive ones
+    int s = 0;
+    nr = 0;
+    for (int q = 0, i = 0; q < L;) {
+      if (i < tb && p.bits[i] == q) {
+        ++i;
+        ++q;
+        continue;
+      }
+      int len = 0;
+      while (q + len < L && !(i < tb && p.bits[i] == q + len)) ++len;
+      if (nr == fsv::kTileRuns) return fail(ctx, SV_EINVAL, "tile of too many runs");
+      ta.run_s[nr] = (uint8_t)s;
+      ta.run_d[nr] = (uint8_t)q;
+      ta.run_m[nr] = (uint32_t)((1ull << len) - 1);
+      ++nr;
+      s += len;
+      q += len;
+    }
+    ta.gates = static_cast<const char*>(ctx->d_gates) + (size_t)p.gates[0] * fsv::kGateEntries * cb;
+    ta.stride = ctx->n_period_params > 0 ? (long long)ng * fsv::kGateEntries : 0;
+    ta.counter = ctx->d_counter;
+    int epi = 0;
+    for (int g : p.gates) epi |= ctx->gates[g].epi;
+    ta.ep = epi_for(ctx, epi & fsv::EPI_DIAG, 0, nullptr);
+    for (int i = 0; i < L && !ctx->obs.general; ++i) ta.cx[i] = ctx->obs.cx[i];
+    if (ta.first) ta.ep.rn = renorm_of(ctx);
+    if (ctx->precision == SV_C64 && ta.stride == 0 && !ta.ep.rn.ring) {
+      ta.in_params = 1;
+      t.tab.reset(new fsv::TileTab<fsv::kTileMaxGates>());
+      for (size_t e = 0; e < p.gates.size() * fsv::kGateEntries; ++e) {
+        const float2 g = host_tab[(size_t)p.gates[0] * fsv::kGateEntries + e];
+        t.tab->g[0][e] = fsv::PackedEntry{{g.x, g.x}, {-g.y, g.y}};
+      }
+      std::memcpy(t.tab->r, p.rounds.data(), sizeof(fsv::TileRound) * p.rounds.size());
+    }
+    for (const auto& r : p.rounds) {
+      ta.any_xorder |= r.xorder[0] | r.xorder[1];
+      ta.any_epi |= r.epi[0] | r.epi[1];
+    }
+    // passes of one shape share the kernel's occupancy query
+    const fsv::TileArgs* like = nullptr;
+    for (const auto& o : ctx->tiles)
+      if (o.ta.ngates == ta.ngates && o.ta.nrounds == ta.nrounds && o.ta.in_params == ta.in_params &&
+          o.ta.any_xorder == ta.any_xorder && o.ta.any_epi == ta.any_epi) {
+        like = &o.ta;
+        t.grid = o.grid;
+      }
+    if (like) ta.buffers = like->buffers;
+    else SV_CUDA(fsv::tile_grid(ctx->precision, &ta, ctx->cfg, &t.grid), "tile pass setup");
+    if (p.measures) {
+      ta.ep.partial = ctx->d_part_evolve + 2 * ctx->part_pairs;
+      ctx->part_pairs += t.grid;
+    }
+    if (ctx->tile_single) {
+      ta.ring = ctx->d_ring;
+      ta.ring_len = kRing;
+      ta.counter_rw = ctx->d_counter;
+    }
+    round_at += p.rounds.size();
+    ctx->tiles.push_back(std::move(t));
+  }
+  // the rounds behind the gate tables (allocated with them)
+  const size_t bytes = rounds.size() * sizeof(fsv::TileRound);
+  char* d_rounds = static_cast<char*>(ctx->d_gates) + ctx->d_gates_bytes;
+  SV_CUDA(cudaMemcpy(d_rounds, rounds.data(), bytes, cudaMemcpyHostToDevice), "upload tile plan");
+  round_at = 0;
+  for (auto& t : ctx->tiles) {
+    t.ta.rounds = reinterpret_cast<fsv::TileRound*>(d_rounds) + round_at;
+    round_at += t.ta.nrounds;
+  }
+  ctx->passes_per_period = (int)plan.size();
+  ctx->launches_per_period = (int)plan.size() + (ctx->tile_single ? 0 : 1);
+  ctx->build_bytes = ctx->d_gates_bytes + bytes;
+  return SV_OK;
+}
+
 void upload_gates(const std::vector<fsv::Gate2>& gates, std::vector<float2>& out, size_t at) {
   for (size_t g = 0; g < gates.size(); ++g) {
     float2* e = &out[at + fsv::kGateEntries * g];
@@ -750,8 +916,9 @@ void upload_gates(const std::vector<fsv::Gate2>& gates, std::vector<double2>& ou
 
 // The gate tables of every period-parameter set, in the context's entry type.
 template <typename E>
-int upload_tables(sv_ctx* ctx, const sv_floquet_params& p, int64_t ntab, int ng) {
-  std::vector<E> tab((size_t)ntab * ng * fsv::kGateEntries);
+int upload_tables(sv_ctx* ctx, const sv_floquet_params& p, int64_t ntab, int ng,
+                  std::vector<E>& tab) {
+  tab.resize((size_t)ntab * ng * fsv::kGateEntries);
   for (int64_t k = 0; k < ntab; ++k) {
     auto gk = k == 0 ? ctx->gates : fsv::period_gates(ctx->L, p, ctx->theta_p[k], ctx->hx_p[k]);
     upload_gates(gk, tab, (size_t)k * ng * fsv::kGateEntries);
@@ -970,7 +1137,9 @@ int sv_build_floquet(sv_ctx* ctx, const sv_floquet_params* p) {
     const int64_t ntab = p->n_period_params > 0 ? p->n_period_params : 1;
     const size_t cb = amp_bytes(ctx->precision);
     ctx->d_gates_bytes = (size_t)ntab * ng * fsv::kGateEntries * cb;
-    if (cudaMalloc(&ctx->d_gates, ctx->d_gates_bytes) != cudaSuccess) {
+    // plain mode: at most one round per gate behind the tables
+    const size_t round_bytes = p->mode == SV_MODE_PLAIN ? (size_t)ng * sizeof(fsv::TileRound) : 0;
+    if (cudaMalloc(&ctx->d_gates, ctx->d_gates_bytes + round_bytes) != cudaSuccess) {
       cudaGetLastError();
       ctx->d_gates = nullptr;
       return fail(ctx, SV_ENOMEM, "gate table allocation failed");
@@ -994,17 +1163,18 @@ int sv_build_floquet(sv_ctx* ctx, const sv_floquet_params* p) {
     }
     SV_CUDA(cudaMemsetAsync(ctx->d_part_evolve, 0, pbytes, ctx->stream), "memset partials");
     int urc = SV_OK;
-    if (ctx->precision == SV_C128) urc = upload_tables<double2>(ctx, *p, ntab, ng);
-    else if (ctx->precision == SV_DF64) urc = upload_tables<float4>(ctx, *p, ntab, ng);
-    else urc = upload_tables<float2>(ctx, *p, ntab, ng);
+    std::vector<float2> host_tab;
+    std::vector<double2> tab64;
+    std::vector<float4> tab_df;
+    if (ctx->precision == SV_C128) urc = upload_tables(ctx, *p, ntab, ng, tab64);
+    else if (ctx->precision == SV_DF64) urc = upload_tables(ctx, *p, ntab, ng, tab_df);
+    else urc = upload_tables(ctx, *p, ntab, ng, host_tab);
     if (urc) return urc;
     ctx->passes_per_period = ng;
     ctx->launches_per_period = ng + 1;
     ctx->build_bytes = ctx->d_gates_bytes;
-    if (p->mode == SV_MODE_MULTIGATE) {
-      int rc = build_multigate(ctx, mplan);
-      if (rc) return rc;
-    }
+    const int rc = p->mode == SV_MODE_MULTIGATE ? build_multigate(ctx, mplan) : build_tiles(ctx, host_tab);
+    if (rc) return rc;
   }
   ctx->built = true;
   return SV_OK;
