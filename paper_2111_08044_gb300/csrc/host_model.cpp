@@ -251,6 +251,11 @@ std::vector<Gate2> period_gates(int L, const sv_floquet_params &p, double theta,
       for (int k = 0; k < 16; ++k) h[k] = cd(p.h_bonds[32 * b + 2 * k], p.h_bonds[32 * b + 2 * k + 1]);
     } else {
       bond_hamiltonian(L, b, p.J, hx, p.hz, p.edge_field_weight, h);
+      // all interior bonds share their term: one exponential for them
+      if (b >= 2 && b < L - 2) {
+        std::memcpy(&gb[16 * (size_t)b], &gb[16], 16 * sizeof(cd));
+        continue;
+      }
     }
     expm_herm4(h, tau, &gb[16 * (size_t)b]);
   }
@@ -348,6 +353,11 @@ std::vector<AdjOp> adjoint_period_ops(int L, const sv_floquet_params &p, double 
   const double tau = p.T / p.K;
   std::vector<AdjOp> gate_ops(L - 1);
   for (int b = 0; b < L - 1; ++b) {
+    if (b >= 2 && b < L - 2) {  // interior bonds share their term and derivative
+      gate_ops[b] = gate_ops[1];
+      gate_ops[b].bond = b;
+      continue;
+    }
     cd h[16], dh[16], g[16], dg[16], gd[16];
     bond_hamiltonian(L, b, p.J, hx, p.hz, p.edge_field_weight, h);
     bond_hamiltonian(L, b, 0.0, 1.0, 0.0, p.edge_field_weight, dh);

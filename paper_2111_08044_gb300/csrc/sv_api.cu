@@ -770,6 +770,40 @@ int build_multigate(sv_ctx* ctx, const std::vector<fsv::MultiPass>& plan) {
   return SV_OK;
 }
 
+// The state bits of a tile pass as TileArgs wants them (false: too many runs).
+bool tile_runs(int L, const fsv::TilePassPlan& p, fsv::TileArgs* ta) {
+  const int tb = (int)p.bits.size();
+  int nr = 0;
+  for (int q = 0; q < tb; ++nr) {  // the tile's bits, in runs of consecutive state bits
+    int len = 1;
+    while (q + len < tb && p.bits[q + len] == p.bits[q] + len) ++len;
+    if (nr == fsv::kTileRuns) return false;
+    ta->erun_m[nr] = (uint16_t)(((1u << len) - 1) << q);
+    ta->erun_s[nr] = (uint8_t)(p.bits[q] - q);
+    q += len;
+  }
+  // the other state bits, in runs of consecutive ones
+  int s = 0;
+  nr = 0;
+  for (int q = 0, i = 0; q < L;) {
+    if (i < tb && p.bits[i] == q) {
+      ++i;
+      ++q;
+      continue;
+    }
+    int len = 0;
+    while (q + len < L && !(i < tb && p.bits[i] == q + len)) ++len;
+    if (nr == fsv::kTileRuns) return false;
+    ta->run_s[nr] = (uint8_t)s;
+    ta->run_d[nr] = (uint8_t)q;
+    ta->run_m[nr] = (uint32_t)((1ull << len) - 1);
+    ++nr;
+    s += len;
+    q += len;
+  }
+  return true;
+}
+
 // The tile passes of a plain-mode period (none on chains too short for them):
 // their rounds on the device, the launch arguments, the partial pairs.
 // host_tab: the first period's complex64 tables.
@@ -794,34 +828,7 @@ int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab) {
     ta.nrounds = (int)p.rounds.size();
     ta.direct_out = p.direct_out ? 1 : 0;
     ta.first = round_at == 0 ? 1 : 0;
-    int nr = 0;
-    for (int q = 0; q < tb; ++nr) {  // the tile's bits, in runs of consecutive state bits
-      int len = 1;
-      while (q + len < tb && p.bits[q + len] == p.bits[q] + len) ++len;
-      if (nr == fsv::kTileRuns) return fail(ctx, SV_EINVAL, "tile of too many runs");
-      ta.erun_m[nr] = (uint16_t)(((1u << len) - 1) << q);
-      ta.erun_s[nr] = (uint8_t)(p.bits[q] - q);
-      q += len;
-    }
-    // the other state bits, in runs of consecutive ones
-    int s = 0;
-    nr = 0;
-    for (int q = 0, i = 0; q < L;) {
-      if (i < tb && p.bits[i] == q) {
-        ++i;
-        ++q;
-        continue;
-      }
-      int len = 0;
-      while (q + len < L && !(i < tb && p.bits[i] == q + len)) ++len;
-      if (nr == fsv::kTileRuns) return fail(ctx, SV_EINVAL, "tile of too many runs");
-      ta.run_s[nr] = (uint8_t)s;
-      ta.run_d[nr] = (uint8_t)q;
-      ta.run_m[nr] = (uint32_t)((1ull << len) - 1);
-      ++nr;
-      s += len;
-      q += len;
-    }
+    if (!tile_runs(L, p, &ta)) return fail(ctx, SV_EINVAL, "tile of too many runs");
     ta.gates = static_cast<const char*>(ctx->d_gates) + (size_t)p.gates[0] * fsv::kGateEntries * cb;
     ta.stride = ctx->n_period_params > 0 ? (long long)ng * fsv::kGateEntries : 0;
     ta.counter = ctx->d_counter;
@@ -880,10 +887,36 @@ int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab) {
   return SV_OK;
 }
 
+// Rounded 4x4 unitaries of one call: a period repeats a few matrices (interior
+// bonds, with and without the folded kicks) over its bonds and Trotter steps,
+// and the rounding's descent costs far more than the comparison.
+class RoundedGates {
+ public:
+  const float2* get(const cd* m) {
+    for (const auto& s : seen_)
+      if (std::memcmp(s->m, m, sizeof(s->m)) == 0) return s->f;
+    std::unique_ptr<Entry> e(new Entry);
+    std::memcpy(e->m, m, sizeof(e->m));
+    fsv::round_unitary4(m, e->f);
+    if (seen_.size() == kMost) seen_.erase(seen_.begin());
+    seen_.push_back(std::move(e));
+    return seen_.back()->f;
+  }
+
+ private:
+  static constexpr size_t kMost = 32;
+  struct Entry {
+    cd m[16];
+    float2 f[16];
+  };
+  std::vector<std::unique_ptr<Entry>> seen_;
+};
+
 void upload_gates(const std::vector<fsv::Gate2>& gates, std::vector<float2>& out, size_t at) {
+  RoundedGates rounded;
   for (size_t g = 0; g < gates.size(); ++g) {
     float2* e = &out[at + fsv::kGateEntries * g];
-    fsv::round_unitary4(gates[g].m, e);
+    std::memcpy(e, rounded.get(gates[g].m), 16 * sizeof(float2));
     for (int k = 0; k < 16; ++k)
       e[16 + k] = make_float2((float)(gates[g].m[k].real() - (double)e[k].x),
                               (float)(gates[g].m[k].imag() - (double)e[k].y));
@@ -928,6 +961,124 @@ int upload_tables(sv_ctx* ctx, const sv_floquet_params& p, int64_t ntab, int ng,
           "upload gates");
   SV_CUDA(cudaStreamSynchronize(ctx->stream), "synchronize");
   return SV_OK;
+}
+
+// ------------------------------------------------------------ adjoint sweep
+
+std::vector<fsv::Gate2> adjoint_bonds(const std::vector<fsv::AdjOp>& ops) {
+  std::vector<fsv::Gate2> g(ops.size());
+  for (size_t o = 0; o < ops.size(); ++o) g[o].bond = ops[o].bond;
+  return g;
+}
+
+int adjoint_tile_bits(const sv_ctx* ctx, const std::vector<fsv::AdjOp>& ops) {
+  return std::min(fsv::kAdjointTileBits,
+                  fsv::tile_bits(ctx->L, adjoint_bonds(ops), SV_C64, ctx->cfg.num_sms));
+}
+
+// The reverse sweep of sv_adjoint in tile passes (complex64): forward to
+// psi_P, lambda = (H0 / L) psi_P, then every period's operations from last to
+// first, several to a pass on tiles of both states.  tab: odag and d of every
+// period's operations.
+int adjoint_tiles(sv_ctx* ctx, int64_t P, const std::vector<fsv::AdjOp>& ops, int tb,
+                  const std::vector<float2>& tab, double* grad_theta, double* grad_hx,
+                  double* energy_density) {
+  const int L = ctx->L;
+  const auto plan = fsv::tile_plan(L, adjoint_bonds(ops), SV_C64, tb);
+  const int np = (int)plan.size();
+  size_t nkick = 0;  // the kick operations come first in each period's list
+  while (nkick < ops.size() && ops[nkick].kind == 0) ++nkick;
+  std::vector<fsv::AdjointPass> passes(np);
+  std::vector<int> grids(np);
+  int pairs = 0;  // partial pairs of a period
+  for (int i = 0; i < np; ++i) {
+    fsv::AdjointPass& ap = passes[i];
+    fsv::TileArgs& ta = ap.ta;
+    ta.L = L;
+    ta.tb = tb;
+    ta.ngates = (int)plan[i].gates.size();
+    ta.nrounds = (int)plan[i].rounds.size();
+    ta.direct_out = plan[i].direct_out ? 1 : 0;
+    if (!tile_runs(L, plan[i], &ta)) return fail(ctx, SV_EINVAL, "tile of too many runs");
+    ap.nkick = (int)std::max<int64_t>(
+        0, std::min<int64_t>((int64_t)nkick - plan[i].gates[0], ta.ngates));
+    SV_CUDA(fsv::adjoint_tile_grid(&ap, ctx->cfg, &grids[i]), "adjoint pass setup");
+    ap.pair_at = pairs;
+    pairs += grids[i];
+  }
+  // partial sums of as many periods as 32 MiB hold
+  const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(P, (32ll << 20) / (16ll * pairs)));
+  const int seed_grid = fsv::adjoint_grid(ctx->cfg);
+  void* d_lam = nullptr;
+  double* d_part = nullptr;
+  double* d_grad = nullptr;
+  auto release = [&]() {
+    cudaFree(d_lam);
+    cudaFree(d_part);
+    cudaFree(d_grad);
+  };
+  const size_t part_n = std::max<size_t>((size_t)chunk * pairs * 2, seed_grid);
+  if (cudaMalloc(&d_lam, (size_t)8 << L) != cudaSuccess ||
+      cudaMalloc(&d_part, sizeof(double) * part_n) != cudaSuccess ||
+      cudaMalloc(&d_grad, sizeof(double) * (2 * (size_t)P + 1)) != cudaSuccess) {
+    cudaGetLastError();
+    release();
+    return fail(ctx, SV_ENOMEM, "adjoint buffers (%zu bytes for lambda)", (size_t)8 << L);
+  }
+  auto run = [&]() -> int {
+    int r = sv_evolve(ctx, P, nullptr, nullptr);
+    if (r) return r;
+    fsv::H0Coef h;
+    h.J = ctx->obs.J;
+    for (int i = 0; i < L; ++i) {
+      h.cx[i] = ctx->obs.cx[i];
+      h.cz[i] = ctx->obs.cz[i];
+    }
+    SV_CUDA(fsv::launch_apply_h0(SV_C64, ctx->state, d_lam, L, h, d_part, ctx->cfg, ctx->stream),
+            "adjoint seed launch");
+    SV_CUDA(fsv::launch_grad_reduce(d_part, seed_grid, d_grad + 2 * P, 0, ctx->stream),
+            "energy reduce launch");
+    std::unique_ptr<fsv::TileTab<fsv::kTileMaxGates>> tt(new fsv::TileTab<fsv::kTileMaxGates>());
+    for (int64_t k1 = P; k1 > 0; k1 -= std::min(k1, chunk)) {
+      const int64_t k0 = k1 - std::min(k1, chunk);
+      for (int64_t k = k1 - 1; k >= k0; --k) {
+        const float2* period = &tab[(size_t)k * ops.size() * 32];
+        double* part = d_part + (size_t)(k - k0) * pairs * 2;
+        for (int i = 0; i < np; ++i) {
+          const fsv::TilePassPlan& p = plan[i];
+          for (size_t e = 0; e < p.gates.size() * 32; ++e) {
+            const float2 g = period[(size_t)p.gates[0] * 32 + e];
+            tt->g[0][e] = fsv::PackedEntry{{g.x, g.x}, {-g.y, g.y}};
+          }
+          std::memcpy(tt->r, p.rounds.data(), sizeof(fsv::TileRound) * p.rounds.size());
+          SV_CUDA(fsv::launch_adjoint_tile(ctx->state, d_lam, passes[i], *tt,
+                                           part + 2 * passes[i].pair_at, grids[i], ctx->stream),
+                  "adjoint pass launch");
+        }
+      }
+      SV_CUDA(fsv::launch_grad_reduce_pairs(d_part, pairs, (int)(k1 - k0), d_grad + 2 * k0,
+                                            ctx->stream),
+              "gradient reduce launch");
+    }
+    std::vector<double> hg(2 * (size_t)P + 1);
+    SV_CUDA(cudaMemcpyAsync(hg.data(), d_grad, sizeof(double) * hg.size(),
+                            cudaMemcpyDeviceToHost, ctx->stream),
+            "gradient readback");
+    // psi is back at its starting point: so is the period counter
+    SV_CUDA(cudaMemsetAsync(ctx->d_counter, 0, sizeof(long long), ctx->stream),
+            "reset counter");
+    SV_CUDA(cudaStreamSynchronize(ctx->stream), "synchronize");
+    for (int64_t k = 0; k < P; ++k) {
+      if (grad_theta) grad_theta[k] = hg[2 * k];
+      if (grad_hx) grad_hx[k] = hg[2 * k + 1];
+    }
+    if (energy_density) *energy_density = hg[2 * P];
+    ctx->counter = 0;
+    return SV_OK;
+  };
+  const int rc = run();
+  release();
+  return rc;
 }
 
 // SV_DF64 state read-out (to_host) or write-in as complex128 amplitudes,
@@ -1399,7 +1550,8 @@ int sv_adjoint(sv_ctx* ctx, int64_t periods, double* grad_theta, double* grad_hx
     tab64.resize(tab_elems);
   else
     tab32.resize(tab_elems);
-  for (int64_t k = 0; k < P; ++k)
+  for (int64_t k = 0; k < P; ++k) {
+    RoundedGates rounded;
     for (size_t o = 0; o < nop; ++o) {
       const fsv::AdjOp& op = ops[k][o];
       const size_t at = ((size_t)k * nop + o) * 32;
@@ -1409,11 +1561,16 @@ int sv_adjoint(sv_ctx* ctx, int64_t periods, double* grad_theta, double* grad_hx
           tab64[at + 16 + e] = make_double2(op.d[e].real(), op.d[e].imag());
         }
       } else {
-        fsv::round_unitary4(op.odag, &tab32[at]);
+        std::memcpy(&tab32[at], rounded.get(op.odag), 16 * sizeof(float2));
         for (int e = 0; e < 16; ++e)
           tab32[at + 16 + e] = make_float2((float)op.d[e].real(), (float)op.d[e].imag());
       }
     }
+  }
+  if (!c128) {
+    const int tb = adjoint_tile_bits(ctx, ops[0]);
+    if (tb) return adjoint_tiles(ctx, P, ops[0], tb, tab32, grad_theta, grad_hx, energy_density);
+  }
   const int grid = fsv::adjoint_grid(ctx->cfg);
   const size_t npart = nop * (size_t)grid;
   void* d_lam = nullptr;

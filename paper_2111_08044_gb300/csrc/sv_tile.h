@@ -117,4 +117,23 @@ cudaError_t tile_grid(int precision, TileArgs* ta, const LaunchCfg& cfg, int* gr
 cudaError_t launch_tile(int precision, void* psi, const TileArgs& ta,
                         const TileTab<kTileMaxGates>* tab, int grid, cudaStream_t s);
 
+// ------------------------------------------------------------ adjoint sweep
+// A pass of the reverse sweep on tiles of psi and lambda (complex64): operations
+// [0, nkick) of the pass differentiate the kick angle, the others the field.
+constexpr int kAdjointTileBits = 11;  // both states of a tile: 36 KiB
+struct AdjointPass {
+  TileArgs ta;
+  int nkick = 0;
+  int pair_at = 0;  // its partial pairs (kick, field) within the period's
+};
+cudaError_t adjoint_tile_grid(AdjointPass* ap, const LaunchCfg& cfg, int* grid);
+// tab: odag (16 entries) and d (16) per operation, and the rounds
+cudaError_t launch_adjoint_tile(void* psi, void* lam, const AdjointPass& ap,
+                                const TileTab<kTileMaxGates>& tab, double* part, int grid,
+                                cudaStream_t s);
+// out[2 k], out[2 k + 1] = 2 x the sums of period k's (kick, field) partial
+// pairs, periods `pairs` pairs apart, fixed order
+cudaError_t launch_grad_reduce_pairs(const double* part, int pairs, int periods, double* out,
+                                     cudaStream_t s);
+
 }  // namespace fsv
