@@ -1,0 +1,494 @@
+// Measurements of a complex64 state of at least 13 sites, in tiles of 2^12
+// amplitudes (on shorter chains a call is its launches and copies either way,
+// and the per-gate and per-amplitude kernels stay).  Times at L = 25 (256 MiB;
+// one read of it takes 40 us at the measured bandwidth):
+//
+//   k_energy_tile   <H0> of the driven chain and the norm: sums of <X> over the
+//                   bits of a tile, and the diagonal part.  A pass covers the
+//                   12 lowest sites or 8 further ones, so the state is read
+//                   ceil((L - 12) / 8) + 1 times; one identity gate pass per
+//                   pair of sites read it L / 2 times: 1160 -> 194 us.
+//   k_moments_tile  H0 psi amplitude by amplitude, for E and sigma_E (Eq. 10 and
+//                   11): partners within the tile from registers and shared
+//                   memory, the others from the tiles whose number differs in
+//                   one bit (or, for a general bond term, two), which mostly
+//                   are in L2.  Bound by that traffic: L - 11 tiles read for one
+//                   (Ising, 1230 -> 269 us), 2 (L - 12) (general bonds, L = 24:
+//                   1085 -> 330 us).
+//   k_overlap_f32   <phi|psi> of a product state from FP64 factor tables
+//   k_factor_f32    and the state itself: the FP64 units (0.59 TFMA/s) bounded
+//                   both; products and sums are FP32 pairs here (an exact
+//                   product and its error, Dekker and Knuth), moved to FP64
+//                   every 16 amplitudes: 741 -> 92 us; L = 24: 188 -> 30 us.
+// Partial sums: FP32 within a thread's tile, FP32 pairs across its terms, FP64
+// across tiles, threads and blocks, in a fixed order.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "sv_device.cuh"
+#include "sv_internal.h"
+#include "sv_kernels.h"
+#include "sv_tile.cuh"
+
+namespace fsv {
+
+namespace {
+
+using namespace dev;
+
+constexpr int kThreads = 256;
+constexpr int kBits = 12;  // tile bits: 16 amplitudes a thread
+constexpr uint32_t kTileBytes = 8u * (1u << kBits) + 16u * (1u << (kBits - 4));
+static_assert(kTileBytes <= 48 * 1024, "no shared-memory opt-in: the calls may be captured");
+
+// Deterministic block sums of K doubles, written to out[K * blockIdx.x + j].
+template <int K>
+__device__ void block_store_k(double (&v)[K], double* out) {
+  __shared__ double sh[K][32];
+#pragma unroll
+  for (int j = 0; j < K; ++j)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int j = 0; j < K; ++j) sh[j][w] = v[j];
+  __syncthreads();
+  if (threadIdx.x < K) {
+    double t = 0.0;
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sh[threadIdx.x][k];
+    out[K * blockIdx.x + threadIdx.x] = t;
+  }
+}
+
+// The diagonal part of H0 over a thread's amplitudes of one contiguous tile:
+// the tile number's share once, the low bits' per amplitude.
+struct TileDiag {
+  float J, cz_bulk, cz_first, cz_last, czsum;
+  int L, nb_hi, flips_hi, last;
+  uint32_t top;  // bit 0 of the tile number at the place above the tile's bits
+  __device__ void init(const EpiParams& ep, int L_) {
+    L = L_;
+    J = (float)ep.J;
+    cz_bulk = (float)ep.cz_bulk;
+    cz_first = (float)ep.cz_first;
+    cz_last = (float)ep.cz_last;
+    czsum = (float)(ep.cz_bulk * (L_ - 2) + ep.cz_first + ep.cz_last);
+  }
+  __device__ void tile(uint32_t t) {
+    const int hi = L - kBits;  // bits of the tile number, at least 1
+    flips_hi = __popc((t ^ (t >> 1)) & ((1u << (hi - 1)) - 1));
+    last = (t >> (hi - 1)) & 1;
+    nb_hi = __popc(t) - last;
+    top = (t & 1u) << kBits;
+  }
+  __device__ __forceinline__ float operator()(uint32_t e) const {
+    const uint32_t x = e | top;
+    const int flips = flips_hi + __popc((x ^ (x >> 1)) & ((1u << kBits) - 1));
+    const int nb = nb_hi + __popc(e & ~1u);
+    const float up = cz_bulk * (float)nb + ((e & 1) ? cz_first : 0.f) + (last ? cz_last : 0.f);
+    return J * (float)(L - 1 - 2 * flips) + czsum - 2.f * up;
+  }
+};
+
+struct EnergyArgs {
+  TileArgs ta;          // layout of the pass
+  float cx[kBits] = {};  // coefficient of each tile bit's <X> (0: another pass's)
+  int low = 0;          // tile bits 0..3 measured too
+  int diag = 0;
+};
+
+// 2 Re <v_0|v_1> over the eight pairs of register bit J
+template <int J>
+__device__ __forceinline__ float pair_sum(const float2 (&v)[16]) {
+  float s = 0.f;
+#pragma unroll
+  for (int m = 0; m < 16; ++m)
+    if (!(m & (1 << J))) s += cdotre(v[m], v[m | (1 << J)]);
+  return 2.f * s;
+}
+
+__global__ void __launch_bounds__(kThreads, 4)
+    k_energy_tile(const float2* __restrict__ psi, const __grid_constant__ EnergyArgs ea,
+                  double* __restrict__ part) {
+  extern __shared__ __align__(16) uint8_t tile[];
+  const TileArgs& ta = ea.ta;
+  const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(tile);
+  const uint32_t ntiles = 1u << (ta.L - kBits);
+  const uint32_t tid = threadIdx.x;
+  const TileIo io = tile_io(ta);
+  TileDiag dg;
+  if (ea.diag) dg.init(ta.ep, ta.L);
+  double acc[2] = {0.0, 0.0};
+  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    load_tile(ta, io, sbuf, psi + tile_base(ta, t));
+    cp_wait<0>();
+    __syncthreads();
+    FloatSum es, ns;
+    if (ea.diag) dg.tile(t);
+    // the tile three times over, each time with other register bits: 8-11,
+    // 4-7 and (where measured) 0-3
+#pragma unroll
+    for (int q = 8; q >= 0; q -= 4) {
+      if (q == 0 && !ea.low) break;
+      const uint32_t e0 = (tid & ((1u << q) - 1)) | ((tid >> q) << (q + 4));
+      float2 v[16];
+#pragma unroll
+      for (int m = 0; m < 16; ++m)
+        v[m] = *reinterpret_cast<const float2*>(tile + tile_byte8(e0 | ((uint32_t)m << q)));
+      es.add(ea.cx[q] * pair_sum<0>(v));
+      es.add(ea.cx[q + 1] * pair_sum<1>(v));
+      es.add(ea.cx[q + 2] * pair_sum<2>(v));
+      es.add(ea.cx[q + 3] * pair_sum<3>(v));
+      if (q == 8 && ea.diag) {
+        float d = 0.f, n = 0.f;
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+          const float p = cabs2(v[m]);
+          n += p;
+          d += p * dg(e0 | ((uint32_t)m << q));
+        }
+        es.add(d);
+        ns.add(n);
+      }
+    }
+    es.flush(acc[0]);
+    ns.flush(acc[1]);
+    __syncthreads();
+  }
+  block_store_k<2>(acc, part);
+}
+
+// ------------------------------------------------------------------ moments
+struct MomentArgs {
+  int L = 0;
+  float cx[34] = {};            // Ising: coefficients of X_i
+  EpiParams ep;                 // Ising: diagonal coefficients
+  float2 h[33][16] = {};        // general: bond terms
+};
+
+// One row of a bond term: out += sum_c h[r][c] w_c, w_c the amplitude with local
+// index c; r, like the amplitudes' order, only known at run time: the row's
+// entries are selected, not indexed.
+__device__ __forceinline__ float2 row_sum(const float2 (&h)[16], int r, float2 out, float2 same,
+                                          float2 lo, float2 hi, float2 both) {
+  // column r, r ^ 1 (site b + 1 flipped), r ^ 2 (site b flipped), r ^ 3
+  float2 d = h[0], l = h[1], u = h[2], x = h[3];
+  if (r == 1) d = h[5], l = h[4], u = h[7], x = h[6];
+  if (r == 2) d = h[10], l = h[11], u = h[8], x = h[9];
+  if (r == 3) d = h[15], l = h[14], u = h[13], x = h[12];
+  out = cmac(out, d, same);
+  out = cmac(out, l, lo);
+  out = cmac(out, u, hi);
+  return cmac(out, x, both);
+}
+
+// A thread's amplitudes: tile indices 2 tid + (0, 1) + 1024 j, j = 0..3 (bit 0 of
+// m: site 0, bits 1 and 2: sites 10 and 11), so that every read of another tile
+// is of whole lines; sites 1..9 are thread bits, their partners in the tile.
+// General bond terms hold four arrays of partners: one block an SM.
+constexpr int kMomentThreads = 512;
+constexpr int kAmps = 8;
+
+template <bool kBonds>
+__global__ void __launch_bounds__(kMomentThreads, kBonds ? 1 : 2)
+    k_moments_tile(const float2* __restrict__ psi, const __grid_constant__ MomentArgs ma,
+                   double* __restrict__ part) {
+  extern __shared__ __align__(16) uint8_t tile[];
+  const int L = ma.L;
+  const uint32_t ntiles = 1u << (L - kBits);
+  const uint32_t tid = threadIdx.x;
+  TileDiag dg;
+  if (!kBonds) dg.init(ma.ep, L);
+  double acc[3] = {0.0, 0.0, 0.0};
+  const uint32_t e0 = 2 * tid;
+  auto set = [](float2 (&u)[kAmps], int j, float4 q) {
+    u[2 * j] = make_float2(q.x, q.y);
+    u[2 * j + 1] = make_float2(q.z, q.w);
+  };
+  auto read = [&](uint32_t from, float2 (&u)[kAmps]) {
+    const float4* p = reinterpret_cast<const float4*>(psi + ((uint64_t)from << kBits));
+#pragma unroll
+    for (int j = 0; j < kAmps / 2; ++j) set(u, j, __ldg(p + tid + kMomentThreads * j));
+  };
+  auto partner = [&](uint32_t flip, float2 (&u)[kAmps]) {  // flip: tile bits 1..9
+#pragma unroll
+    for (int j = 0; j < kAmps / 2; ++j)
+      set(u, j, *reinterpret_cast<const float4*>(tile + tile_byte8((e0 ^ flip) + 1024 * j)));
+  };
+  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    float2 v[kAmps], hv[kAmps], a[kAmps];
+    read(t, v);
+#pragma unroll
+    for (int j = 0; j < kAmps / 2; ++j)
+      *reinterpret_cast<float4*>(tile + tile_byte8(e0 + 1024 * j)) =
+          make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
+    __syncthreads();
+    if (!kBonds) {
+      dg.tile(t);
+      auto add = [&](float c, const float2 (&u)[kAmps]) {
+#pragma unroll
+        for (int m = 0; m < kAmps; ++m) {
+          hv[m].x += c * u[m].x;
+          hv[m].y += c * u[m].y;
+        }
+      };
+#pragma unroll
+      for (int m = 0; m < kAmps; ++m) {
+        const float d = dg(e0 + 1024 * (m >> 1) + (m & 1));
+        hv[m] = make_float2(d * v[m].x, d * v[m].y);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {  // sites 0, 10, 11: within the thread
+          const float c = ma.cx[k == 0 ? 0 : 9 + k];
+          hv[m].x += c * v[m ^ (1 << k)].x;
+          hv[m].y += c * v[m ^ (1 << k)].y;
+        }
+      }
+#pragma unroll
+      for (int i = 1; i < 10; ++i) {
+        partner(1u << i, a);
+        add(ma.cx[i], a);
+      }
+#pragma unroll 4
+      for (int i = kBits; i < L; ++i) {
+        read(t ^ (1u << (i - kBits)), a);
+        add(ma.cx[i], a);
+      }
+    } else {
+      float2 b[kAmps], c[kAmps];
+      // (10, 11): within the thread
+#pragma unroll
+      for (int m = 0; m < kAmps; ++m) {
+        const int r = 2 * ((m >> 1) & 1) + (m >> 2);
+        hv[m] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          hv[m] = cmac(hv[m], ma.h[10][4 * r + q], v[(m & 1) | ((q >> 1) << 1) | ((q & 1) << 2)]);
+      }
+      // (0, 1)
+      partner(2, a);
+      const int s1 = tid & 1;
+#pragma unroll
+      for (int m = 0; m < kAmps; ++m)
+        hv[m] = row_sum(ma.h[0], 2 * (m & 1) + s1, hv[m], v[m], a[m], v[m ^ 1], a[m ^ 1]);
+      // (i, i + 1), i = 1..8: both thread bits; a holds site i's partner
+#pragma unroll 1
+      for (int i = 1; i < 9; ++i) {
+        partner(2u << i, b);
+        partner(3u << i, c);
+        const int r = 2 * (int)((tid >> (i - 1)) & 1) + (int)((tid >> i) & 1);
+#pragma unroll
+        for (int m = 0; m < kAmps; ++m) {
+          hv[m] = row_sum(ma.h[i], r, hv[m], v[m], b[m], a[m], c[m]);
+          a[m] = b[m];
+        }
+      }
+      // (9, 10)
+      const int s9 = (int)(tid >> 8);
+#pragma unroll
+      for (int m = 0; m < kAmps; ++m)
+        hv[m] = row_sum(ma.h[9], 2 * s9 + ((m >> 1) & 1), hv[m], v[m], v[m ^ 2], a[m], a[m ^ 2]);
+      // (11, 12): site 12 is the tile number's bit 0
+      read(t ^ 1u, a);
+      const int s12 = (int)(t & 1u);
+#pragma unroll
+      for (int m = 0; m < kAmps; ++m)
+        hv[m] = row_sum(ma.h[11], 2 * (m >> 2) + s12, hv[m], v[m], a[m], v[m ^ 4], a[m ^ 4]);
+#pragma unroll 1
+      for (int i = kBits; i + 1 < L; ++i) {  // a holds site i's partner
+        const uint32_t bit = 1u << (i - kBits);
+        read(t ^ (2 * bit), b);
+        read(t ^ (3 * bit), c);
+        const int r = 2 * (int)((t & bit) != 0) + (int)((t & (2 * bit)) != 0);
+#pragma unroll
+        for (int m = 0; m < kAmps; ++m) {
+          hv[m] = row_sum(ma.h[i], r, hv[m], v[m], b[m], a[m], c[m]);
+          a[m] = b[m];
+        }
+      }
+    }
+    FloatSum s[3];
+#pragma unroll
+    for (int m = 0; m < kAmps; ++m) {
+      s[0].add(v[m].x * hv[m].x + v[m].y * hv[m].y);
+      s[1].add(hv[m].x * hv[m].x + hv[m].y * hv[m].y);
+      s[2].add(v[m].x * v[m].x + v[m].y * v[m].y);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) s[k].flush(acc[k]);
+    __syncthreads();
+  }
+  block_store_k<3>(acc, part);
+}
+
+// --------------------------------------------------- products of FP64 factors
+// Double-precision table entry as FP32 pairs (48 bits).
+__device__ __forceinline__ float4 split_pair(double2 v) {
+  const float xr = (float)v.x, xi = (float)v.y;
+  return make_float4(xr, (float)(v.x - (double)xr), xi, (float)(v.y - (double)xi));
+}
+// (s, c) += (g.hi + g.lo) v: exact leading product, every error term in c
+__device__ __forceinline__ void add_product(float gh, float gl, float v, float& s, float& c) {
+  const float p = __fmul_rn(gh, v);
+  float e = __fmaf_rn(gh, v, -p);
+  e = __fmaf_rn(gl, v, e);
+  const df t = two_sum(s, p);
+  s = t.hi;
+  c = __fadd_rn(c, __fadd_rn(t.lo, e));
+}
+
+__global__ void __launch_bounds__(kThreads, 2)
+    k_overlap_f32(const float2* __restrict__ psi, int L, const double2* __restrict__ lo,
+                  const double2* __restrict__ hi, double* __restrict__ part) {
+  // the thread's 16 entries of the low table: 2 tid + (0, 1) + 512 j
+  float4 g[16];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) g[m] = split_pair(lo[2 * threadIdx.x + 512 * (m >> 1) + (m & 1)]);
+  const uint32_t chunks = 1u << (L - kBits);
+  double acc[2] = {0.0, 0.0};
+  for (uint32_t k = blockIdx.x; k < chunks; k += gridDim.x) {
+    const float4* p = reinterpret_cast<const float4*>(psi + ((uint64_t)k << kBits));
+    float4 u[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) u[j] = __ldg(p + threadIdx.x + kThreads * j);
+    float rs = 0.f, rc = 0.f, is = 0.f, ic = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float2 v[2];
+      unpack(u[j], v);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float4 f = g[2 * j + q];
+        add_product(f.x, f.y, v[q].x, rs, rc);
+        add_product(f.z, f.w, v[q].y, rs, rc);
+        add_product(f.x, f.y, v[q].y, is, ic);
+        add_product(-f.z, -f.w, v[q].x, is, ic);
+      }
+    }
+    const double re = (double)rs + (double)rc, im = (double)is + (double)ic;
+    const double2 h = hi[k];
+    acc[0] += h.x * re + h.y * im;
+    acc[1] += h.x * im - h.y * re;
+  }
+  block_store_k<2>(acc, part);
+}
+
+// a b - c d with FP32 pairs, rounded once
+__device__ __forceinline__ float mul_sub(float ah, float al, float bh, float bl, float ch, float cl,
+                                         float dh, float dl) {
+  return dot2_acc(df(0.f, 0.f), df(ah, al), df(bh, bl), df(-ch, -cl), df(dh, dl)).hi;
+}
+
+__global__ void __launch_bounds__(kThreads, 2)
+    k_factor_f32(float2* __restrict__ psi, int L, const double2* __restrict__ lo,
+                 const double2* __restrict__ hi) {
+  float4 g[16];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) g[m] = split_pair(lo[2 * threadIdx.x + 512 * (m >> 1) + (m & 1)]);
+  const uint32_t chunks = 1u << (L - kBits);
+  for (uint32_t k = blockIdx.x; k < chunks; k += gridDim.x) {
+    const float4 h = split_pair(hi[k]);
+    float4* p = reinterpret_cast<float4*>(psi + ((uint64_t)k << kBits));
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float o[4];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float4 f = g[2 * j + q];
+        o[2 * q] = mul_sub(f.x, f.y, h.x, h.y, f.z, f.w, h.z, h.w);
+        o[2 * q + 1] = mul_sub(f.x, f.y, h.z, h.w, -f.z, -f.w, h.x, h.y);
+      }
+      p[threadIdx.x + kThreads * j] = make_float4(o[0], o[1], o[2], o[3]);
+    }
+  }
+}
+
+int grid_of(int L, const LaunchCfg& cfg, int per_sm) {
+  return (int)std::min<uint64_t>(1ull << (L - kBits), (uint64_t)cfg.num_sms * per_sm);
+}
+
+}  // namespace
+
+bool observe_supported(int precision, int L) { return precision == SV_C64 && L > kBits; }
+
+int observe_energy_pairs(int L, const LaunchCfg& cfg) {
+  return ((L - kBits + 7) / 8 + 1) * grid_of(L, cfg, 4);
+}
+
+cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, const EpiParams& diag,
+                               double* part, const LaunchCfg& cfg, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  const int grid = grid_of(L, cfg, 4);
+  // the 12 lowest sites; then 8 at a time beside the lowest 4 state bits
+  for (int first = 0; first < L && e == cudaSuccess; first += first == 0 ? kBits : 8) {
+    EnergyArgs ea;
+    TileArgs& ta = ea.ta;
+    ta.L = L;
+    ta.tb = kBits;
+    ta.ep = diag;
+    ea.low = ea.diag = first == 0;
+    const int win = first == 0 ? 0 : std::min(first, L - 8);  // first window site
+    if (first == 0) {
+      ta.erun_m[0] = (1u << kBits) - 1;
+      ta.run_m[0] = ~0u;
+      ta.run_d[0] = kBits;
+      for (int q = 0; q < kBits; ++q) ea.cx[q] = (float)h.cx[q];
+    } else {
+      ta.erun_m[0] = 15;
+      ta.erun_m[1] = 0xff0;
+      ta.erun_s[1] = (uint8_t)(win - 4);
+      ta.run_m[0] = (uint32_t)((1ull << (win - 4)) - 1);
+      ta.run_d[0] = 4;
+      ta.run_s[1] = (uint8_t)(win - 4);
+      ta.run_m[1] = (uint32_t)((1ull << (L - win - 8)) - 1);
+      ta.run_d[1] = (uint8_t)(win + 8);
+      for (int q = 0; q < 8; ++q)
+        if (win + q >= first) ea.cx[4 + q] = (float)h.cx[win + q];
+    }
+    k_energy_tile<<<grid, kThreads, kTileBytes, s>>>(static_cast<const float2*>(psi), ea, part);
+    e = cudaGetLastError();
+    part += 2 * grid;
+  }
+  return e;
+}
+
+int observe_moments_grid(int L, const LaunchCfg& cfg) { return grid_of(L, cfg, 2); }
+
+cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h, const EpiParams& diag,
+                                const cd* bonds, double* part, const LaunchCfg& cfg,
+                                cudaStream_t s) {
+  MomentArgs ma;
+  ma.L = L;
+  ma.ep = diag;
+  for (int i = 0; i < L; ++i) ma.cx[i] = (float)h.cx[i];
+  for (int b = 0; bonds && b + 1 < L; ++b)
+    for (int k = 0; k < 16; ++k)
+      ma.h[b][k] = make_float2((float)bonds[16 * b + k].real(), (float)bonds[16 * b + k].imag());
+  const int grid = observe_moments_grid(L, cfg);
+  const float2* p = static_cast<const float2*>(psi);
+  if (bonds) k_moments_tile<true><<<grid, kMomentThreads, kTileBytes, s>>>(p, ma, part);
+  else k_moments_tile<false><<<grid, kMomentThreads, kTileBytes, s>>>(p, ma, part);
+  return cudaGetLastError();
+}
+
+int observe_overlap_grid(int L, const LaunchCfg& cfg) { return grid_of(L, cfg, 2); }
+
+cudaError_t launch_overlap_f32(const void* psi, int L, const void* lo, const void* hi, double* part,
+                               const LaunchCfg& cfg, cudaStream_t s) {
+  k_overlap_f32<<<observe_overlap_grid(L, cfg), kThreads, 0, s>>>(
+      static_cast<const float2*>(psi), L, static_cast<const double2*>(lo),
+      static_cast<const double2*>(hi), part);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_factor_f32(void* psi, int L, const void* lo, const void* hi, const LaunchCfg& cfg,
+                              cudaStream_t s) {
+  k_factor_f32<<<grid_of(L, cfg, 2), kThreads, 0, s>>>(static_cast<float2*>(psi), L,
+                                                      static_cast<const double2*>(lo),
+                                                      static_cast<const double2*>(hi));
+  return cudaGetLastError();
+}
+
+}  // namespace fsv

@@ -8,11 +8,13 @@
 #include <cstdarg>
 #include <cstdio>
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <limits>
 #include <memory>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "sv_batch.h"
@@ -25,6 +27,7 @@ using fsv::cd;
 
 namespace {
 constexpr int kRing = 1024;  // energy ring (periods between host readbacks)
+constexpr size_t kWorkKept = (size_t)8 << 20;  // largest workspace a context keeps
 }
 
 struct sv_ctx {
@@ -82,6 +85,9 @@ struct sv_ctx {
   // in_period_layout says whether it currently is in the plan's start layout.
   bool keep_layout = false;
   bool in_period_layout = false;
+
+  char* d_work = nullptr;  // workspace of the measurements
+  size_t work_bytes = 0;
 
   int launches_per_period = 0;
   int passes_per_period = 0;
@@ -470,9 +476,63 @@ int check_ready(sv_ctx* ctx, bool need_built) {
   return SV_OK;
 }
 
+fsv::H0Coef h0_coef(const sv_ctx* ctx) {
+  fsv::H0Coef h;
+  h.J = ctx->obs.J;
+  for (int i = 0; i < ctx->L && !ctx->obs.general; ++i) {
+    h.cx[i] = ctx->obs.cx[i];
+    h.cz[i] = ctx->obs.cz[i];
+  }
+  return h;
+}
+
+// Energy density and norm from the measurement's partial pairs.
+int read_measurement(sv_ctx* ctx, long long pairs, double* e_out, double* n_out) {
+  SV_CUDA(fsv::launch_period_reduce(ctx->d_part_meas, pairs, ctx->L, ctx->d_meas, 1, ctx->d_counter,
+                                    0, ctx->stream),
+          "measurement reduce");
+  double h[2];
+  SV_CUDA(cudaMemcpyAsync(h, ctx->d_meas, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream),
+          "copy energy");
+  SV_CUDA(cudaStreamSynchronize(ctx->stream), "synchronize");
+  if (e_out) *e_out = h[0];
+  if (n_out) *n_out = h[1];
+  return SV_OK;
+}
+
+// Device workspace of at least `bytes`, kept with the context up to 8 MiB
+// (larger requests: *own is set and the caller frees it in stream order).
+int workspace(sv_ctx* ctx, size_t bytes, char** out, bool* own) {
+  *own = bytes > kWorkKept;
+  if (*own) {
+    SV_CUDA(cudaMallocAsync(reinterpret_cast<void**>(out), bytes, ctx->stream), "workspace");
+    return SV_OK;
+  }
+  if (ctx->work_bytes < bytes) {
+    cudaFree(ctx->d_work);
+    ctx->d_work = nullptr;
+    ctx->work_bytes = 0;
+    if (cudaMalloc(&ctx->d_work, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      ctx->d_work = nullptr;
+      return fail(ctx, SV_ENOMEM, "workspace of %zu bytes", bytes);
+    }
+    ctx->work_bytes = bytes;
+  }
+  *out = ctx->d_work;
+  return SV_OK;
+}
+
 // Read-only measurement of <H0> and the norm of the current state.
 int measure(sv_ctx* ctx, double* e_out, double* n_out) {
   const int L = ctx->L;
+  if (fsv::observe_supported(ctx->precision, L)) {
+    const int pairs = fsv::observe_energy_pairs(L, ctx->cfg);
+    SV_CUDA(fsv::launch_energy_tile(ctx->state, L, h0_coef(ctx), epi_for(ctx, fsv::EPI_DIAG, 0, nullptr),
+                                    ctx->d_part_meas, ctx->cfg, ctx->stream),
+            "measurement launch");
+    return read_measurement(ctx, pairs, e_out, n_out);
+  }
   struct Item {
     int bond, flags;
   };
@@ -491,16 +551,7 @@ int measure(sv_ctx* ctx, double* e_out, double* n_out) {
                                    ctx->stream),
             "measurement launch");
   }
-  SV_CUDA(fsv::launch_period_reduce(ctx->d_part_meas, (long long)items.size() * ctx->maxb, L,
-                                    ctx->d_meas, 1, ctx->d_counter, 0, ctx->stream),
-          "measurement reduce");
-  double h[2];
-  SV_CUDA(cudaMemcpyAsync(h, ctx->d_meas, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream),
-          "copy energy");
-  SV_CUDA(cudaStreamSynchronize(ctx->stream), "synchronize");
-  if (e_out) *e_out = h[0];
-  if (n_out) *n_out = h[1];
-  return SV_OK;
+  return read_measurement(ctx, (long long)items.size() * ctx->maxb, e_out, n_out);
 }
 
 // Copy ring slots of periods c0 .. c0+count-1 (count <= kRing) to the host.
@@ -531,20 +582,28 @@ int read_ring(sv_ctx* ctx, int64_t c0, int64_t count, double* e_out, double* n_o
 // E = <H0>, sigma_E and <psi|psi> of the current state (Ising or general
 // two-site chain), partials summed on the host in a fixed order.
 int energy_moments(sv_ctx* ctx, double* energy, double* sigma_e, double* norm2) {
-  const int grid = fsv::moments_grid(ctx->cfg);
+  const bool tiles = fsv::observe_supported(ctx->precision, ctx->L);
+  const int grid = tiles ? fsv::observe_moments_grid(ctx->L, ctx->cfg) : fsv::moments_grid(ctx->cfg);
   const bool c128 = ctx->precision == SV_C128;
-  const size_t nh = ctx->obs.general ? ctx->obs.h.size() : 0;
+  const size_t nh = ctx->obs.general && !tiles ? ctx->obs.h.size() : 0;
   const size_t hb_bytes = nh * (c128 ? sizeof(double2) : sizeof(float2));
   char* d_buf = nullptr;
-  SV_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&d_buf), hb_bytes + sizeof(double) * 3 * grid,
-                          ctx->stream),
-          "moments scratch");
+  bool own = false;
+  {
+    int rc = workspace(ctx, hb_bytes + sizeof(double) * 3 * grid, &d_buf, &own);
+    if (rc) return rc;
+  }
   double* d_part = reinterpret_cast<double*>(d_buf + hb_bytes);
   std::vector<double> part((size_t)3 * grid);
   std::vector<double2> h64;
   std::vector<float2> h32;
   cudaError_t e = cudaSuccess;
-  if (ctx->obs.general) {
+  if (tiles) {
+    e = fsv::launch_moments_tile(ctx->state, ctx->L, h0_coef(ctx),
+                                 epi_for(ctx, ctx->obs.general ? 0 : fsv::EPI_DIAG, 0, nullptr),
+                                 ctx->obs.general ? ctx->obs.h.data() : nullptr, d_part, ctx->cfg,
+                                 ctx->stream);
+  } else if (ctx->obs.general) {
     for (const fsv::cd& v : ctx->obs.h) {
       h64.push_back(make_double2(v.real(), v.imag()));
       h32.push_back(make_float2((float)v.real(), (float)v.imag()));
@@ -555,13 +614,7 @@ int energy_moments(sv_ctx* ctx, double* energy, double* sigma_e, double* norm2) 
       e = fsv::launch_bond_moments(ctx->precision, ctx->state, ctx->L, d_buf, d_part, ctx->cfg,
                                    ctx->stream);
   } else {
-    fsv::H0Coef h;
-    h.J = ctx->obs.J;
-    for (int i = 0; i < ctx->L; ++i) {
-      h.cx[i] = ctx->obs.cx[i];
-      h.cz[i] = ctx->obs.cz[i];
-    }
-    e = fsv::launch_h0_moments(ctx->precision, ctx->state, ctx->L, h, d_part, ctx->cfg,
+    e = fsv::launch_h0_moments(ctx->precision, ctx->state, ctx->L, h0_coef(ctx), d_part, ctx->cfg,
                                ctx->stream);
   }
   if (e == cudaSuccess)
@@ -569,7 +622,7 @@ int energy_moments(sv_ctx* ctx, double* energy, double* sigma_e, double* norm2) 
                         cudaMemcpyDeviceToHost, ctx->stream);
   // the host buffers must outlive the copies above
   const cudaError_t es = cudaStreamSynchronize(ctx->stream);
-  cudaFreeAsync(d_buf, ctx->stream);
+  if (own) cudaFreeAsync(d_buf, ctx->stream);
   if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) return cuda_fail(ctx, e, "energy moments");
   double s1 = 0.0, s2 = 0.0, sn = 0.0;  // fixed order
@@ -606,17 +659,21 @@ int factor_tables(sv_ctx* ctx, int L, int group, const double* factors, int* m_o
   }
   const int m = std::min(L, 12) / group * group;
   auto table = [&](int first, int count, std::vector<double>* t) {
-    t->assign(2ull << count, 0.0);
-    for (uint64_t x = 0; x < (1ull << count); ++x) {
-      std::complex<double> v = 1.0;
-      for (int s = 0; s < count; s += group) {
+    // one group of sites after another, each entry the product of its factors
+    // in site order
+    std::vector<std::complex<double>> v(1ull << count);
+    v[0] = 1.0;
+    for (int s = 0; s < count; s += group) {
+      const std::complex<double>* g = &f[(size_t)((first + s) / group) * width];
+      const uint64_t n = 1ull << s;
+      for (int bits = width - 1; bits >= 0; --bits) {
         int r = 0;  // the group's local index, its lowest site the high bit
-        for (int k = 0; k < group; ++k) r = 2 * r + (int)((x >> (s + k)) & 1);
-        v *= f[(size_t)((first + s) / group) * width + r];
+        for (int k = 0; k < group; ++k) r = 2 * r + ((bits >> k) & 1);
+        for (uint64_t x = 0; x < n; ++x) v[x + (n * bits)] = v[x] * g[r];
       }
-      (*t)[2 * x] = v.real();
-      (*t)[2 * x + 1] = v.imag();
     }
+    t->resize(2ull << count);
+    std::memcpy(t->data(), v.data(), sizeof(double) * t->size());
   };
   table(0, m, lo);
   table(m, L - m, hi);
@@ -633,26 +690,29 @@ int product_overlap(sv_ctx* ctx, int group, const double* factors, double* overl
   int rc = factor_tables(ctx, L, group, factors, &m, &lo, &hi);
   if (rc) return rc;
   DeviceGuard dg(ctx->device);
-  const int grid = fsv::moments_grid(ctx->cfg);
+  const bool tiles = fsv::observe_supported(ctx->precision, L);
+  const int grid = tiles ? fsv::observe_overlap_grid(L, ctx->cfg) : fsv::moments_grid(ctx->cfg);
   const size_t lo_b = sizeof(double) * lo.size(), hi_b = sizeof(double) * hi.size();
   char* d_buf = nullptr;
-  SV_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&d_buf), lo_b + hi_b + sizeof(double) * 2 * grid,
-                          ctx->stream),
-          "overlap scratch");
+  bool own = false;
+  rc = workspace(ctx, lo_b + hi_b + sizeof(double) * 2 * grid, &d_buf, &own);
+  if (rc) return rc;
   double* d_part = reinterpret_cast<double*>(d_buf + lo_b + hi_b);
   std::vector<double> part((size_t)2 * grid);
   cudaError_t e = cudaMemcpyAsync(d_buf, lo.data(), lo_b, cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_buf + lo_b, hi.data(), hi_b, cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess)
-    e = fsv::launch_product_overlap(ctx->precision, ctx->state, L, m, d_buf, d_buf + lo_b,
-                                    d_part, ctx->cfg, ctx->stream);
+    e = tiles ? fsv::launch_overlap_f32(ctx->state, L, d_buf, d_buf + lo_b, d_part, ctx->cfg,
+                                        ctx->stream)
+              : fsv::launch_product_overlap(ctx->precision, ctx->state, L, m, d_buf, d_buf + lo_b,
+                                            d_part, ctx->cfg, ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(part.data(), d_part, sizeof(double) * part.size(),
                         cudaMemcpyDeviceToHost, ctx->stream);
   // the host tables must outlive the copies above
   const cudaError_t es = cudaStreamSynchronize(ctx->stream);
-  cudaFreeAsync(d_buf, ctx->stream);
+  if (own) cudaFreeAsync(d_buf, ctx->stream);
   if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) return cuda_fail(ctx, e, "product overlap");
   double re = 0.0, im = 0.0;  // fixed order
@@ -947,15 +1007,42 @@ void upload_gates(const std::vector<fsv::Gate2>& gates, std::vector<double2>& ou
     }
 }
 
+// f(k) for k = 0..n-1 over the host's cores (each period's tables are its own);
+// false if one of them ran out of memory.
+template <typename F>
+bool for_periods(int64_t n, const F& f) {
+  std::atomic<int64_t> next{0};
+  std::atomic<bool> ok{true};
+  auto work = [&]() {
+    for (int64_t k = next++; k < n && ok; k = next++) {
+      try {
+        f(k);
+      } catch (...) {
+        ok = false;
+      }
+    }
+  };
+  std::vector<std::thread> th;
+  try {
+    const int64_t hw = std::min<int64_t>(16, std::max(1u, std::thread::hardware_concurrency()));
+    for (int64_t i = 1; i < std::min(n, hw); ++i) th.emplace_back(work);
+  } catch (...) {  // fewer threads do
+  }
+  work();
+  for (auto& t : th) t.join();
+  return ok;
+}
+
 // The gate tables of every period-parameter set, in the context's entry type.
 template <typename E>
 int upload_tables(sv_ctx* ctx, const sv_floquet_params& p, int64_t ntab, int ng,
                   std::vector<E>& tab) {
   tab.resize((size_t)ntab * ng * fsv::kGateEntries);
-  for (int64_t k = 0; k < ntab; ++k) {
+  const bool ok = for_periods(ntab, [&](int64_t k) {
     auto gk = k == 0 ? ctx->gates : fsv::period_gates(ctx->L, p, ctx->theta_p[k], ctx->hx_p[k]);
     upload_gates(gk, tab, (size_t)k * ng * fsv::kGateEntries);
-  }
+  });
+  if (!ok) return fail(ctx, SV_ENOMEM, "gate tables");
   SV_CUDA(cudaMemcpyAsync(ctx->d_gates, tab.data(), ctx->d_gates_bytes, cudaMemcpyHostToDevice,
                           ctx->stream),
           "upload gates");
@@ -1028,13 +1115,7 @@ int adjoint_tiles(sv_ctx* ctx, int64_t P, const std::vector<fsv::AdjOp>& ops, in
   auto run = [&]() -> int {
     int r = sv_evolve(ctx, P, nullptr, nullptr);
     if (r) return r;
-    fsv::H0Coef h;
-    h.J = ctx->obs.J;
-    for (int i = 0; i < L; ++i) {
-      h.cx[i] = ctx->obs.cx[i];
-      h.cz[i] = ctx->obs.cz[i];
-    }
-    SV_CUDA(fsv::launch_apply_h0(SV_C64, ctx->state, d_lam, L, h, d_part, ctx->cfg, ctx->stream),
+    SV_CUDA(fsv::launch_apply_h0(SV_C64, ctx->state, d_lam, L, h0_coef(ctx), d_part, ctx->cfg, ctx->stream),
             "adjoint seed launch");
     SV_CUDA(fsv::launch_grad_reduce(d_part, seed_grid, d_grad + 2 * P, 0, ctx->stream),
             "energy reduce launch");
@@ -1472,21 +1553,25 @@ int sv_init_pairs(sv_ctx* ctx, int L, const double* pair_states) {
   if (L != ctx->L) free_build(ctx);
   const size_t lo_b = sizeof(double) * lo.size(), hi_b = sizeof(double) * hi.size();
   char* d_buf = nullptr;
-  SV_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&d_buf), lo_b + hi_b, ctx->stream),
-          "pair tables");
+  bool own = false;
+  {
+    int rc = workspace(ctx, lo_b + hi_b, &d_buf, &own);
+    if (rc) return rc;
+  }
   cudaError_t e = cudaMemcpyAsync(d_buf, lo.data(), lo_b, cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_buf + lo_b, hi.data(), hi_b, cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess)
-    e = fsv::launch_factor_state(ctx->precision, ctx->state, L, m, d_buf, d_buf + lo_b, ctx->cfg,
-                                 ctx->stream);
+    e = fsv::observe_supported(ctx->precision, L)
+            ? fsv::launch_factor_f32(ctx->state, L, d_buf, d_buf + lo_b, ctx->cfg, ctx->stream)
+            : fsv::launch_factor_state(ctx->precision, ctx->state, L, m, d_buf, d_buf + lo_b,
+                                       ctx->cfg, ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(ctx->d_counter, 0, sizeof(long long), ctx->stream);
   // the host tables must outlive the copies above
   const cudaError_t es = cudaStreamSynchronize(ctx->stream);
-  cudaFreeAsync(d_buf, ctx->stream);
+  if (own) cudaFreeAsync(d_buf, ctx->stream);
   if (e == cudaSuccess) e = es;
-  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "pair state");
   ctx->L = L;
   ctx->inited = true;
@@ -1540,8 +1625,7 @@ int sv_adjoint(sv_ctx* ctx, int64_t periods, double* grad_theta, double* grad_hx
   DeviceGuard dg(ctx->device);
   // operation tables of every period, reverse order within a period
   std::vector<std::vector<fsv::AdjOp>> ops((size_t)P);
-  for (int64_t k = 0; k < P; ++k)
-    ops[k] = fsv::adjoint_period_ops(L, ctx->params, ctx->theta_p[k], ctx->hx_p[k]);
+  ops[0] = fsv::adjoint_period_ops(L, ctx->params, ctx->theta_p[0], ctx->hx_p[0]);
   const size_t nop = ops[0].size();
   const size_t tab_elems = (size_t)P * nop * 32;  // odag, d per operation
   std::vector<float2> tab32;
@@ -1550,7 +1634,8 @@ int sv_adjoint(sv_ctx* ctx, int64_t periods, double* grad_theta, double* grad_hx
     tab64.resize(tab_elems);
   else
     tab32.resize(tab_elems);
-  for (int64_t k = 0; k < P; ++k) {
+  const bool tables_ok = for_periods(P, [&](int64_t k) {
+    if (k > 0) ops[k] = fsv::adjoint_period_ops(L, ctx->params, ctx->theta_p[k], ctx->hx_p[k]);
     RoundedGates rounded;
     for (size_t o = 0; o < nop; ++o) {
       const fsv::AdjOp& op = ops[k][o];
@@ -1566,7 +1651,8 @@ int sv_adjoint(sv_ctx* ctx, int64_t periods, double* grad_theta, double* grad_hx
           tab32[at + 16 + e] = make_float2((float)op.d[e].real(), (float)op.d[e].imag());
       }
     }
-  }
+  });
+  if (!tables_ok) return fail(ctx, SV_ENOMEM, "adjoint tables");
   if (!c128) {
     const int tb = adjoint_tile_bits(ctx, ops[0]);
     if (tb) return adjoint_tiles(ctx, P, ops[0], tb, tab32, grad_theta, grad_hx, energy_density);
@@ -1879,6 +1965,7 @@ void sv_destroy(sv_ctx* ctx) {
   cudaFree(ctx->d_ident);
   cudaFree(ctx->d_spinors);
   cudaFree(ctx->d_part_meas);
+  cudaFree(ctx->d_work);
   cudaFree(ctx->d_ring);
   cudaFree(ctx->d_meas);
   cudaFree(ctx->d_counter);

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <complex>
 #include <cstdint>
 
 namespace fsv {
@@ -143,6 +144,24 @@ cudaError_t launch_factor_state(int precision, void* psi, int L, int m, const vo
 cudaError_t launch_product_overlap(int precision, const void* psi, int L, int m,
                                    const void* lo, const void* hi, double* partial,
                                    const LaunchCfg& cfg, cudaStream_t s);
+
+// The same measurements of a complex64 state of at least 13 sites in tiles
+// (k_observe.cu); m = 12 in the factor tables.
+bool observe_supported(int precision, int L);
+// (energy, norm) partial pairs that launch_energy_tile writes
+int observe_energy_pairs(int L, const LaunchCfg& cfg);
+cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, const EpiParams& diag,
+                               double* part, const LaunchCfg& cfg, cudaStream_t s);
+// bonds: general bond terms on the host ((L - 1) x 16), or NULL for the Ising chain
+int observe_moments_grid(int L, const LaunchCfg& cfg);
+cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h, const EpiParams& diag,
+                                const std::complex<double>* bonds, double* part,
+                                const LaunchCfg& cfg, cudaStream_t s);
+int observe_overlap_grid(int L, const LaunchCfg& cfg);
+cudaError_t launch_overlap_f32(const void* psi, int L, const void* lo, const void* hi, double* part,
+                               const LaunchCfg& cfg, cudaStream_t s);
+cudaError_t launch_factor_f32(void* psi, int L, const void* lo, const void* hi, const LaunchCfg& cfg,
+                              cudaStream_t s);
 
 // lambda = (H0 / L) psi; partial[block] = that block's share of
 // Re <psi|lambda>.

@@ -98,8 +98,24 @@ extern "C" int sv_energy_noalloc(const void* psi_dev, int L, int precision,
   // the gate passes launch at most 4 blocks per SM; cap the SM count so that
   // every pass fits in its kMaxBlocks slice of the scratch
   cfg.num_sms = sym.num_sms < kMaxBlocks / 4 ? sym.num_sms : kMaxBlocks / 4;
-  const void* ident = precision == SV_C128 ? sym.ident128 : sym.ident64;
   const double ew = p->edge_field_weight;
+  if (fsv::observe_supported(precision, L)) {
+    // the same passes as sv_expect_energy (at most four, four blocks an SM)
+    fsv::H0Coef h;
+    fsv::EpiParams ep;
+    ep.J = p->J;
+    ep.cz_first = p->hz * fsv::site_field_share(L, 0, ew);
+    ep.cz_last = p->hz * fsv::site_field_share(L, L - 1, ew);
+    ep.cz_bulk = p->hz * fsv::site_field_share(L, 1, ew);
+    for (int i = 0; i < L; ++i) h.cx[i] = p->hx * fsv::site_field_share(L, i, ew);
+    const int pairs = fsv::observe_energy_pairs(L, cfg);
+    if (pairs > kMaxPasses * kMaxBlocks) return SV_EINVAL;
+    cudaError_t e = fsv::launch_energy_tile(psi_dev, L, h, ep, sym.scratch, cfg, s);
+    if (e == cudaSuccess)
+      e = fsv::launch_period_reduce(sym.scratch, pairs, L, out_dev, 1, sym.counter, /*advance=*/0, s);
+    return e == cudaSuccess ? SV_OK : SV_ECUDA;
+  }
+  const void* ident = precision == SV_C128 ? sym.ident128 : sym.ident64;
   int npass = 0;
   int bonds[kMaxPasses], flags[kMaxPasses];
   for (int b = 0; b + 1 < L; b += 2) {
