@@ -460,8 +460,8 @@ int sv_host_store_view(int L, const sv_floquet_params *p, int n, int pass, int *
 
 /* ------------------------------------------------------------------ batch
  * Many independent chains (each its own L, parameters and product state)
- * evolved together on one device.  Chains of up to 14 sites can stay in one
- * CTA's shared memory for a whole run (resident form); the others run the
+ * evolved together on one device.  Chains of up to 14 sites can stay in the
+ * shared memory of one CTA or a cluster for a whole run (resident form); the others run the
  * plain, block or multi-gate forms.  One CUDA graph advances every chain by
  * a run of periods, the chains as independent branches (within a run a
  * chain's block periods may start off site 0; every run hands back the

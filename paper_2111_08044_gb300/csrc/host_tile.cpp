@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "sv_batch.h"
 #include "sv_tile.h"
 
 namespace fsv {
@@ -45,10 +46,10 @@ int tile_threads(int precision, int tb) {
 // Gates [at, end) of one pass in a tile of 2^tb amplitudes and its state bits
 // before filling up (end = at: the tile is too small for the gate).
 static int pass_end(int L, const std::vector<Gate2>& gates, int precision, int tb, int at,
-                    uint64_t* bits) {
+                    int max_gates, uint64_t* bits) {
   const int ng = (int)gates.size(), first = at;
   uint64_t set = (1ull << std::min(line_bits(precision), L)) - 1;
-  while (at < ng && at - first < kTileMaxGates) {
+  while (at < ng && at - first < max_gates) {
     const Gate2& g = gates[at];
     uint64_t need = set | (3ull << g.bond);
     if (energy_group(L, precision, g.bond, g.epi) == TILE_E_SWEEP) need |= 0xff;
@@ -60,14 +61,18 @@ static int pass_end(int L, const std::vector<Gate2>& gates, int precision, int t
   return at;
 }
 
-std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int precision, int tb) {
+static int most_gates(int precision) { return precision == SV_C64 ? kTileTabSlots : kTileMaxGates; }
+
+std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int precision, int tb,
+                                    int max_gates) {
+  if (max_gates == 0) max_gates = most_gates(precision);
   std::vector<TilePassPlan> out;
   const int ng = (int)gates.size();
   int at = 0;
   while (at < ng) {
     TilePassPlan p;
     uint64_t set = 0;
-    const int end = pass_end(L, gates, precision, tb, at, &set);
+    const int end = pass_end(L, gates, precision, tb, at, max_gates, &set);
     while (at < end) p.gates.push_back(at++);
     if (p.gates.empty()) return {};  // a tile too small for one gate
     for (int q = 0; __builtin_popcountll(set) < tb; ++q) set |= 1ull << q;  // lowest free bits
@@ -83,11 +88,11 @@ std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int 
       const Gate2& a = gates[p.gates[i]];
       std::vector<int> reg = {where[a.bond], where[a.bond + 1]};
       const int ea = energy_group(L, precision, a.bond, a.epi);
-      r.gate[0] = (int8_t)i;
+      r.gate[0] = (uint8_t)i;
+      r.count = 1;
       r.bond[0] = (uint8_t)a.bond;
       r.epi[0] = (uint8_t)a.epi;
       r.egroup[0] = (uint8_t)ea;
-      r.gate[1] = -1;
       size_t next = i + 1;
       if (precision == SV_C64) {
         // a second gate: on other sites, the first gate's sums not taken from
@@ -100,7 +105,8 @@ std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int 
           if (apart && ea != TILE_E_SWEEP && !bit0) {
             reg.push_back(where[b.bond]);
             reg.push_back(where[b.bond + 1]);
-            r.gate[1] = (int8_t)next;
+            r.gate[1] = (uint8_t)next;
+            r.count = 2;
             r.bond[1] = (uint8_t)b.bond;
             r.epi[1] = (uint8_t)b.epi;
             r.egroup[1] = (uint8_t)eb;
@@ -120,7 +126,7 @@ std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int 
         r.sbit[k] = (uint8_t)p.bits[reg[k]];
         r.ins[k] = (uint16_t)(0xffffu << sorted[k]);
       }
-      for (int k = 0; k < 2 && r.gate[k] >= 0; ++k)
+      for (int k = 0; k < r.count; ++k)
         r.xorder[k] = xor_order(L, precision, r.bond[k]) ? 1 : 0;
       p.measures = p.measures || r.epi[0] || r.epi[1];
       p.rounds.push_back(r);
@@ -145,7 +151,7 @@ int tile_bits(int L, const std::vector<Gate2>& gates, int precision, int num_sms
   int best = 0;
   double best_t = 0;
   for (int tb = std::min(L, 6); tb <= std::min(L, kTileMaxBits); ++tb) {
-    if (tb > cap && !(precision == SV_C64 && tb == L)) continue;
+    if (tb > cap) continue;
     const double tiles = (double)(1ull << (L - tb));
     const double per_sm = (double)((int64_t)((tiles + num_sms - 1) / num_sms));
     const double amps = (double)(1ull << tb);
@@ -153,7 +159,7 @@ int tile_bits(int L, const std::vector<Gate2>& gates, int precision, int num_sms
     const int ng = (int)gates.size();
     for (int at = 0; at < ng;) {
       uint64_t set = 0;
-      const int end = pass_end(L, gates, precision, tb, at, &set);
+      const int end = pass_end(L, gates, precision, tb, at, most_gates(precision), &set);
       if (end == at) {
         t = -1;
         break;
@@ -181,6 +187,44 @@ int tile_bits(int L, const std::vector<Gate2>& gates, int precision, int num_sms
     }
   }
   return best;
+}
+
+std::vector<ResidentRound> resident_rounds(const std::vector<Gate2>& gates, const ResidentShape& sh) {
+  std::vector<ResidentRound> out;
+  // rounds do not reach across the tables held at a time
+  for (size_t at = 0; at < gates.size(); at += kResidentGates) {
+    const std::vector<Gate2> part(gates.begin() + at,
+                                  gates.begin() + std::min(gates.size(), at + kResidentGates));
+    const auto plan = tile_plan(sh.L, part, SV_C64, sh.L, kResidentGates);
+    if (plan.size() != 1) return {};
+    for (const TileRound& r : plan[0].rounds) {
+      ResidentRound o;
+      std::memset(&o, 0, sizeof(o));
+      int bits[4];
+      for (int k = 0; k < 4; ++k) {
+        o.sbit[k] = r.sbit[k];
+        o.remote |= sh.local(r.sbit[k]) ? 0 : 1;
+      }
+      for (int k = 0; k < 4; ++k) {
+        bits[k] = o.remote ? r.sbit[k] : sh.place(r.sbit[k]);
+        o.off[k] = o.remote ? 1u << bits[k] : tile_byte8(1u << bits[k]);
+      }
+      std::sort(bits, bits + 4);
+      for (int k = 0; k < 4; ++k) o.ins[k] = ~0u << bits[k];
+      o.count = r.count;
+      for (int k = 0; k < 2; ++k) {
+        o.bond[k] = r.bond[k];
+        o.epi[k] = r.epi[k];
+        o.egroup[k] = r.egroup[k];
+        o.xorder[k] = r.xorder[k];
+        if (r.egroup[k] == TILE_E_SWEEP) o.sweep = (uint8_t)(k + 1);
+      }
+      out.push_back(o);
+    }
+  }
+  for (size_t k = 0; k < out.size(); ++k)
+    out[k].cluster = out[k].remote || out[(k + 1) % out.size()].remote ? 1 : 0;
+  return out;
 }
 
 }  // namespace fsv

@@ -17,7 +17,6 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <cstring>
 
 #include "sv_device.cuh"
 #include "sv_internal.h"
@@ -213,11 +212,10 @@ __device__ __forceinline__ void derivative16(const uint64_t (&v)[16], const uint
 // was bound by its launch and by L2 (8.4 us an operation at L = 20, where its
 // FMAs take 1.4 us); with four to six a pass the FP32 pipe is the bound.  Each
 // group's arithmetic is that of k_adjoint_gate.
-template <int kSlots>
 __global__ void __launch_bounds__(128, 4)
     k_adjoint_tile(float2* __restrict__ psi, float2* __restrict__ lam,
                    const __grid_constant__ AdjointPass ap, double* __restrict__ part,
-                   const __grid_constant__ TileTab<kSlots> tab) {
+                   const __grid_constant__ TileTab tab) {
   extern __shared__ __align__(16) uint8_t tile_smem[];
   const TileArgs& ta = ap.ta;
   const uint32_t tile_bytes = tile_byte8(1u << ta.tb);
@@ -257,7 +255,7 @@ __global__ void __launch_bounds__(128, 4)
       derivative16<0, 1, 2, 3>(v, l, from(ga), ga < ap.nkick ? sum[0] : sum[1]);
       apply16<0, 1, 2, 3>(v, from(ga));
       apply16<0, 1, 2, 3>(l, from(ga));
-      if (gb >= 0) {
+      if (rd.count == 2) {
         derivative16<2, 3, 0, 1>(v, l, from(gb), gb < ap.nkick ? sum[0] : sum[1]);
         apply16<2, 3, 0, 1>(v, from(gb));
         apply16<2, 3, 0, 1>(l, from(gb));
@@ -393,24 +391,14 @@ cudaError_t launch_grad_reduce(const double* partials, long long n, double* out,
   return cudaGetLastError();
 }
 
-namespace {
-bool adjoint_small(const TileArgs& ta) {
-  return ta.ngates <= kTileTabSmall && ta.nrounds <= kTileTabSmall;
-}
-const void* adjoint_kernel(const TileArgs& ta) {
-  return adjoint_small(ta) ? reinterpret_cast<const void*>(k_adjoint_tile<kTileTabSmall>)
-                           : reinterpret_cast<const void*>(k_adjoint_tile<kTileMaxGates>);
-}
-}  // namespace
-
 cudaError_t adjoint_tile_grid(AdjointPass* ap, const LaunchCfg& cfg, int* grid) {
   const TileArgs& ta = ap->ta;
   const int smem = 2 * (int)tile_byte8(1u << ta.tb);
   int per_sm = 1;
-  cudaError_t e = cudaFuncSetAttribute(adjoint_kernel(ta), cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(k_adjoint_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        2 * (int)tile_byte8(1u << kAdjointTileBits));
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, adjoint_kernel(ta),
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adjoint_tile,
                                                       tile_threads(SV_C64, ta.tb), smem);
   const uint64_t most = (uint64_t)cfg.num_sms * (per_sm > 0 ? per_sm : 1);
   const uint64_t tiles = 1ull << (ta.L - ta.tb);
@@ -418,21 +406,12 @@ cudaError_t adjoint_tile_grid(AdjointPass* ap, const LaunchCfg& cfg, int* grid) 
   return e;
 }
 
-cudaError_t launch_adjoint_tile(void* psi, void* lam, const AdjointPass& ap,
-                                const TileTab<kTileMaxGates>& tab, double* part, int grid,
-                                cudaStream_t s) {
-  const TileArgs& ta = ap.ta;
-  TileTab<kTileTabSmall> small;
-  void* args[] = {&psi, &lam, const_cast<AdjointPass*>(&ap), &part, nullptr};
-  if (adjoint_small(ta)) {
-    std::memcpy(small.g, tab.g, sizeof(small.g));
-    std::memcpy(small.r, tab.r, sizeof(small.r));
-    args[4] = &small;
-  } else {
-    args[4] = const_cast<TileTab<kTileMaxGates>*>(&tab);
-  }
-  return cudaLaunchKernel(adjoint_kernel(ta), dim3(grid), dim3(tile_threads(SV_C64, ta.tb)), args,
-                          2 * (size_t)tile_byte8(1u << ta.tb), s);
+cudaError_t launch_adjoint_tile(void* psi, void* lam, const AdjointPass& ap, const TileTab& tab,
+                                double* part, int grid, cudaStream_t s) {
+  const int tb = ap.ta.tb;
+  k_adjoint_tile<<<grid, tile_threads(SV_C64, tb), 2 * tile_byte8(1u << tb), s>>>(
+      static_cast<float2*>(psi), static_cast<float2*>(lam), ap, part, tab);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_grad_reduce_pairs(const double* part, int pairs, int periods, double* out,

@@ -1,11 +1,13 @@
-// Batched evolution of many independent chains: the resident form.
+// Batch chains of two to kShortMaxL sites: one block a chain, its state in shared
+// memory for a run of periods, one group of four amplitudes a thread and gate.
 //
-// A chain of L <= 14 sites (at most 128 KiB of complex64 amplitudes) lives
-// in one CTA's shared memory for a whole run of periods: the CTA loads it,
-// applies every gate of every period in shared memory (the Eq. 2
-// contraction per group of four amplitudes), measures the energy density
-// and norm at the end of each period, and writes the state back once.  One
-// launch runs all resident chains, one CTA each.
+// A chain that short is one or two warps at most, so that the length of a warp's
+// chain of instructions per gate bounds it, not the device's rates; the resident
+// form of longer chains (two gates on 16 amplitudes a thread) takes fewer
+// instructions in all but more in a row.  Tables and coefficients in shared
+// memory, the diagonal energies of a thread's amplitudes in registers for the
+// run.  16 chains of eight sites: 11.2 us a period of 28 gates, with the tables
+// read from L2 and the diagonal energies built every period 12.4 us.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -19,88 +21,97 @@ namespace {
 
 using namespace dev;
 
-constexpr int kThreads = 512;
+constexpr int kThreads = 128;
 
-__global__ void __launch_bounds__(kThreads, 1)
-    k_chain_resident(const ResidentChain* __restrict__ chains, const long long* __restrict__ counter,
-                     int periods, int ring_len) {
-  extern __shared__ float2 sp[];
-  const ResidentChain& ch = chains[blockIdx.x];
+__global__ void __launch_bounds__(kThreads)
+    k_chain_short(const ChainArgs* __restrict__ chains, const long long* __restrict__ counter,
+                  int periods, int ring_len) {
+  __shared__ float2 sp[1 << kShortMaxL];
+  __shared__ __align__(16) float2 tables[kShortGates * kGateEntries];
+  __shared__ int bonds[kShortGates];
+  __shared__ ChainArgs ch;
+  __shared__ double se[kThreads / 32], sn[kThreads / 32];
+  for (uint32_t k = threadIdx.x; k < sizeof(ChainArgs) / 4; k += kThreads)
+    reinterpret_cast<uint32_t*>(&ch)[k] = reinterpret_cast<const uint32_t*>(chains + blockIdx.x)[k];
+  const long long p0 = counter[0];
+  if (periods == 0) periods = (int)counter[1];
+  __syncthreads();
   const int L = ch.L;
   const uint32_t n = 1u << L;
-  const long long p0 = *counter;
-  // the chain's coefficients in FP32 once, so that the per-amplitude
-  // measurement below runs no FP64 instruction
-  __shared__ float s_cz[kResidentMaxL], s_cx[kResidentMaxL];
-  if (threadIdx.x < (unsigned)L) {
-    s_cz[threadIdx.x] = (float)ch.cz[threadIdx.x];
-    s_cx[threadIdx.x] = (float)ch.cx[threadIdx.x];
+  // a period of more gates is read from global memory
+  const bool held = ch.ngates <= kShortGates;
+  if (held) {
+    for (int k = threadIdx.x; k < ch.ngates * (kGateEntries / 2); k += kThreads)
+      reinterpret_cast<float4*>(tables)[k] = __ldg(reinterpret_cast<const float4*>(ch.gates) + k);
+    for (int k = threadIdx.x; k < ch.ngates; k += kThreads) bonds[k] = __ldg(ch.bonds + k);
   }
-  const float Jf = (float)ch.J;
-  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) sp[i] = ch.psi[i];
+  for (uint32_t i = threadIdx.x; i < n; i += kThreads) sp[i] = ch.psi[i];
   __syncthreads();
-  __shared__ double se[kThreads / 32], sn[kThreads / 32];
+  // diagonal energy of the thread's amplitudes, site by site
+  constexpr int kAmps = (1 << kShortMaxL) / kThreads;
+  float diag[kAmps];
+#pragma unroll
+  for (int k = 0; k < kAmps; ++k) {
+    const uint32_t x = threadIdx.x + k * kThreads;
+    float d = 0.f;
+    for (int i = 0; i < L; ++i) {
+      const float zi = ((x >> i) & 1) ? -1.f : 1.f;
+      d += ch.cz[i] * zi;
+      if (i + 1 < L) d += ch.Jf * zi * (((x >> (i + 1)) & 1) ? -1.f : 1.f);
+    }
+    diag[k] = d;
+  }
+  const uint32_t q = threadIdx.x;
+  auto gate = [&](int b, const float4* gs) {
+    const uint32_t lowmask = (1u << b) - 1;
+    // local index r = 2 b_b + b_{b+1}: offsets of r = 0..3
+    const uint32_t o1 = 2u << b, o2 = 1u << b, o3 = 3u << b;
+    const uint32_t x = (q & lowmask) | ((q >> b) << (b + 2));
+    const float2 v0 = sp[x], v1 = sp[x + o1], v2 = sp[x + o2], v3 = sp[x + o3];
+    float2 w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) w[r] = czero<float2>();
+    // residual products first, then the table's on top: a bare first
+    // product with a fixed table entry would bias the norm downwards
+#pragma unroll
+    for (int part = 1; part >= 0; --part) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float4 s = gs[8 * part + 2 * r], t = gs[8 * part + 2 * r + 1];
+        w[r] = cmac(w[r], make_float2(s.x, s.y), v0);
+        w[r] = cmac(w[r], make_float2(s.z, s.w), v1);
+        w[r] = cmac(w[r], make_float2(t.x, t.y), v2);
+        w[r] = cmac(w[r], make_float2(t.z, t.w), v3);
+      }
+    }
+    sp[x] = w[0];
+    sp[x + o1] = w[1];
+    sp[x + o2] = w[2];
+    sp[x + o3] = w[3];
+  };
   for (int p = 0; p < periods; ++p) {
     for (int g = 0; g < ch.ngates; ++g) {
-      const int b = ch.bonds[g];
-      float2 G[16], Gl[16];  // gate and its FP32 rounding residual
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        G[k] = ch.gates[kGateEntries * g + k];
-        Gl[k] = ch.gates[kGateEntries * g + 16 + k];
-      }
-      const uint32_t lowmask = (1u << b) - 1;
-      // local index r = 2 b_b + b_{b+1}: offsets of r = 0..3
-      const uint32_t o1 = 2u << b, o2 = 1u << b, o3 = 3u << b;
-      for (uint32_t q = threadIdx.x; q < (n >> 2); q += blockDim.x) {
-        const uint32_t x = (q & lowmask) | ((q >> b) << (b + 2));
-        const float2 v0 = sp[x], v1 = sp[x + o1], v2 = sp[x + o2], v3 = sp[x + o3];
-        float2 w[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          // residual products first, then the table's on top: a bare first
-          // product with a fixed table entry would bias the norm downwards
-          float2 a = czero<float2>();
-          a = cmac(a, Gl[4 * r + 0], v0);
-          a = cmac(a, Gl[4 * r + 1], v1);
-          a = cmac(a, Gl[4 * r + 2], v2);
-          a = cmac(a, Gl[4 * r + 3], v3);
-          a = cmac(a, G[4 * r + 0], v0);
-          a = cmac(a, G[4 * r + 1], v1);
-          a = cmac(a, G[4 * r + 2], v2);
-          a = cmac(a, G[4 * r + 3], v3);
-          w[r] = a;
-        }
-        sp[x] = w[0];
-        sp[x + o1] = w[1];
-        sp[x + o2] = w[2];
-        sp[x + o3] = w[3];
+      if (q < (n >> 2)) {
+        if (held) gate(bonds[g], reinterpret_cast<const float4*>(tables + kGateEntries * g));
+        else gate(__ldg(ch.bonds + g), reinterpret_cast<const float4*>(ch.gates + kGateEntries * g));
       }
       __syncthreads();
     }
-    // <H0> and the norm of the period's final state (natural layout)
-    // per-thread sums over its amplitudes, compensated (Kahan) in FP32
-    float es = 0.f, ec = 0.f, ns = 0.f, nc = 0.f;
-    for (uint32_t x = threadIdx.x; x < n; x += blockDim.x) {
+    // <H0> and the norm of the period's final state
+    double e = 0.0, nn = 0.0;
+#pragma unroll
+    for (int k = 0; k < kAmps; ++k) {
+      const uint32_t x = threadIdx.x + k * kThreads;
+      if (x >= n) break;
       const float2 v = sp[x];
       const float pr = cabs2(v);
-      float d = 0.f;
-      for (int i = 0; i < L; ++i) {
-        const float zi = ((x >> i) & 1) ? -1.f : 1.f;
-        d += s_cz[i] * zi;
-        if (i + 1 < L) d += Jf * zi * (((x >> (i + 1)) & 1) ? -1.f : 1.f);
-      }
       float ex = 0.f;
-      for (int i = 0; i < L; ++i)
-        if (!((x >> i) & 1)) ex += 2.f * s_cx[i] * cdotre(v, sp[x | (1u << i)]);
-      const float ye = (pr * d + ex) - ec, te = es + ye;
-      ec = (te - es) - ye;
-      es = te;
-      const float yn = pr - nc, tn = ns + yn;
-      nc = (tn - ns) - yn;
-      ns = tn;
+#pragma unroll
+      for (int i = 0; i < kShortMaxL; ++i)
+        if (i < L && !((x >> i) & 1)) ex += 2.f * ch.cx[i] * cdotre(v, sp[x | (1u << i)]);
+      e += (double)(pr * diag[k] + ex);
+      nn += (double)pr;
     }
-    double e = (double)es - (double)ec, nn = (double)ns - (double)nc;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       e += __shfl_xor_sync(0xffffffffu, e, o);
@@ -112,41 +123,32 @@ __global__ void __launch_bounds__(kThreads, 1)
       sn[w] = nn;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == kThreads - 32) {  // its warp has no gates in chains below nine sites
       double te = 0.0, tn = 0.0;
-      for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
+      for (int k = 0; k < kThreads / 32; ++k) {
         te += se[k];
         tn += sn[k];
       }
       const long long slot = (p0 + p) % ring_len;
-      ch.ring[2 * slot] = te / ((double)L * tn);
-      ch.ring[2 * slot + 1] = tn;
+      double* const out = ch.ring + 2 * slot * ch.ring_stride;
+      out[0] = te / ((double)L * tn);
+      out[1] = tn;
     }
-    __syncthreads();
   }
-  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) ch.psi[i] = sp[i];
+  for (uint32_t i = threadIdx.x; i < n; i += kThreads) ch.psi[i] = sp[i];
 }
-
-__global__ void k_advance(long long* counter, int periods) { *counter += periods; }
 
 }  // namespace
 
-size_t resident_smem_bytes(int L) { return sizeof(float2) << L; }
-
-cudaError_t resident_prepare(int max_L) {
-  return cudaFuncSetAttribute(k_chain_resident, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)resident_smem_bytes(max_L));
+cudaError_t short_prepare() {
+  // the carve-out of the resident form's blocks, so that both share an SM
+  return cudaFuncSetAttribute(k_chain_short, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
 }
 
-cudaError_t launch_chain_resident(const ResidentChain* chains, int nchains, int max_L,
-                                  long long* counter, int periods, int ring_len,
-                                  cudaStream_t s) {
-  if (nchains <= 0 || periods <= 0) return cudaSuccess;
-  k_chain_resident<<<nchains, kThreads, resident_smem_bytes(max_L), s>>>(chains, counter,
-                                                                        periods, ring_len);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_advance<<<1, 1, 0, s>>>(counter, periods);
+cudaError_t launch_chain_short(const ChainArgs* chains, int nchains, const long long* counter,
+                               int periods, int ring_len, cudaStream_t s) {
+  if (nchains <= 0) return cudaSuccess;
+  k_chain_short<<<nchains, kThreads, 0, s>>>(chains, counter, periods, ring_len);
   return cudaGetLastError();
 }
 

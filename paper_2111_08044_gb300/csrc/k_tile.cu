@@ -11,8 +11,8 @@
 // 0.55 us of it the launch).  With four to six gates a pass the FP32 pipe is
 // the bound.  A pass of four gates at L = 27 takes 588 us (467 us of FMAs at
 // the pipe's 36.8 TFMA/s), where four passes of one gate take 1350 us; a period
-// 17.9 ms (104 gates), before 35.2 ms, at L = 20 0.18 ms for 0.39 ms, at L = 12
-// 47 us for 128 us.
+// 17.9 ms (104 gates), before 35.2 ms, at L = 20 0.18 ms for 0.39 ms.  Chains of
+// up to 15 sites stay in shared memory between periods instead (k_resident.cu).
 //
 // complex64 (k_tile_f32): a thread holds 16 amplitudes (four register bits
 // of the tile) and applies two gates on disjoint sites before it hands them
@@ -43,191 +43,7 @@ namespace {
 
 using namespace dev;
 
-__device__ __forceinline__ double period_scale(const Renorm& rn, long long c) {
-  if (!rn.ring || rn.every <= 0) return 1.0;
-  if (c <= 0 || c % rn.every != 0) return 1.0;
-  const double n2 = *reinterpret_cast<const volatile double*>(rn.ring + 2 * ((c - 1) % rn.ring_len) + 1);
-  return n2 > 0.0 ? 1.0 / sqrt(n2) : 1.0;
-}
-
-// Energy terms of one group of four amplitudes w[r] (r = 2 b_i + b_{i+1}), as
-// the per-gate kernels form them: fixed products first, then one chain of
-// sums per grouping.
-template <typename R>
-struct GroupTerms {
-  R hi, lo, p[4], d[4];
-};
-template <typename R>
-__device__ __forceinline__ void group_terms(const typename CT<R>::C (&w)[4], int epi,
-                                            const Diag<R>& dg, uint64_t x,
-                                            const uint64_t (&off)[4], GroupTerms<R>& t) {
-  if (epi & EPI_X_HI) t.hi = cdotre(w[0], w[2]) + cdotre(w[1], w[3]);
-  if (epi & EPI_X_LO) t.lo = cdotre(w[0], w[1]) + cdotre(w[2], w[3]);
-  if (epi & EPI_DIAG) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      t.p[r] = cabs2(w[r]);
-      t.d[r] = dg(x + off[r]);
-    }
-  }
-}
-// es + c t in one rounding (complex64: as the per-gate kernels add it)
-template <typename R>
-__device__ __forceinline__ R add_term(R es, R c, R t) {
-  return es + c * t;
-}
-template <>
-__device__ __forceinline__ float add_term<float>(float es, float c, float t) {
-  return __fmaf_rn(c, t, es);
-}
-template <typename R>
-__device__ __forceinline__ void group_chain(const GroupTerms<R>& t, int epi, R cxh, R cxl, R& es,
-                                            R& ns) {
-  if (epi & EPI_X_HI) es = add_term<R>(es, cxh * (R)2, t.hi);
-  if (epi & EPI_X_LO) es = add_term<R>(es, cxl * (R)2, t.lo);
-  if (epi & EPI_DIAG) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      ns += t.p[r];
-      es += t.p[r] * t.d[r];
-    }
-  }
-}
-
 // ------------------------------------------------------------- complex64
-// The gate on register bits (J0: site b, J1: site b + 1) of a thread's 16
-// amplitudes; K0, K1 are the other two register bits.  get(e): entry e of the
-// table (16, then 16 of its residual).  Residual products first (see
-// k_plain.cu).  Packed FMAs on (re, im) pairs, each half the scalar chain: with
-// the entries in the constant bank they run at the FP32 pipe's full rate (37.7
-// TFMA/s in registers; scalar FMAs with the same operands 35.0, with entries
-// loaded from shared memory 33) and leave half the issue slots to the loads,
-// stores and addresses.  Each entry serves the four groups in turn.
-template <int J0, int J1, int K0, int K1, bool kXor, typename G>
-__device__ __forceinline__ void gate16(uint64_t (&v)[16], const G& get) {
-  auto idx = [](int r, int k) {
-    return ((r >> 1) << J0) | ((r & 1) << J1) | ((k & 1) << K0) | ((k >> 1) << K1);
-  };
-  uint64_t s[16], w[4][4];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const float2 t = un2(v[m]);
-    s[m] = pk2(t.y, t.x);
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) w[r][k] = 0;
-#pragma unroll
-    for (int part = 1; part >= 0; --part) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = kXor ? r ^ j : j;
-        const ulonglong2 g = get(16 * part + 4 * r + c);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) w[r][k] = fma2(g.x, v[idx(c, k)], w[r][k]);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) w[r][k] = fma2(g.y, s[idx(c, k)], w[r][k]);
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[idx(r, k)] = w[r][k];
-}
-
-template <int J0, int J1, int K0, int K1>
-__device__ __forceinline__ void measure16(const uint64_t (&v)[16], const TileArgs& ta,
-                                          const TileRound& rd, int which, uint64_t x0,
-                                          bool active, FloatSum& esum, FloatSum& nsum) {
-  const int epi = rd.epi[which], bond = rd.bond[which];
-  const float cxh = (float)ta.cx[bond], cxl = (float)ta.cx[bond + 1];
-  Diag<float> dg;
-  if (epi & EPI_DIAG) dg.init(ta.ep, ta.L);
-  const uint64_t ro[4] = {1ull << rd.sbit[0], 1ull << rd.sbit[1], 1ull << rd.sbit[2],
-                          1ull << rd.sbit[3]};
-  const uint64_t off[4] = {0, ro[J1], ro[J0], ro[J0] + ro[J1]};
-  const bool odd = threadIdx.x & 1;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    float2 w[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-      w[r] = un2(v[((r >> 1) << J0) | ((r & 1) << J1) | ((k & 1) << K0) | ((k >> 1) << K1)]);
-    const uint64_t x = x0 + ((k & 1) ? ro[K0] : 0) + ((k >> 1) ? ro[K1] : 0);
-    GroupTerms<float> t;
-    group_terms<float>(w, epi, dg, x, off, t);
-    float es = 0.f, ns = 0.f;
-    group_chain<float>(t, epi, cxh, cxl, es, ns);
-    bool take = active;
-    if (rd.egroup[which] == TILE_E_PAIR) {
-      // the neighbour's sum (bit 0 clear) continues in the lane with bit 0 set
-      float e2 = __shfl_xor_sync(0xffffffffu, es, 1), n2 = 0.f;
-      if (epi & EPI_DIAG) n2 = __shfl_xor_sync(0xffffffffu, ns, 1);
-      group_chain<float>(t, epi, cxh, cxl, e2, n2);
-      es = e2;
-      ns = n2;
-      take = active && odd;
-    }
-    if (take) {
-      esum.add(es);
-      if (epi & EPI_DIAG) nsum.add(ns);
-    }
-  }
-}
-
-// A measured gate on bonds 0..5 of a chain of at least 8 sites, from the tile:
-// the sums of the per-gate kernel, whose threads hold bits 0, 6 and 7.
-__device__ __noinline__ void measure_sweep(const uint8_t* tile, const TileArgs& ta, int bond, int epi,
-                                           uint64_t tbase, FloatSum& esum, FloatSum& nsum) {
-  const float cxh = (float)ta.cx[bond], cxl = (float)ta.cx[bond + 1];
-  Diag<float> dg;
-  if (epi & EPI_DIAG) dg.init(ta.ep, ta.L);
-  const uint32_t nv = 1u << (ta.tb - 3);
-  auto at = [&](uint32_t e) { return *reinterpret_cast<const float2*>(tile + tile_byte8(e)); };
-  for (uint32_t vt = threadIdx.x; vt < nv; vt += blockDim.x) {
-    const uint32_t e0 = ((vt & 31u) << 1) | ((vt >> 5) << 8);
-    float2 w[4][2];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int k = 0; k < 2; ++k) w[c][k] = at(e0 | (c << 6) | k);
-    float es = 0.f, ns = 0.f;
-    if (epi & EPI_X_HI) {
-      float s = 0.f;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-          s += cdotre(w[c][k], at((e0 | (c << 6) | k) ^ (1u << bond)));
-      es += cxh * s;
-    }
-    if (epi & EPI_X_LO) {
-      float s = 0.f;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-          s += cdotre(w[c][k], at((e0 | (c << 6) | k) ^ (2u << bond)));
-      es += cxl * s;
-    }
-    if (epi & EPI_DIAG) {
-      const uint64_t x0 = tbase + elem_state(ta, e0);
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const float pr = cabs2(w[c][k]);
-          ns += pr;
-          es += pr * dg(x0 + ((uint64_t)c << 6) + k);
-        }
-    }
-    esum.add(es);
-    if (epi & EPI_DIAG) nsum.add(ns);
-  }
-}
-
 // sum of (e, n) over the block in thread 0 (fixed order)
 __device__ __forceinline__ void block_sum_pair(double& e, double& n, double* sh) {
 #pragma unroll
@@ -299,9 +115,8 @@ __device__ __forceinline__ void load_packed(const TileArgs& ta, PackedEntry* gs,
 template <int kSlots, bool kXor, bool kEpi, int kThreads, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_tile_f32(float2* __restrict__ psi, const __grid_constant__ TileArgs ta,
-               const __grid_constant__ TileTab<kSlots ? kSlots : 1> tab) {
+               const __grid_constant__ TileTabOf<kSlots ? kSlots : 1> tab) {
   extern __shared__ __align__(16) uint8_t tile_smem[];
-  __shared__ double red[2 * 16];
   const uint32_t tile_bytes = tile_byte8(1u << ta.tb);
   PackedEntry* gs = reinterpret_cast<PackedEntry*>(tile_smem + (size_t)ta.buffers * tile_bytes);
   TileRound* rds = reinterpret_cast<TileRound*>(gs + (size_t)ta.ngates * kGateEntries);
@@ -318,100 +133,92 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
     for (int k = threadIdx.x; k < 2 * ta.nrounds; k += blockDim.x)
       reinterpret_cast<uint4*>(rds)[k] = reinterpret_cast<const uint4*>(ta.rounds)[k];
   const bool reload = kSlots == 0 && (ta.stride != 0 || (ta.first && ta.ep.rn.ring));
-  const long long c0 = reload || ta.periods > 0 ? *ta.counter : 0;
-  const int periods = ta.periods > 0 ? ta.periods : 1;
+  const long long c0 = reload ? *ta.counter : 0;
   double eacc = 0.0, nacc = 0.0;
   FloatSum esum, nsum;
-  for (int p = 0; p < periods; ++p) {
-    if (kSlots == 0 && (p == 0 || reload)) load_packed(ta, gs, c0 + p);
-    int cur = 0;
-    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-      const uint64_t tbase = tile_base(ta, t);
-      uint8_t* tile = tile_smem + (size_t)cur * tile_bytes;
-      if (ta.buffers == 2 && t + gridDim.x < ntiles) {
-        load_tile(ta, io, sbuf + (cur ^ 1) * tile_bytes, psi + tile_base(ta, t + gridDim.x));
-        cp_wait<1>();
-      } else {
-        cp_wait<0>();
-      }
-      __syncthreads();
-      for (int r = 0; r < ta.nrounds; ++r) {
-        const TileRound& rd = kSlots ? tab.r[r] : rds[r];
-        const uint32_t e0 = thread_elem<4>(rd, tid);
-        uint8_t* const at = tile + tile_byte8(e0);
-        uint64_t v[16];
-        const uint32_t sl0 = rd.slot[0], sl1 = rd.slot[1], sl2 = rd.slot[2], sl3 = rd.slot[3];
+  if (kSlots == 0) load_packed(ta, gs, c0);
+  int cur = 0;
+  const int last_r = ta.direct_out ? ta.nrounds - 1 : -1;  // the round that writes the state
+  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const uint64_t tbase = tile_base(ta, t);
+    uint8_t* tile = tile_smem + (size_t)cur * tile_bytes;
+    if (ta.buffers == 2 && t + gridDim.x < ntiles) {
+      load_tile(ta, io, sbuf + (cur ^ 1) * tile_bytes, psi + tile_base(ta, t + gridDim.x));
+      cp_wait<1>();
+    } else {
+      cp_wait<0>();
+    }
+    __syncthreads();
+    for (int r = 0; r < ta.nrounds; ++r) {
+      const TileRound& rd = kSlots ? tab.r[r] : rds[r];
+      const uint32_t e0 = thread_elem<4>(rd, tid);
+      uint8_t* const at = tile + tile_byte8(e0);
+      uint64_t v[16];
+      const uint32_t sl0 = rd.slot[0], sl1 = rd.slot[1], sl2 = rd.slot[2], sl3 = rd.slot[3];
 #pragma unroll
-        for (int m = 0; m < 16; ++m)
-          v[m] = *reinterpret_cast<const uint64_t*>(
-              at + (((m & 1) ? sl0 : 0) + ((m & 2) ? sl1 : 0) + ((m & 4) ? sl2 : 0) + ((m & 8) ? sl3 : 0)));
-        const int ga = rd.gate[0], gb = rd.gate[1];
-        auto from = [&](int g) {
-          return [&, g](int e) {
-            return *reinterpret_cast<const ulonglong2*>(kSlots ? &tab.g[g][e]
-                                                               : &gs[g * kGateEntries + e]);
-          };
+      for (int m = 0; m < 16; ++m)
+        v[m] = *reinterpret_cast<const uint64_t*>(
+            at + (((m & 1) ? sl0 : 0) + ((m & 2) ? sl1 : 0) + ((m & 4) ? sl2 : 0) + ((m & 8) ? sl3 : 0)));
+      const int ga = rd.gate[0], gb = rd.gate[1];
+      auto from = [&](int g) {
+        return [&, g](int e) {
+          return *reinterpret_cast<const ulonglong2*>(kSlots ? &tab.g[g][e]
+                                                             : &gs[g * kGateEntries + e]);
         };
-        if (kXor && rd.xorder[0]) gate16<0, 1, 2, 3, true>(v, from(ga));
-        else gate16<0, 1, 2, 3, false>(v, from(ga));
-        if (kEpi && rd.epi[0] && rd.egroup[0] != TILE_E_SWEEP)
-          measure16<0, 1, 2, 3>(v, ta, rd, 0, tbase + elem_state(ta, e0), active, esum, nsum);
-        if (gb >= 0) {
-          if (kXor && rd.xorder[1]) gate16<2, 3, 0, 1, true>(v, from(gb));
-          else gate16<2, 3, 0, 1, false>(v, from(gb));
-          if (kEpi && rd.epi[1] && rd.egroup[1] != TILE_E_SWEEP)
-            measure16<2, 3, 0, 1>(v, ta, rd, 1, tbase + elem_state(ta, e0), active, esum, nsum);
-        }
-        if (active) {
-          if (r == ta.nrounds - 1 && ta.direct_out && p == periods - 1) {
-            uint64_t* out = reinterpret_cast<uint64_t*>(psi + tbase + xout);
-            const uint64_t ro[4] = {1ull << rd.sbit[0], 1ull << rd.sbit[1], 1ull << rd.sbit[2],
-                                    1ull << rd.sbit[3]};
+      };
+      if (kXor && rd.xorder[0]) gate16<0, 1, 2, 3, true>(v, from(ga));
+      else gate16<0, 1, 2, 3, false>(v, from(ga));
+      if (kEpi && rd.epi[0] && rd.egroup[0] != TILE_E_SWEEP)
+        measure16<0, 1, 2, 3>(v, ta.L, ta.cx, ta.ep, rd, 0, tbase + elem_state(ta, e0), active, esum,
+                              nsum);
+      if (rd.count == 2) {
+        if (kXor && rd.xorder[1]) gate16<2, 3, 0, 1, true>(v, from(gb));
+        else gate16<2, 3, 0, 1, false>(v, from(gb));
+        if (kEpi && rd.epi[1] && rd.egroup[1] != TILE_E_SWEEP)
+          measure16<2, 3, 0, 1>(v, ta.L, ta.cx, ta.ep, rd, 1, tbase + elem_state(ta, e0), active, esum,
+                                nsum);
+      }
+      if (active) {
+        if (r == last_r) {
+          uint64_t* out = reinterpret_cast<uint64_t*>(psi + tbase + xout);
+          const uint64_t ro[4] = {1ull << rd.sbit[0], 1ull << rd.sbit[1], 1ull << rd.sbit[2],
+                                  1ull << rd.sbit[3]};
 #pragma unroll
-            for (int m = 0; m < 16; ++m)
-              out[((m & 1) ? ro[0] : 0) + ((m & 2) ? ro[1] : 0) + ((m & 4) ? ro[2] : 0) +
-                  ((m & 8) ? ro[3] : 0)] = v[m];
-          } else {
+          for (int m = 0; m < 16; ++m)
+            out[((m & 1) ? ro[0] : 0) + ((m & 2) ? ro[1] : 0) + ((m & 4) ? ro[2] : 0) +
+                ((m & 8) ? ro[3] : 0)] = v[m];
+        } else {
 #pragma unroll
-            for (int m = 0; m < 16; ++m)
-              *reinterpret_cast<uint64_t*>(at + (((m & 1) ? sl0 : 0) + ((m & 2) ? sl1 : 0) +
-                                               ((m & 4) ? sl2 : 0) + ((m & 8) ? sl3 : 0))) = v[m];
-          }
-        }
-        // between rounds, and before the buffer takes another tile
-        __syncthreads();
-        if (kEpi) {
-          const int sw = rd.egroup[1] == TILE_E_SWEEP ? 1 : rd.egroup[0] == TILE_E_SWEEP ? 0 : -1;
-          if (sw >= 0) {
-            measure_sweep(tile, ta, rd.bond[sw], rd.epi[sw], tbase, esum, nsum);
-            __syncthreads();
-          }
+          for (int m = 0; m < 16; ++m)
+            *reinterpret_cast<uint64_t*>(at + (((m & 1) ? sl0 : 0) + ((m & 2) ? sl1 : 0) +
+                                             ((m & 4) ? sl2 : 0) + ((m & 8) ? sl3 : 0))) = v[m];
         }
       }
-      if (kEpi && ta.any_epi) {
-        esum.flush(eacc);
-        nsum.flush(nacc);
-      }
-      if (!ta.direct_out && p == periods - 1) {
-        store_tile(ta, io, tile, psi + tbase);
-        __syncthreads();
-      }
-      if (ta.buffers == 2) cur ^= 1;
-      else if (t + gridDim.x < ntiles) {
-        load_tile(ta, io, sbuf, psi + tile_base(ta, t + gridDim.x));
+      // between rounds, and before the buffer takes another tile
+      __syncthreads();
+      if (kEpi) {
+        const int sw = rd.egroup[1] == TILE_E_SWEEP ? 1 : rd.egroup[0] == TILE_E_SWEEP ? 0 : -1;
+        if (sw >= 0) {
+          measure_sweep(tile, ta.tb, ta.L, ta.cx, ta.ep, rd.bond[sw], rd.epi[sw],
+                        [&](uint32_t e) { return tbase + elem_state(ta, e); }, esum, nsum);
+          __syncthreads();
+        }
       }
     }
-    if (ta.periods > 0) {
-      block_sum_pair(eacc, nacc, red);
-      if (threadIdx.x == 0) ring_store(ta, c0 + p, eacc, nacc);
-      eacc = 0.0;
-      nacc = 0.0;
+    if (kEpi && ta.any_epi) {
+      esum.flush(eacc);
+      nsum.flush(nacc);
+    }
+    if (!ta.direct_out) {
+      store_tile(ta, io, tile, psi + tbase);
       __syncthreads();
+    }
+    if (ta.buffers == 2) cur ^= 1;
+    else if (t + gridDim.x < ntiles) {
+      load_tile(ta, io, sbuf, psi + tile_base(ta, t + gridDim.x));
     }
   }
-  if (ta.periods > 0) {
-    if (threadIdx.x == 0) *ta.counter_rw = c0 + periods;
-  } else if (kEpi && ta.ep.partial) {
+  if (kEpi && ta.ep.partial) {
     block_store_pair(eacc, nacc, ta.ep.partial);
   }
 }
@@ -517,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
           __syncthreads();
         }
         if (rd.epi[0] && active) {
-          const R cxh = (R)ta.cx[rd.bond[0]], cxl = (R)ta.cx[rd.bond[0] + 1];
+          const R cxh = (R)ta.cx64[rd.bond[0]], cxl = (R)ta.cx64[rd.bond[0] + 1];
           Diag<R> dg;
           if (rd.epi[0] & EPI_DIAG) dg.init(ta.ep, ta.L);
           const uint64_t off[4] = {0, xl, xh, xh + xl};
@@ -565,24 +372,13 @@ size_t tile_smem_bytes(int precision, const TileArgs& ta) {
   return b;
 }
 
-template <int kSlots>
-const void* f32_kernel(const TileArgs& ta) {
-  if (ta.tb > 12) return reinterpret_cast<const void*>(k_tile_f32<kSlots, true, true, 512, 1>);
-  // a whole chain in one block, or tables in shared memory: the general form
-  if (kSlots != kTileTabSmall)
-    return reinterpret_cast<const void*>(k_tile_f32<kSlots, true, true, 256, 2>);
-  if (ta.any_epi) return reinterpret_cast<const void*>(k_tile_f32<kTileTabSmall, true, true, 256, 2>);
-  return ta.any_xorder ? reinterpret_cast<const void*>(k_tile_f32<kTileTabSmall, true, false, 256, 3>)
-                       : reinterpret_cast<const void*>(k_tile_f32<kTileTabSmall, false, false, 256, 3>);
-}
-
-bool small_tab(const TileArgs& ta) { return ta.ngates <= kTileTabSmall && ta.nrounds <= kTileTabSmall; }
-
 const void* tile_kernel(int precision, const TileArgs& ta) {
   if (precision == SV_DF64) return reinterpret_cast<const void*>(k_tile_wide<df, 256, 2>);
   if (precision == SV_C128) return reinterpret_cast<const void*>(k_tile_wide<double, 512, 2>);
-  if (!ta.in_params) return f32_kernel<0>(ta);
-  return small_tab(ta) ? f32_kernel<kTileTabSmall>(ta) : f32_kernel<kTileMaxGates>(ta);
+  if (!ta.in_params) return reinterpret_cast<const void*>(k_tile_f32<0, true, true, 256, 2>);
+  if (ta.any_epi) return reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, true, 256, 2>);
+  return ta.any_xorder ? reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, false, 256, 3>)
+                       : reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, false, false, 256, 3>);
 }
 
 }  // namespace
@@ -607,24 +403,13 @@ cudaError_t tile_grid(int precision, TileArgs* ta, const LaunchCfg& cfg, int* gr
   return e;
 }
 
-cudaError_t launch_tile(int precision, void* psi, const TileArgs& ta,
-                        const TileTab<kTileMaxGates>* tab, int grid, cudaStream_t s) {
-  const int threads = tile_threads(precision, ta.tb);
-  const size_t smem = tile_smem_bytes(precision, ta);
-  const void* kernel = tile_kernel(precision, ta);
-  TileTab<kTileTabSmall> small;
-  TileTab<1> none;
+cudaError_t launch_tile(int precision, void* psi, const TileArgs& ta, const TileTab* tab, int grid,
+                        cudaStream_t s) {
+  TileTabOf<1> none;
   void* args[] = {&psi, const_cast<TileArgs*>(&ta), nullptr};
-  if (precision == SV_C64 && !ta.in_params) {
-    args[2] = &none;
-  } else if (precision == SV_C64 && small_tab(ta)) {
-    std::memcpy(small.g, tab->g, sizeof(small.g));
-    std::memcpy(small.r, tab->r, sizeof(small.r));
-    args[2] = &small;
-  } else if (precision == SV_C64) {
-    args[2] = const_cast<TileTab<kTileMaxGates>*>(tab);
-  }
-  return cudaLaunchKernel(kernel, dim3(grid), dim3(threads), args, smem, s);
+  if (precision == SV_C64) args[2] = ta.in_params ? (void*)const_cast<TileTab*>(tab) : (void*)&none;
+  return cudaLaunchKernel(tile_kernel(precision, ta), dim3(grid), dim3(tile_threads(precision, ta.tb)),
+                          args, tile_smem_bytes(precision, ta), s);
 }
 
 }  // namespace fsv

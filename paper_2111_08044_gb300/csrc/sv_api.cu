@@ -70,10 +70,14 @@ struct sv_ctx {
   struct TileLaunch {
     fsv::TileArgs ta;
     int grid = 0;
-    std::unique_ptr<fsv::TileTab<fsv::kTileMaxGates>> tab;  // complex64, fixed gates
+    std::unique_ptr<fsv::TileTab> tab;  // complex64, fixed gates
   };
   std::vector<TileLaunch> tiles;
-  bool tile_single = false;  // one tile holds the chain: whole periods in one launch
+  bool tile_single = false;  // one block (or cluster) holds the chain: runs of whole
+                             // periods in one launch
+  bool resident = false;     // complex64: that launch is the resident form's
+  fsv::ChainArgs chain;
+  fsv::ResidentShape shape;
   long long part_pairs = 0;  // partial pairs of a period
 
   cudaGraphExec_t graph = nullptr;       // one period
@@ -162,6 +166,7 @@ void free_build(sv_ctx* ctx) {
   ctx->mg.clear();
   ctx->tiles.clear();
   ctx->tile_single = false;
+  ctx->resident = false;
   if (ctx->block) {
     fsv::block_free(ctx->block);
     ctx->block = nullptr;
@@ -215,11 +220,17 @@ int enqueue_multigate_period(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev) {
   return SV_OK;
 }
 
-// `periods` periods of a chain that one tile holds, in one launch.
+// `periods` periods of a chain that one block or cluster holds, in one launch.
 int enqueue_tile_run(sv_ctx* ctx, int64_t periods, cudaStream_t s) {
+  if (ctx->resident) {
+    fsv::ChainArgs ch = ctx->chain;
+    ch.psi = static_cast<float2*>(ctx->state);
+    SV_CUDA(fsv::launch_resident_chain(ch, ctx->shape, (int)periods, kRing, s), "resident launch");
+    return SV_OK;
+  }
   fsv::TileArgs ta = ctx->tiles[0].ta;
   ta.periods = (int)periods;
-  SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, ta, ctx->tiles[0].tab.get(), 1, s), "tile launch");
+  SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, ta, nullptr, 1, s), "tile launch");
   return SV_OK;
 }
 
@@ -248,7 +259,7 @@ int enqueue_tile_period(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev) {
 // Enqueue one plain-mode period on stream s.
 int enqueue_plain_period(sv_ctx* ctx, cudaStream_t s) {
   if (ctx->params.mode == SV_MODE_MULTIGATE) return enqueue_multigate_period(ctx, s, nullptr);
-  if (!ctx->tiles.empty()) return enqueue_tile_period(ctx, s, nullptr);
+  if (ctx->tile_single || !ctx->tiles.empty()) return enqueue_tile_period(ctx, s, nullptr);
   const int ng = (int)ctx->gates.size();
   const size_t cbytes = amp_bytes(ctx->precision);
   const long long stride = ctx->n_period_params > 0 ? (long long)ng * fsv::kGateEntries : 0;
@@ -318,9 +329,14 @@ int launch_periods(sv_ctx* ctx, int64_t count, bool last) {
   const bool off = off_natural(ctx);
   if (count <= 0) return SV_OK;
   if (ctx->tile_single) {
-    int rc = enqueue_tile_run(ctx, count, ctx->stream);
-    if (rc) return rc;
-    ctx->counter += count;
+    // runs of at most 2^15 gates a launch (tens of milliseconds)
+    const int64_t most = std::max<int64_t>(1, 32768 / (int64_t)ctx->gates.size());
+    for (int64_t k = 0; k < count; k += most) {
+      const int64_t n = std::min(most, count - k);
+      int rc = enqueue_tile_run(ctx, n, ctx->stream);
+      if (rc) return rc;
+      ctx->counter += n;
+    }
     return SV_OK;
   }
   if (off && !ctx->in_period_layout) {
@@ -734,7 +750,7 @@ int enqueue_period_profiled(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev, bool l
     return SV_OK;
   }
   if (ctx->params.mode == SV_MODE_MULTIGATE) return enqueue_multigate_period(ctx, s, ev);
-  if (!ctx->tiles.empty()) return enqueue_tile_period(ctx, s, ev);
+  if (ctx->tile_single || !ctx->tiles.empty()) return enqueue_tile_period(ctx, s, ev);
   const int ng = (int)ctx->gates.size();
   const size_t cbytes = amp_bytes(ctx->precision);
   const long long stride = ctx->n_period_params > 0 ? (long long)ng * fsv::kGateEntries : 0;
@@ -864,11 +880,49 @@ bool tile_runs(int L, const fsv::TilePassPlan& p, fsv::TileArgs* ta) {
   return true;
 }
 
+// A plain-mode chain held in a block's or cluster's shared memory.
+int build_resident_chain(sv_ctx* ctx) {
+  const int L = ctx->L;
+  const auto rounds = fsv::resident_rounds(ctx->gates, ctx->shape);
+  fsv::ChainArgs& ch = ctx->chain;
+  ch = fsv::ChainArgs();
+  ch.L = L;
+  ch.ngates = (int)ctx->gates.size();
+  ch.nrounds = (int)rounds.size();
+  ch.gates = static_cast<const float2*>(ctx->d_gates);
+  ch.stride = ctx->n_period_params > 0 ? (long long)ch.ngates * fsv::kGateEntries : 0;
+  ch.ring = ctx->d_ring;
+  ch.counter = ctx->d_counter;
+  for (int i = 0; i < L && !ctx->obs.general; ++i) ch.cx[i] = (float)ctx->obs.cx[i];
+  ch.ep = epi_for(ctx, ctx->obs.general ? 0 : fsv::EPI_DIAG, 0, nullptr);
+  ch.ep.rn = renorm_of(ctx);
+  const size_t bytes = rounds.size() * sizeof(fsv::ResidentRound);
+  char* d_rounds = static_cast<char*>(ctx->d_gates) + ctx->d_gates_bytes;  // behind the tables
+  SV_CUDA(cudaMemcpy(d_rounds, rounds.data(), bytes, cudaMemcpyHostToDevice), "upload rounds");
+  ch.rounds = reinterpret_cast<const fsv::ResidentRound*>(d_rounds);
+  ctx->tile_single = ctx->resident = true;
+  ctx->passes_per_period = 1;
+  ctx->launches_per_period = 1;
+  ctx->build_bytes = ctx->d_gates_bytes + bytes;
+  return SV_OK;
+}
+
 // The tile passes of a plain-mode period (none on chains too short for them):
 // their rounds on the device, the launch arguments, the partial pairs.
 // host_tab: the first period's complex64 tables.
 int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab) {
   const int L = ctx->L, ng = (int)ctx->gates.size();
+  if (ctx->precision == SV_C64 && L >= 5 && L <= fsv::kResidentPlainMaxL) {
+    int clusters = 0;
+    for (int most = 16; clusters < 1 && most >= 8; most /= 2) {
+      ctx->shape = fsv::resident_shape(true, L, most);
+      if (fsv::resident_prepare(true, ctx->shape, ng, &clusters) != cudaSuccess) {
+        cudaGetLastError();
+        clusters = 0;
+      }
+    }
+    if (clusters > 0) return build_resident_chain(ctx);
+  }
   const int tb = fsv::tile_bits(L, ctx->gates, ctx->precision, ctx->cfg.num_sms);
   if (tb == 0) return SV_OK;
   const auto plan = fsv::tile_plan(L, ctx->gates, ctx->precision, tb);
@@ -895,11 +949,14 @@ int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab) {
     int epi = 0;
     for (int g : p.gates) epi |= ctx->gates[g].epi;
     ta.ep = epi_for(ctx, epi & fsv::EPI_DIAG, 0, nullptr);
-    for (int i = 0; i < L && !ctx->obs.general; ++i) ta.cx[i] = ctx->obs.cx[i];
+    for (int i = 0; i < L && !ctx->obs.general; ++i) {
+      ta.cx64[i] = ctx->obs.cx[i];
+      ta.cx[i] = (float)ctx->obs.cx[i];
+    }
     if (ta.first) ta.ep.rn = renorm_of(ctx);
     if (ctx->precision == SV_C64 && ta.stride == 0 && !ta.ep.rn.ring) {
       ta.in_params = 1;
-      t.tab.reset(new fsv::TileTab<fsv::kTileMaxGates>());
+      t.tab.reset(new fsv::TileTab());
       for (size_t e = 0; e < p.gates.size() * fsv::kGateEntries; ++e) {
         const float2 g = host_tab[(size_t)p.gates[0] * fsv::kGateEntries + e];
         t.tab->g[0][e] = fsv::PackedEntry{{g.x, g.x}, {-g.y, g.y}};
@@ -972,15 +1029,23 @@ class RoundedGates {
   std::vector<std::unique_ptr<Entry>> seen_;
 };
 
-void upload_gates(const std::vector<fsv::Gate2>& gates, std::vector<float2>& out, size_t at) {
+}  // namespace
+namespace fsv {
+void gate_tables(const std::vector<Gate2>& gates, float2* out) {
   RoundedGates rounded;
   for (size_t g = 0; g < gates.size(); ++g) {
-    float2* e = &out[at + fsv::kGateEntries * g];
+    float2* e = out + kGateEntries * g;
     std::memcpy(e, rounded.get(gates[g].m), 16 * sizeof(float2));
     for (int k = 0; k < 16; ++k)
       e[16 + k] = make_float2((float)(gates[g].m[k].real() - (double)e[k].x),
                               (float)(gates[g].m[k].imag() - (double)e[k].y));
   }
+}
+}  // namespace fsv
+namespace {
+
+void upload_gates(const std::vector<fsv::Gate2>& gates, std::vector<float2>& out, size_t at) {
+  fsv::gate_tables(gates, &out[at]);
 }
 
 // double-float entries (re hi, re lo, im hi, im lo): hi the nearest float,
@@ -1119,7 +1184,7 @@ int adjoint_tiles(sv_ctx* ctx, int64_t P, const std::vector<fsv::AdjOp>& ops, in
             "adjoint seed launch");
     SV_CUDA(fsv::launch_grad_reduce(d_part, seed_grid, d_grad + 2 * P, 0, ctx->stream),
             "energy reduce launch");
-    std::unique_ptr<fsv::TileTab<fsv::kTileMaxGates>> tt(new fsv::TileTab<fsv::kTileMaxGates>());
+    std::unique_ptr<fsv::TileTab> tt(new fsv::TileTab());
     for (int64_t k1 = P; k1 > 0; k1 -= std::min(k1, chunk)) {
       const int64_t k0 = k1 - std::min(k1, chunk);
       for (int64_t k = k1 - 1; k >= k0; --k) {
@@ -1370,7 +1435,10 @@ int sv_build_floquet(sv_ctx* ctx, const sv_floquet_params* p) {
     const size_t cb = amp_bytes(ctx->precision);
     ctx->d_gates_bytes = (size_t)ntab * ng * fsv::kGateEntries * cb;
     // plain mode: at most one round per gate behind the tables
-    const size_t round_bytes = p->mode == SV_MODE_PLAIN ? (size_t)ng * sizeof(fsv::TileRound) : 0;
+    const size_t round_bytes =
+        p->mode == SV_MODE_PLAIN
+            ? (size_t)ng * std::max(sizeof(fsv::TileRound), sizeof(fsv::ResidentRound))
+            : 0;
     if (cudaMalloc(&ctx->d_gates, ctx->d_gates_bytes + round_bytes) != cudaSuccess) {
       cudaGetLastError();
       ctx->d_gates = nullptr;

@@ -4,8 +4,8 @@
 //
 // Every chain gets a context (sv_ctx) on its slice for initialisation and,
 // for the plain, block and multi-gate forms, for its evolution graph.  Chains of at most
-// 14 sites may instead run the resident form (k_batch.cu): one launch
-// advances all of them, each in one CTA's shared memory.  An evolution is
+// 14 sites may instead run the resident form (k_resident.cu): one launch per
+// length advances them, each in the shared memory of one CTA or of a cluster.  An evolution is
 // one CUDA graph per run of M periods: the resident launch; one branch per
 // group of tensor-core chains whose plans share their structure (same L),
 // each pass of all its chains one launch over all their tiles and each
@@ -19,8 +19,9 @@
 // CUDA-core block form at widths n = 5, 6 and 7, the tensor-core block form
 // as a group, the plain, multi-gate and resident forms), and keeps the
 // fastest (most chain-periods per second) for all chains of that L.  The resident form is
-// timed on all chains of that L (one CTA each, so its rate grows with their
-// number); the others, which fill the device with one chain, on up to eight.
+// timed on all chains of that L (one or a few CTAs each, so its rate grows with
+// their number), the tensor-core form on a group that fills the device, the
+// others, which fill it with one chain, on up to eight.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,6 +35,33 @@
 
 #include "sv_batch.h"
 #include "sv_block.h"
+
+// The resident chains' device tables: descriptors, gates, rounds (or the
+// short chains' bonds), energy rings and the shared period counter; the launches, one
+// per chain length (shape.L = 0: the chains of up to kShortMaxL sites).
+struct ResidentSet {
+  struct Class {
+    fsv::ResidentShape shape;
+    int first = 0, count = 0, ngates = 0;
+    Class() { shape.L = 0; }
+  };
+  fsv::ChainArgs* d_res = nullptr;
+  float2* d_gates = nullptr;
+  fsv::ResidentRound* d_rounds = nullptr;
+  double* d_ring = nullptr;
+  long long* d_count = nullptr;
+  int count = 0;
+  std::vector<Class> classes;
+  std::vector<int> place;  // ring of the k-th chain of the set
+  void release() {
+    cudaFree(d_res);
+    cudaFree(d_gates);
+    cudaFree(d_rounds);
+    cudaFree(d_ring);
+    cudaFree(d_count);
+    *this = ResidentSet();
+  }
+};
 
 struct sv_batch {
   int device = 0;
@@ -50,14 +78,12 @@ struct sv_batch {
   std::vector<sv_ctx*> ctx;
   // resident chains
   std::vector<int> res;
-  fsv::ResidentChain* d_res = nullptr;
-  float2* d_rgates = nullptr;
-  int* d_rbonds = nullptr;
-  double* d_rring = nullptr;
-  long long* d_rcount = nullptr;
-  int res_maxL = 0;
+  ResidentSet rset;
   // graphs of one period and of M periods of every chain
   cudaGraphExec_t g1 = nullptr, gm = nullptr;
+  // of a batch whose chains all are resident: d_count[1] (run) periods
+  cudaGraphExec_t gr = nullptr;
+  int64_t run = 0;
   std::vector<fsv::BlockGroup*> groups;  // chain groups the two graphs launch
   int M = 16;
   int64_t counter = 0;
@@ -102,87 +128,115 @@ bool form_fits(int form, int L) {
   }
 }
 
-// The resident chains' device tables: descriptors, gates, bonds, energy
-// rings and the shared period counter.
-struct ResidentSet {
-  fsv::ResidentChain* d_res = nullptr;
-  float2* d_gates = nullptr;
-  int* d_bonds = nullptr;
-  double* d_ring = nullptr;
-  long long* d_count = nullptr;
-  int max_L = 0;
-  int count = 0;
-  void release() {
-    cudaFree(d_res);
-    cudaFree(d_gates);
-    cudaFree(d_bonds);
-    cudaFree(d_ring);
-    cudaFree(d_count);
-    *this = ResidentSet();
-  }
-};
-
 int build_resident(sv_batch* b, const std::vector<int>& chains, ResidentSet* rs) {
   *rs = ResidentSet();
   if (chains.empty()) return SV_OK;
   const int ring = fsv::ctx_ring_len();
-  std::vector<fsv::ResidentChain> hd(chains.size());
-  std::vector<float2> gates;
-  std::vector<int> bonds;
-  std::vector<size_t> goff(chains.size());
-  for (size_t k = 0; k < chains.size(); ++k) {
-    const int c = chains[k];
-    const sv_floquet_params& p = b->params[c];
-    auto pg = fsv::period_gates(b->L[c], p, p.theta, p.hx);
-    goff[k] = bonds.size();
-    for (auto& g : pg) {
-      float2 m[fsv::kGateEntries];
-      fsv::round_unitary4(g.m, m);
-      for (int e = 0; e < 16; ++e)
-        m[16 + e] = make_float2((float)(g.m[e].real() - (double)m[e].x),
-                                (float)(g.m[e].imag() - (double)m[e].y));
-      gates.insert(gates.end(), m, m + fsv::kGateEntries);
-      bonds.push_back(g.bond);
+  // chains of one length together, each length one launch; set order: by length,
+  // then as given
+  std::vector<int> order(chains.size());
+  for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int x, int y) { return b->L[chains[x]] > b->L[chains[y]]; });
+  // a chain takes several blocks where the device has SMs left over
+  int sms = 0;
+  BCUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device), "SM count");
+  std::map<int, int> count, blocks;
+  for (int c : chains) ++count[b->L[c]];
+  int used = (int)chains.size();
+  for (auto& kv : count) blocks[kv.first] = 1;
+  for (bool grew = true; grew;) {
+    grew = false;
+    for (auto it = count.rbegin(); it != count.rend(); ++it) {  // the longest chains first
+      const int L = it->first, n = it->second, now = blocks[L];
+      if (now >= 8 || used + n * now > sms) continue;
+      if (fsv::resident_shape(false, L, 2 * now).kbits == fsv::resident_shape(false, L, now).kbits) continue;
+      blocks[L] = 2 * now;
+      used += n * now;
+      grew = true;
+      break;
     }
-    fsv::Observable o = fsv::observable(b->L[c], p);
-    fsv::ResidentChain& r = hd[k];
-    r.L = b->L[c];
-    r.ngates = (int)pg.size();
-    r.J = o.J;
-    for (int i = 0; i < r.L; ++i) {
-      r.cx[i] = o.cx[i];
-      r.cz[i] = o.cz[i];
-    }
-    rs->max_L = std::max(rs->max_L, r.L);
   }
+  std::vector<fsv::ChainArgs> hd(chains.size());
+  std::vector<float2> gates;
+  std::vector<fsv::ResidentRound> rounds;
+  std::vector<int> bonds;
+  std::vector<size_t> goff(chains.size()), roff(chains.size()), boff(chains.size());
+  for (size_t k = 0; k < chains.size(); ++k) {
+    const int c = chains[order[k]];
+    const int L = b->L[c];
+    const sv_floquet_params& p = b->params[c];
+    auto pg = fsv::period_gates(L, p, p.theta, p.hx);
+    goff[k] = gates.size();
+    gates.resize(gates.size() + pg.size() * fsv::kGateEntries);
+    fsv::gate_tables(pg, &gates[goff[k]]);
+    fsv::ChainArgs& r = hd[k];
+    r.L = L;
+    r.ngates = (int)pg.size();
+    fsv::Observable o = fsv::observable(L, p);
+    r.Jf = (float)o.J;
+    for (int i = 0; i < L; ++i) {
+      r.cx[i] = (float)o.cx[i];
+      r.cz[i] = (float)o.cz[i];
+    }
+    boff[k] = bonds.size();
+    roff[k] = rounds.size();
+    if (L <= fsv::kShortMaxL) {
+      for (auto& g : pg) bonds.push_back(g.bond);
+      if (rs->classes.empty() || rs->classes.back().shape.L != 0) rs->classes.push_back({});
+    } else {
+      const fsv::ResidentShape sh = fsv::resident_shape(false, L, blocks[L]);
+      auto rr = fsv::resident_rounds(pg, sh);
+      r.nrounds = (int)rr.size();
+      rounds.insert(rounds.end(), rr.begin(), rr.end());
+      if (rs->classes.empty() || rs->classes.back().shape.L != L) {
+        rs->classes.push_back({});
+        rs->classes.back().shape = sh;
+      }
+      ResidentSet::Class& cl = rs->classes.back();
+      cl.ngates = std::max(cl.ngates, r.ngates);
+    }
+    if (rs->classes.back().count++ == 0) rs->classes.back().first = (int)k;
+  }
+  for (const auto& cl : rs->classes)
+    BCUDA(cl.shape.L ? fsv::resident_prepare(false, cl.shape, cl.ngates, nullptr) : fsv::short_prepare(),
+          "resident attributes");
   rs->count = (int)chains.size();
-  if (cudaMalloc(&rs->d_res, sizeof(fsv::ResidentChain) * hd.size()) != cudaSuccess ||
+  rs->place.resize(chains.size());
+  for (size_t k = 0; k < chains.size(); ++k) rs->place[order[k]] = (int)k;
+  const size_t round_b = sizeof(fsv::ResidentRound) * rounds.size(), bond_b = sizeof(int) * bonds.size();
+  if (cudaMalloc(&rs->d_res, sizeof(fsv::ChainArgs) * hd.size()) != cudaSuccess ||
       cudaMalloc(&rs->d_gates, sizeof(float2) * gates.size()) != cudaSuccess ||
-      cudaMalloc(&rs->d_bonds, sizeof(int) * bonds.size()) != cudaSuccess ||
+      cudaMalloc(&rs->d_rounds, round_b + bond_b + 16) != cudaSuccess ||
       cudaMalloc(&rs->d_ring, sizeof(double) * 2 * ring * hd.size()) != cudaSuccess ||
-      cudaMalloc(&rs->d_count, sizeof(long long)) != cudaSuccess) {
+      cudaMalloc(&rs->d_count, 2 * sizeof(long long)) != cudaSuccess) {
     cudaGetLastError();
     rs->release();
     return bfail(b, SV_ENOMEM, "resident tables");
   }
+  int* d_bonds = reinterpret_cast<int*>(reinterpret_cast<char*>(rs->d_rounds) + round_b);
   for (size_t k = 0; k < chains.size(); ++k) {
-    fsv::ResidentChain& r = hd[k];
-    r.psi = reinterpret_cast<float2*>(b->base + b->off[chains[k]]);
-    r.gates = rs->d_gates + fsv::kGateEntries * goff[k];
-    r.bonds = rs->d_bonds + goff[k];
-    r.ring = rs->d_ring + 2 * (size_t)ring * k;
+    fsv::ChainArgs& r = hd[k];
+    r.psi = reinterpret_cast<float2*>(b->base + b->off[chains[order[k]]]);
+    r.gates = rs->d_gates + goff[k];
+    r.rounds = rs->d_rounds + roff[k];
+    r.bonds = d_bonds + boff[k];
+    r.ring = rs->d_ring + 2 * k;
+    r.ring_stride = (long long)chains.size();
   }
-  BCUDA(cudaMemcpyAsync(rs->d_res, hd.data(), sizeof(fsv::ResidentChain) * hd.size(),
+  BCUDA(cudaMemcpyAsync(rs->d_res, hd.data(), sizeof(fsv::ChainArgs) * hd.size(),
                         cudaMemcpyHostToDevice, b->stream),
         "upload resident descriptors");
   BCUDA(cudaMemcpyAsync(rs->d_gates, gates.data(), sizeof(float2) * gates.size(),
                         cudaMemcpyHostToDevice, b->stream),
         "upload resident gates");
-  BCUDA(cudaMemcpyAsync(rs->d_bonds, bonds.data(), sizeof(int) * bonds.size(),
-                        cudaMemcpyHostToDevice, b->stream),
-        "upload resident bonds");
-  BCUDA(cudaMemsetAsync(rs->d_count, 0, sizeof(long long), b->stream), "reset counter");
-  BCUDA(fsv::resident_prepare(rs->max_L), "resident attributes");
+  if (round_b)
+    BCUDA(cudaMemcpyAsync(rs->d_rounds, rounds.data(), round_b, cudaMemcpyHostToDevice, b->stream),
+          "upload resident rounds");
+  if (bond_b)
+    BCUDA(cudaMemcpyAsync(d_bonds, bonds.data(), bond_b, cudaMemcpyHostToDevice, b->stream),
+          "upload resident bonds");
+  BCUDA(cudaMemsetAsync(rs->d_count, 0, 2 * sizeof(long long), b->stream), "reset counter");
   BCUDA(cudaStreamSynchronize(b->stream), "synchronize");
   return SV_OK;
 }
@@ -247,7 +301,7 @@ void free_groups(std::vector<fsv::BlockGroup*>* groups) {
 }
 
 // One graph advancing `periods` periods of the given graph-form chains and
-// of the resident set (if any).  Tensor-core chains run in groups, built on
+// of the resident set (if any); 0 (a resident set alone): d_count[1] periods.  Tensor-core chains run in groups, built on
 // the first call (groups empty) and reused by later ones; the caller frees
 // them after the graphs.
 int make_graph(sv_batch* b, const std::vector<int>& chains, const ResidentSet* rs, int periods,
@@ -260,23 +314,39 @@ int make_graph(sv_batch* b, const std::vector<int>& chains, const ResidentSet* r
     return rc;
   };
   if (rs && rs->count > 0) {
-    cudaGraph_t rg = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeRelaxed);
-    if (e == cudaSuccess) {
-      cudaError_t le = fsv::launch_chain_resident(rs->d_res, rs->count, rs->max_L, rs->d_count,
-                                                  periods, fsv::ctx_ring_len(), b->cap_stream);
-      e = cudaStreamEndCapture(b->cap_stream, &rg);
-      if (le != cudaSuccess) e = le;
+    // each length's launch is a branch of its own; the counter advances after
+    // all of them
+    std::vector<cudaGraphNode_t> runs;
+    const int ring = fsv::ctx_ring_len();
+    for (size_t k = 0; k <= rs->classes.size(); ++k) {
+      cudaGraph_t rg = nullptr;
+      cudaError_t e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeRelaxed);
+      if (e == cudaSuccess) {
+        cudaError_t le;
+        if (k == rs->classes.size()) {
+          le = fsv::launch_advance(rs->d_count, periods, b->cap_stream);
+        } else {
+          const ResidentSet::Class& c = rs->classes[k];
+          le = c.shape.L ? fsv::launch_resident_batch(rs->d_res + c.first, c.count, c.shape,
+                                                      c.ngates, rs->d_count, periods, ring, b->cap_stream)
+                         : fsv::launch_chain_short(rs->d_res + c.first, c.count, rs->d_count, periods,
+                                                  ring, b->cap_stream);
+        }
+        e = cudaStreamEndCapture(b->cap_stream, &rg);
+        if (le != cudaSuccess) e = le;
+      }
+      if (e != cudaSuccess) {
+        if (rg) cudaGraphDestroy(rg);
+        return fail_g(bfail(b, SV_ECUDA, "resident capture: %s", cudaGetErrorString(e)));
+      }
+      cudaGraphNode_t node;
+      const bool last = k == rs->classes.size();
+      e = cudaGraphAddChildGraphNode(&node, g, last ? runs.data() : nullptr, last ? runs.size() : 0, rg);
+      cudaGraphDestroy(rg);
+      if (e != cudaSuccess)
+        return fail_g(bfail(b, SV_ECUDA, "resident node: %s", cudaGetErrorString(e)));
+      runs.push_back(node);
     }
-    if (e != cudaSuccess) {
-      if (rg) cudaGraphDestroy(rg);
-      return fail_g(bfail(b, SV_ECUDA, "resident capture: %s", cudaGetErrorString(e)));
-    }
-    cudaGraphNode_t node;
-    e = cudaGraphAddChildGraphNode(&node, g, nullptr, 0, rg);
-    cudaGraphDestroy(rg);
-    if (e != cudaSuccess)
-      return fail_g(bfail(b, SV_ECUDA, "resident node: %s", cudaGetErrorString(e)));
   }
   std::vector<int> rest;
   if (groups->empty()) {
@@ -400,8 +470,13 @@ int autotune(sv_batch* b) {
   for (int c = 0; c < b->n; ++c) byL[b->L[c]].push_back(c);
   for (auto& kv : byL) {
     const int L = kv.first;
-    std::vector<int> sample(kv.second.begin(),
-                            kv.second.begin() + std::min<size_t>(8, kv.second.size()));
+    auto first = [&](size_t n) {
+      return std::vector<int>(kv.second.begin(), kv.second.begin() + std::min(n, kv.second.size()));
+    };
+    const std::vector<int> sample = first(8);
+    // enough chains that their tiles fill the device (2^21 amplitudes): a group
+    // of eight at L = 15 leaves half of the SMs without a tile
+    const std::vector<int> group = first(std::max<size_t>(8, L < 21 ? (size_t)1 << (21 - L) : 1));
     int best = SV_BATCH_PLAIN, best_n = 0;
     double best_rate = -1.0;
     for (int f : {SV_BATCH_RESIDENT, SV_BATCH_BLOCK_TC, SV_BATCH_BLOCK_SIMT, SV_BATCH_PLAIN,
@@ -411,12 +486,13 @@ int autotune(sv_batch* b) {
         // widths for the CUDA-core form
         if (f != SV_BATCH_BLOCK_SIMT && n != kDefaultWidth) continue;
         if (f == SV_BATCH_BLOCK_SIMT && n > L) continue;
-        // a resident chain uses one CTA, so its form scales with the chain
-        // count up to the SM count: it is timed on every chain of this L;
-        // the other forms fill the device with one chain's passes (the
-        // tensor-core form as one group of the sample)
+        // a resident chain uses one CTA or a few, so its form scales with the
+        // chain count up to the SM count: it is timed on every chain of this L;
+        // the tensor-core form as one group; the other forms fill the device with
+        // one chain's passes
         double rate = 0.0;
-        int rc = time_form(b, f == SV_BATCH_RESIDENT ? kv.second : sample, f, n, &rate);
+        int rc = time_form(b, f == SV_BATCH_RESIDENT ? kv.second : f == SV_BATCH_BLOCK_TC ? group : sample,
+                           f, n, &rate);
         if (rc) return rc;
         if (rate > best_rate) {
           best_rate = rate;
@@ -444,37 +520,16 @@ int setup(sv_batch* b) {
       if (rc) return rc;
     }
   }
-  ResidentSet rs;
-  int rc = build_resident(b, b->res, &rs);
-  if (rc) return rc;
-  b->d_res = rs.d_res;
-  b->d_rgates = rs.d_gates;
-  b->d_rbonds = rs.d_bonds;
-  b->d_rring = rs.d_ring;
-  b->d_rcount = rs.d_count;
-  b->res_maxL = rs.max_L;
-  return SV_OK;
-}
-
-ResidentSet resident_view(const sv_batch* b) {
-  ResidentSet rs;
-  rs.d_res = b->d_res;
-  rs.d_gates = b->d_rgates;
-  rs.d_bonds = b->d_rbonds;
-  rs.d_ring = b->d_rring;
-  rs.d_count = b->d_rcount;
-  rs.max_L = b->res_maxL;
-  rs.count = (int)b->res.size();
-  return rs;
+  return build_resident(b, b->res, &b->rset);
 }
 
 void destroy(sv_batch* b) {
   if (!b) return;
   if (b->g1) cudaGraphExecDestroy(b->g1);
   if (b->gm) cudaGraphExecDestroy(b->gm);
+  if (b->gr) cudaGraphExecDestroy(b->gr);
   free_groups(&b->groups);
-  ResidentSet rs = resident_view(b);
-  rs.release();
+  b->rset.release();
   for (sv_ctx* c : b->ctx)
     if (c) sv_destroy(c);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
@@ -580,13 +635,17 @@ int sv_batch_evolve(sv_batch* b, int64_t periods, double* energy_out, double* no
   std::vector<int> graph_chains;
   for (int c = 0; c < b->n; ++c)
     if (b->form[c] != SV_BATCH_RESIDENT) graph_chains.push_back(c);
-  ResidentSet rs = resident_view(b);
-  if (!b->g1) {
-    int rc = make_graph(b, graph_chains, &rs, 1, &b->g1, &b->groups);
+  const bool all_resident = graph_chains.empty();
+  if (!b->g1 && !all_resident) {
+    int rc = make_graph(b, graph_chains, &b->rset, 1, &b->g1, &b->groups);
     if (rc) return rc;
   }
-  if (!b->gm && periods >= b->M) {
-    int rc = make_graph(b, graph_chains, &rs, b->M, &b->gm, &b->groups);
+  if (!b->gm && !all_resident && periods >= b->M) {
+    int rc = make_graph(b, graph_chains, &b->rset, b->M, &b->gm, &b->groups);
+    if (rc) return rc;
+  }
+  if (!b->gr && all_resident && periods > 0) {
+    int rc = make_graph(b, graph_chains, &b->rset, 0, &b->gr, &b->groups);
     if (rc) return rc;
   }
   const int ring = fsv::ctx_ring_len();
@@ -595,6 +654,18 @@ int sv_batch_evolve(sv_batch* b, int64_t periods, double* energy_out, double* no
   while (done < periods) {
     const int64_t chunk = std::min<int64_t>(periods - done, ring);
     int64_t k = 0;
+    while (all_resident && k < chunk) {
+      // a run of any length is one launch per chain length
+      const int64_t n = std::min<int64_t>(chunk - k, 128);
+      if (b->run != n) {
+        b->run = n;
+        BCUDA(cudaMemcpyAsync(b->rset.d_count + 1, &b->run, sizeof(b->run), cudaMemcpyHostToDevice,
+                              b->stream),
+              "run length");
+      }
+      BCUDA(cudaGraphLaunch(b->gr, b->stream), "graph launch");
+      k += n;
+    }
     for (; b->gm && k + b->M <= chunk; k += b->M)
       BCUDA(cudaGraphLaunch(b->gm, b->stream), "graph launch");
     for (; k < chunk; ++k) BCUDA(cudaGraphLaunch(b->g1, b->stream), "graph launch");
@@ -608,16 +679,22 @@ int sv_batch_evolve(sv_batch* b, int64_t periods, double* energy_out, double* no
       fsv::ctx_advance(b->ctx[c], chunk);
     }
     if (!b->res.empty() && (energy_out || norm_out)) {
-      rbuf.resize(2 * (size_t)ring * b->res.size());
-      BCUDA(cudaMemcpyAsync(rbuf.data(), b->d_rring, sizeof(double) * rbuf.size(),
+      // the slots written, every chain's pair of a slot together
+      const size_t row = 2 * b->res.size(), at = (size_t)(b->counter % ring);
+      const size_t head = std::min<size_t>(chunk, ring - at);
+      rbuf.resize(row * chunk);
+      BCUDA(cudaMemcpyAsync(rbuf.data(), b->rset.d_ring + row * at, sizeof(double) * row * head,
                             cudaMemcpyDeviceToHost, b->stream),
             "resident ring readback");
+      if (head < (size_t)chunk)
+        BCUDA(cudaMemcpyAsync(rbuf.data() + row * head, b->rset.d_ring,
+                              sizeof(double) * row * (chunk - head), cudaMemcpyDeviceToHost, b->stream),
+              "resident ring readback");
       BCUDA(cudaStreamSynchronize(b->stream), "synchronize");
       for (size_t r = 0; r < b->res.size(); ++r) {
         const int c = b->res[r];
-        for (int64_t q = 0; q < chunk; ++q) {
-          const int64_t slot = (b->counter + q) % ring;
-          const double* src = rbuf.data() + 2 * ((size_t)ring * r + slot);
+        const double* src = rbuf.data() + 2 * b->rset.place[r];
+        for (int64_t q = 0; q < chunk; ++q, src += row) {
           if (energy_out) energy_out[(size_t)c * periods + done + q] = src[0];
           if (norm_out) norm_out[(size_t)c * periods + done + q] = src[1];
         }

@@ -125,5 +125,193 @@ __device__ __forceinline__ void store_tile(const TileArgs& ta, const TileIo& io,
   }
 }
 
+__device__ __forceinline__ double period_scale(const Renorm& rn, long long c) {
+  if (!rn.ring || rn.every <= 0) return 1.0;
+  if (c <= 0 || c % rn.every != 0) return 1.0;
+  const double n2 = *reinterpret_cast<const volatile double*>(rn.ring + 2 * ((c - 1) % rn.ring_len) + 1);
+  return n2 > 0.0 ? 1.0 / sqrt(n2) : 1.0;
+}
+
+// Energy terms of one group of four amplitudes w[r] (r = 2 b_i + b_{i+1}), as
+// the per-gate kernels form them: fixed products first, then one chain of
+// sums per grouping.
+template <typename R>
+struct GroupTerms {
+  R hi, lo, p[4], d[4];
+};
+template <typename R>
+__device__ __forceinline__ void group_terms(const typename CT<R>::C (&w)[4], int epi,
+                                            const Diag<R>& dg, uint64_t x,
+                                            const uint64_t (&off)[4], GroupTerms<R>& t) {
+  if (epi & EPI_X_HI) t.hi = cdotre(w[0], w[2]) + cdotre(w[1], w[3]);
+  if (epi & EPI_X_LO) t.lo = cdotre(w[0], w[1]) + cdotre(w[2], w[3]);
+  if (epi & EPI_DIAG) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      t.p[r] = cabs2(w[r]);
+      t.d[r] = dg(x + off[r]);
+    }
+  }
+}
+// es + c t in one rounding (complex64: as the per-gate kernels add it)
+template <typename R>
+__device__ __forceinline__ R add_term(R es, R c, R t) {
+  return es + c * t;
+}
+template <>
+__device__ __forceinline__ float add_term<float>(float es, float c, float t) {
+  return __fmaf_rn(c, t, es);
+}
+template <typename R>
+__device__ __forceinline__ void group_chain(const GroupTerms<R>& t, int epi, R cxh, R cxl, R& es,
+                                            R& ns) {
+  if (epi & EPI_X_HI) es = add_term<R>(es, cxh * (R)2, t.hi);
+  if (epi & EPI_X_LO) es = add_term<R>(es, cxl * (R)2, t.lo);
+  if (epi & EPI_DIAG) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      ns += t.p[r];
+      es += t.p[r] * t.d[r];
+    }
+  }
+}
+
+// The gate on register bits (J0: site b, J1: site b + 1) of a thread's 16
+// amplitudes; K0, K1 are the other two register bits.  get(e): entry e of the
+// table (16, then 16 of its residual).  Residual products first (see
+// k_plain.cu).  Packed FMAs on (re, im) pairs, each half the scalar chain: with
+// the entries in the constant bank they run at the FP32 pipe's full rate (37.7
+// TFMA/s in registers; scalar FMAs with the same operands 35.0, with entries
+// loaded from shared memory 33) and leave half the issue slots to the loads,
+// stores and addresses.  Each entry serves the four groups in turn.
+template <int J0, int J1, int K0, int K1, bool kXor, typename G>
+__device__ __forceinline__ void gate16(uint64_t (&v)[16], const G& get) {
+  auto idx = [](int r, int k) {
+    return ((r >> 1) << J0) | ((r & 1) << J1) | ((k & 1) << K0) | ((k >> 1) << K1);
+  };
+  uint64_t s[16], w[4][4];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const float2 t = un2(v[m]);
+    s[m] = pk2(t.y, t.x);
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[r][k] = 0;
+#pragma unroll
+    for (int part = 1; part >= 0; --part) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = kXor ? r ^ j : j;
+        const ulonglong2 g = get(16 * part + 4 * r + c);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[r][k] = fma2(g.x, v[idx(c, k)], w[r][k]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[r][k] = fma2(g.y, s[idx(c, k)], w[r][k]);
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[idx(r, k)] = w[r][k];
+}
+
+template <int J0, int J1, int K0, int K1, typename Round>
+__device__ __forceinline__ void measure16(const uint64_t (&v)[16], int L, const float* cx,
+                                          const EpiParams& ep, const Round& rd, int which,
+                                          uint64_t x0, bool active, FloatSum& esum,
+                                          FloatSum& nsum) {
+  const int epi = rd.epi[which], bond = rd.bond[which];
+  const float cxh = cx[bond], cxl = cx[bond + 1];
+  Diag<float> dg;
+  if (epi & EPI_DIAG) dg.init(ep, L);
+  const uint64_t ro[4] = {1ull << rd.sbit[0], 1ull << rd.sbit[1], 1ull << rd.sbit[2],
+                          1ull << rd.sbit[3]};
+  const uint64_t off[4] = {0, ro[J1], ro[J0], ro[J0] + ro[J1]};
+  const bool odd = threadIdx.x & 1;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float2 w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      w[r] = un2(v[((r >> 1) << J0) | ((r & 1) << J1) | ((k & 1) << K0) | ((k >> 1) << K1)]);
+    const uint64_t x = x0 + ((k & 1) ? ro[K0] : 0) + ((k >> 1) ? ro[K1] : 0);
+    GroupTerms<float> t;
+    group_terms<float>(w, epi, dg, x, off, t);
+    float es = 0.f, ns = 0.f;
+    group_chain<float>(t, epi, cxh, cxl, es, ns);
+    bool take = active;
+    if (rd.egroup[which] == TILE_E_PAIR) {
+      // the neighbour's sum (bit 0 clear) continues in the lane with bit 0 set
+      float e2 = __shfl_xor_sync(0xffffffffu, es, 1), n2 = 0.f;
+      if (epi & EPI_DIAG) n2 = __shfl_xor_sync(0xffffffffu, ns, 1);
+      group_chain<float>(t, epi, cxh, cxl, e2, n2);
+      es = e2;
+      ns = n2;
+      take = active && odd;
+    }
+    if (take) {
+      esum.add(es);
+      if (epi & EPI_DIAG) nsum.add(ns);
+    }
+  }
+}
+
+// A measured gate on bonds 0..5 of a chain of at least 8 sites, from the tile:
+// the sums of the per-gate kernel, whose threads hold bits 0, 6 and 7.
+// state(e): state index of tile index e; 2^tb amplitudes in the tile.
+template <typename S>
+__device__ __forceinline__ void measure_sweep(const uint8_t* tile, int tb, int L, const float* cx,
+                                              const EpiParams& ep, int bond, int epi, const S& state,
+                                              FloatSum& esum, FloatSum& nsum) {
+  const float cxh = cx[bond], cxl = cx[bond + 1];
+  Diag<float> dg;
+  if (epi & EPI_DIAG) dg.init(ep, L);
+  const uint32_t nv = 1u << (tb - 3);
+  auto at = [&](uint32_t e) { return *reinterpret_cast<const float2*>(tile + tile_byte8(e)); };
+  for (uint32_t vt = threadIdx.x; vt < nv; vt += blockDim.x) {
+    const uint32_t e0 = ((vt & 31u) << 1) | ((vt >> 5) << 8);
+    float2 w[4][2];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) w[c][k] = at(e0 | (c << 6) | k);
+    float es = 0.f, ns = 0.f;
+    if (epi & EPI_X_HI) {
+      float s = 0.f;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+          s += cdotre(w[c][k], at((e0 | (c << 6) | k) ^ (1u << bond)));
+      es += cxh * s;
+    }
+    if (epi & EPI_X_LO) {
+      float s = 0.f;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+          s += cdotre(w[c][k], at((e0 | (c << 6) | k) ^ (2u << bond)));
+      es += cxl * s;
+    }
+    if (epi & EPI_DIAG) {
+      const uint64_t x0 = state(e0);
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float pr = cabs2(w[c][k]);
+          ns += pr;
+          es += pr * dg(x0 + ((uint64_t)c << 6) + k);
+        }
+    }
+    esum.add(es);
+    if (epi & EPI_DIAG) nsum.add(ns);
+  }
+}
+
 }  // namespace dev
 }  // namespace fsv

@@ -12,8 +12,9 @@
 
 namespace fsv {
 
-constexpr int kTileMaxBits = 13;   // largest tile: 2^13 complex64 amplitudes (64 KiB)
-constexpr int kTileMaxGates = 56;  // gates and rounds a pass holds (its parameters stay below 32 KiB)
+constexpr int kTileMaxBits = 12;   // largest tile: 2^12 complex64 amplitudes (32 KiB)
+constexpr int kTileTabSlots = 8;   // gates and rounds of a complex64 pass
+constexpr int kTileMaxGates = 96;  // gates of a pass of the wider types
 constexpr int kTileRuns = 4;  // runs of consecutive state bits inside, and outside, a tile
 
 // How a round's measured gate sums its energy terms (the FP32 grouping of
@@ -28,7 +29,7 @@ enum : int {
 // the amplitudes that a thread holds.  The thread's tile index is its number
 // with a zero inserted at each register bit, lowest first.
 struct __align__(16) TileRound {
-  int8_t gate[2];     // slots of the gates in the pass's table (-1: none)
+  uint8_t gate[2];    // slots of the gates in the pass's table
   uint8_t bond[2];
   uint8_t epi[2];     // EPI_* of each gate
   uint8_t egroup[2];  // TILE_E_* of each measured gate
@@ -37,7 +38,8 @@ struct __align__(16) TileRound {
                       // b and b + 1 of the first gate, then of the second
   uint8_t sbit[4];    // their state bits
   uint8_t xorder[2];  // each gate's products in the order r ^ j (see tile_plan)
-  uint8_t pad[2];
+  uint8_t count;      // gates of the round
+  uint8_t pad;
 };
 static_assert(sizeof(TileRound) == 32, "two 16-byte loads a round");
 
@@ -61,7 +63,9 @@ struct TilePassPlan {
 // The passes of a period in tiles of 2^tb amplitudes (tb >= 4, tb <= L).
 // Gates are taken in the order given; a pass ends where the next gate's
 // sites no longer fit beside the pass's.  pairs: two gates a round.
-std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int precision, int tb);
+// max_gates: gates of a pass (0: the type's).
+std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int precision, int tb,
+                                    int max_gates = 0);
 // Tile size for a chain (a model of launches, waves and arithmetic; 0: the
 // chain is too short for tiles).
 int tile_bits(int L, const std::vector<Gate2>& gates, int precision, int num_sms);
@@ -76,11 +80,11 @@ struct __align__(16) PackedEntry {
 // constant bank, a table entry is a uniform FMA operand that costs no load and
 // no register.
 template <int kSlots>
-struct TileTab {
+struct TileTabOf {
   PackedEntry g[kSlots][kGateEntries];
   TileRound r[kSlots];
 };
-constexpr int kTileTabSmall = 8;  // passes of up to 8 rounds and gates
+using TileTab = TileTabOf<kTileTabSlots>;
 
 struct TileArgs {
   int L = 0, tb = 0;
@@ -100,7 +104,8 @@ struct TileArgs {
   int any_xorder = 0, any_epi = 0;    // over the pass's gates
   long long stride = 0;               // per-period table stride (entries; 0: one table)
   const long long* counter = nullptr;
-  double cx[34] = {};                 // <X> coefficients (measured gates)
+  float cx[34] = {};                  // complex64: <X> coefficients (measured gates)
+  double cx64[34] = {};               // the wider types'
   EpiParams ep;                       // diagonal coefficients, renormalisation, partials
   // a whole period in one pass on one tile: `periods` periods in one launch,
   // each period's energy and norm written to the ring, the counter advanced
@@ -115,7 +120,7 @@ struct TileArgs {
 cudaError_t tile_grid(int precision, TileArgs* ta, const LaunchCfg& cfg, int* grid);
 // tab: the pass's tables and rounds on the host (in_params; else unused)
 cudaError_t launch_tile(int precision, void* psi, const TileArgs& ta,
-                        const TileTab<kTileMaxGates>* tab, int grid, cudaStream_t s);
+                        const TileTab* tab, int grid, cudaStream_t s);
 
 // ------------------------------------------------------------ adjoint sweep
 // A pass of the reverse sweep on tiles of psi and lambda (complex64): operations
@@ -129,8 +134,7 @@ struct AdjointPass {
 cudaError_t adjoint_tile_grid(AdjointPass* ap, const LaunchCfg& cfg, int* grid);
 // tab: odag (16 entries) and d (16) per operation, and the rounds
 cudaError_t launch_adjoint_tile(void* psi, void* lam, const AdjointPass& ap,
-                                const TileTab<kTileMaxGates>& tab, double* part, int grid,
-                                cudaStream_t s);
+                                const TileTab& tab, double* part, int grid, cudaStream_t s);
 // out[2 k], out[2 k + 1] = 2 x the sums of period k's (kick, field) partial
 // pairs, periods `pairs` pairs apart, fixed order
 cudaError_t launch_grad_reduce_pairs(const double* part, int pairs, int periods, double* out,
