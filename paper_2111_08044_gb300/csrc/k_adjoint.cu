@@ -229,6 +229,8 @@ __global__ void __launch_bounds__(128, 4)
   const TileIo io = tile_io(ta);
   const uint64_t xout = elem_state(ta, thread_elem<4>(tab.r[ta.nrounds - 1], tid));
   double acc[2] = {0.0, 0.0};
+  grid_wait();
+  grid_trigger();
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint64_t tbase = tile_base(ta, t);
     load_tile(ta, io, sbuf, psi + tbase);
@@ -395,23 +397,23 @@ cudaError_t adjoint_tile_grid(AdjointPass* ap, const LaunchCfg& cfg, int* grid) 
   const TileArgs& ta = ap->ta;
   const int smem = 2 * (int)tile_byte8(1u << ta.tb);
   int per_sm = 1;
-  cudaError_t e = cudaFuncSetAttribute(k_adjoint_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       2 * (int)tile_byte8(1u << kAdjointTileBits));
+  cudaError_t e =
+      cudaFuncSetAttribute(k_adjoint_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kEvenSmemMax);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adjoint_tile,
                                                       tile_threads(SV_C64, ta.tb), smem);
   const uint64_t most = (uint64_t)cfg.num_sms * (per_sm > 0 ? per_sm : 1);
   const uint64_t tiles = 1ull << (ta.L - ta.tb);
   *grid = (int)(tiles < most ? tiles : most);
+  ap->ta.smem = (uint32_t)even_smem(*grid, cfg.num_sms, smem);
   return e;
 }
 
 cudaError_t launch_adjoint_tile(void* psi, void* lam, const AdjointPass& ap, const TileTab& tab,
                                 double* part, int grid, cudaStream_t s) {
-  const int tb = ap.ta.tb;
-  k_adjoint_tile<<<grid, tile_threads(SV_C64, tb), 2 * tile_byte8(1u << tb), s>>>(
-      static_cast<float2*>(psi), static_cast<float2*>(lam), ap, part, tab);
-  return cudaGetLastError();
+  void* args[] = {&psi, &lam, const_cast<AdjointPass*>(&ap), &part, const_cast<TileTab*>(&tab)};
+  return launch_overlapped(reinterpret_cast<const void*>(k_adjoint_tile), grid,
+                           tile_threads(SV_C64, ap.ta.tb), ap.ta.smem, s, args);
 }
 
 cudaError_t launch_grad_reduce_pairs(const double* part, int pairs, int periods, double* out,

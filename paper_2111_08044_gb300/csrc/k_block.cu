@@ -464,7 +464,7 @@ cudaError_t ensure_maps(BlockPlan* bp, void* psi) {
 cudaError_t launch_pass(BlockPlan* bp, size_t k, void* psi, cudaStream_t s) {
   if (bp->tensor_cores)
     return launch_block_tc(bp->args[k], psi, bp->maps.data() + k * block_tc_map_bytes(),
-                           bp->d_status, bp->grid, s);
+                           bp->d_status, bp->grid, s, bp->cfg.alone());
   return launch_block_simt(bp->args[k], psi, bp->grid, s);
 }
 

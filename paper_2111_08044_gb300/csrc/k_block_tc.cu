@@ -639,6 +639,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       epilogue_sync();
     }
+    grid_wait();
     const float sc = (float)renorm_scale(pa.ep.rn);
     const uint64_t sc2 = f2(sc, sc);
     // per-thread energy and norm over its tiles: compensated FP32 sums
@@ -950,6 +951,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       } else {
         load_w(pa.W);
       }
+      grid_wait();  // (the operands are the plan's: no kernel writes them)
+      grid_trigger();
       int wload = 0;  // group: operand blocks loaded after the first
       const long long nloads = 4 * my_tiles;
       long long issued = 0;
@@ -1345,25 +1348,22 @@ cudaError_t block_tc_prepare() {
 }
 
 cudaError_t launch_block_tc(const PassArgs& pa, void* psi, const void* map, int* status,
-                            int grid, cudaStream_t s) {
+                            int grid, cudaStream_t s, bool overlap) {
   PassArgs p = pa;
   p.psi = psi;
   alignas(64) CUtensorMap maps[2];
   std::memcpy(maps, map, sizeof(maps));
   constexpr long long kMinTilesSpecialised = 32;  // tiles per CTA
   const long long per_cta = (p.ntiles + grid - 1) / grid;
-  const dim3 g(grid), b(kThreads);
-  if (per_cta < kMinTilesSpecialised)
-    k_block_tc<true, false, false><<<g, b, kSmemBytes, s>>>(maps[0], maps[1], p, status, nullptr, 0);
-  else if (p.diag && p.x_mask)
-    k_block_tc<false, true, true><<<g, b, kSmemBytes, s>>>(maps[0], maps[1], p, status, nullptr, 0);
-  else if (p.diag)
-    k_block_tc<false, false, true><<<g, b, kSmemBytes, s>>>(maps[0], maps[1], p, status, nullptr, 0);
-  else if (p.x_mask)
-    k_block_tc<false, true, false><<<g, b, kSmemBytes, s>>>(maps[0], maps[1], p, status, nullptr, 0);
-  else
-    k_block_tc<false, false, false><<<g, b, kSmemBytes, s>>>(maps[0], maps[1], p, status, nullptr, 0);
-  return cudaGetLastError();
+  const void* k = (const void*)k_block_tc<false, false, false>;
+  if (per_cta < kMinTilesSpecialised) k = (const void*)k_block_tc<true, false, false>;
+  else if (p.diag && p.x_mask) k = (const void*)k_block_tc<false, true, true>;
+  else if (p.diag) k = (const void*)k_block_tc<false, false, true>;
+  else if (p.x_mask) k = (const void*)k_block_tc<false, true, false>;
+  const GroupChain* group = nullptr;
+  int nt_log2 = 0;
+  void* args[] = {&maps[0], &maps[1], &p, &status, &group, &nt_log2};
+  return launch_overlapped(k, grid, kThreads, kSmemBytes, s, args, overlap);
 }
 
 cudaError_t launch_block_tc_group(const PassArgs& pa, const GroupChain* chains, int nt_log2,

@@ -357,11 +357,13 @@ __global__ void __launch_bounds__(kThreads) k_gate_small(
 }
 
 // ------------------------------------------------------------- period reduce
-__device__ void period_reduce_block(const double* __restrict__ partials, long long n, int L,
+__device__ void period_reduce_block(const double* partials, long long n, int L,
                                     double* __restrict__ ring, int ring_len, long long* counter,
                                     int advance) {
   __shared__ double se[256], sn[256];
   double e = 0.0, nn = 0.0;
+  grid_wait();
+  grid_trigger();
   for (long long k = threadIdx.x; k < n; k += blockDim.x) {
     e += partials[2 * k];
     nn += partials[2 * k + 1];
@@ -386,7 +388,7 @@ __device__ void period_reduce_block(const double* __restrict__ partials, long lo
   }
 }
 
-__global__ void __launch_bounds__(256) k_period_reduce(const double* __restrict__ partials,
+__global__ void __launch_bounds__(256) k_period_reduce(const double* partials,
                                                        long long n, int L,
                                                        double* __restrict__ ring,
                                                        int ring_len, long long* counter,
@@ -584,8 +586,8 @@ cudaError_t launch_plain_gate(int precision, void* psi, int L, int bond,
 cudaError_t launch_period_reduce(const double* partials, long long n, int L, double* ring,
                                  int ring_len, long long* counter, int advance,
                                  cudaStream_t s) {
-  k_period_reduce<<<1, 256, 0, s>>>(partials, n, L, ring, ring_len, counter, advance);
-  return cudaGetLastError();
+  void* args[] = {&partials, &n, &L, &ring, &ring_len, &counter, &advance};
+  return launch_overlapped(reinterpret_cast<const void*>(k_period_reduce), 1, 256, 0, s, args);
 }
 
 cudaError_t launch_period_reduce_many(const ReduceItem* items, int count, cudaStream_t s) {

@@ -128,6 +128,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
   const TileIo io = tile_io(ta);
   const TileRound& last = kSlots ? tab.r[ta.nrounds - 1] : ta.rounds[ta.nrounds - 1];
   const uint64_t xout = elem_state(ta, thread_elem<4>(last, tid));
+  grid_wait();
+  grid_trigger();
   load_tile(ta, io, sbuf, psi + tile_base(ta, blockIdx.x));
   if (kSlots == 0)
     for (int k = threadIdx.x; k < 2 * ta.nrounds; k += blockDim.x)
@@ -251,6 +253,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
       cp_async16((uint32_t)__cvta_generic_to_shared(to + tile_slot16(e)), from + elem_state(ta, e));
     cp_commit();
   };
+  grid_wait();
+  grid_trigger();
   load(tile, blockIdx.x);
   for (int k = threadIdx.x; k < 2 * ta.nrounds; k += blockDim.x)
     reinterpret_cast<uint4*>(rds)[k] = reinterpret_cast<const uint4*>(ta.rounds)[k];
@@ -387,8 +391,8 @@ cudaError_t tile_grid(int precision, TileArgs* ta, const LaunchCfg& cfg, int* gr
   const uint64_t tiles = 1ull << (ta->L - ta->tb);
   const void* kernel = tile_kernel(precision, *ta);
   // every pass of an instance asks for the same limit (its largest)
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (precision == SV_C64 ? 104 : 64) * 1024);
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEvenSmemMax);
   // complex128 works between two copies; elsewhere a second buffer takes the
   // next tile while this one is computed
   int per_sm = 1;
@@ -400,16 +404,20 @@ cudaError_t tile_grid(int precision, TileArgs* ta, const LaunchCfg& cfg, int* gr
     if (tiles <= (uint64_t)cfg.num_sms * per_sm) break;  // one tile a block: nothing to prefetch
   }
   *grid = (int)std::min<uint64_t>(tiles, (uint64_t)cfg.num_sms * per_sm);
+  ta->overlap = cfg.alone();
+  ta->smem = (uint32_t)tile_smem_bytes(precision, *ta);
+  if (ta->overlap) ta->smem = (uint32_t)even_smem(*grid, cfg.num_sms, ta->smem);
   return e;
 }
 
 cudaError_t launch_tile(int precision, void* psi, const TileArgs& ta, const TileTab* tab, int grid,
                         cudaStream_t s) {
+  if (ta.smem < tile_smem_bytes(precision, ta)) return cudaErrorInvalidValue;
   TileTabOf<1> none;
   void* args[] = {&psi, const_cast<TileArgs*>(&ta), nullptr};
   if (precision == SV_C64) args[2] = ta.in_params ? (void*)const_cast<TileTab*>(tab) : (void*)&none;
-  return cudaLaunchKernel(tile_kernel(precision, ta), dim3(grid), dim3(tile_threads(precision, ta.tb)),
-                          args, tile_smem_bytes(precision, ta), s);
+  return launch_overlapped(tile_kernel(precision, ta), grid, tile_threads(precision, ta.tb), ta.smem, s,
+                           args, ta.overlap);
 }
 
 }  // namespace fsv

@@ -975,8 +975,11 @@ int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab) {
         like = &o.ta;
         t.grid = o.grid;
       }
-    if (like) ta.buffers = like->buffers;
-    else SV_CUDA(fsv::tile_grid(ctx->precision, &ta, ctx->cfg, &t.grid), "tile pass setup");
+    if (like) {
+      ta.buffers = like->buffers;
+      ta.overlap = like->overlap;
+      ta.smem = like->smem;
+    } else SV_CUDA(fsv::tile_grid(ctx->precision, &ta, ctx->cfg, &t.grid), "tile pass setup");
     if (p.measures) {
       ta.ep.partial = ctx->d_part_evolve + 2 * ctx->part_pairs;
       ctx->part_pairs += t.grid;

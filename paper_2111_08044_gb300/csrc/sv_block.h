@@ -163,7 +163,7 @@ int block_status(BlockPlan* bp, cudaStream_t s);
 // CUDA-core FP32 pass (any n, R); tensor-core pass (n = 6, R = 7).
 cudaError_t launch_block_simt(const PassArgs& pa, void* psi, int grid, cudaStream_t s);
 cudaError_t launch_block_tc(const PassArgs& pa, void* psi, const void* map, int* status,
-                            int grid, cudaStream_t s);
+                            int grid, cudaStream_t s, bool overlap);
 // One tensor-core pass over the tiles of a chain group: pa is the pass's
 // structure with ntiles = chains x 2^nt_log2; chains: device array, one per
 // chain.  CTA b takes the contiguous tiles [b T / grid, (b + 1) T / grid).

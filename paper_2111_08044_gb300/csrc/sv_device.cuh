@@ -11,6 +11,16 @@
 
 namespace fsv {
 namespace dev {
+// A kernel launched with launch_overlapped (sv_kernels.h) may start while the one
+// before it in the stream still runs: what earlier kernels write is read, and what
+// they read is written, after grid_wait, which every block reaches (it returns when
+// they have completed; at once after another kind of launch).  grid_trigger, after
+// it: the next such kernel may start where an SM has room.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 
 template <typename R>
 struct CT;

@@ -66,7 +66,39 @@ struct LaunchCfg {
   // at least this many tiles per CTA in block passes (0: one wave over the
   // SMs); batches set it so that several chains' passes share the device
   int min_tiles_per_cta = 0;
+  bool alone() const { return min_tiles_per_cta == 0; }  // no other chain's passes beside
 };
+
+// Launch of a kernel that begins with grid_wait (sv_device.cuh) before it touches
+// what earlier kernels of the stream write.  overlap: it may start while the kernel
+// before it still runs, so that its launch, its setup and (tensor-core passes) its
+// operands are not waited for: a period of seven launches of 8 us at L = 14 takes
+// 57 us, one after the other 63 us.  Not for passes beside other chains' (batches): blocks that
+// wait keep theirs off the SM (12 plain chains of 16..18 sites: 8.3 ms for 7.6).
+inline cudaError_t launch_overlapped(const void* kernel, int grid, int threads, size_t smem,
+                                     cudaStream_t s, void** args, bool overlap = true) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+// Dynamic shared memory for a grid of overlapped blocks: at least `need`, and so much
+// that no SM takes more than its share of the grid.  (Blocks that start early go
+// where there is room, not where it is even: without it a pass of 256 tiles at L = 20
+// took half as long again.)
+inline size_t even_smem(int grid, int num_sms, size_t need) {
+  const size_t per_sm = (grid + num_sms - 1) / num_sms;
+  const size_t least = 228 * 1024 / (per_sm + 1) - 1024 + 1;
+  return need > least ? need : least;
+}
+constexpr int kEvenSmemMax = 116 * 1024;  // its largest padding (one block an SM)
 
 // Grid (blocks of 256 threads) used by the plain gate pass for this L and
 // bond; it is also the number of partial pairs the pass writes.

@@ -92,6 +92,8 @@ struct TileArgs {
   int direct_out = 0;
   int first = 0;                   // the period's first pass (folded renormalisation)
   int buffers = 1;                 // tile buffers (2: the next tile loads during this one)
+  int overlap = 0;                 // launched while the pass before still runs
+  uint32_t smem = 0;               // dynamic shared memory
   // state bits of the tile index, in runs: (e & m) << s
   uint8_t erun_s[kTileRuns] = {};
   uint16_t erun_m[kTileRuns] = {};
@@ -115,7 +117,8 @@ struct TileArgs {
   long long* counter_rw = nullptr;
 };
 
-// grid of a pass (also its number of partial pairs) and its tile buffers; opts
+// grid of a pass (also its number of partial pairs), its tile buffers and shared
+// memory; opts
 // its kernel into the shared memory it needs (at build time, outside a capture)
 cudaError_t tile_grid(int precision, TileArgs* ta, const LaunchCfg& cfg, int* grid);
 // tab: the pass's tables and rounds on the host (in_params; else unused)
