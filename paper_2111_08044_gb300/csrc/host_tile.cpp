@@ -147,11 +147,18 @@ std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int 
 
 int tile_bits(int L, const std::vector<Gate2>& gates, int precision, int num_sms) {
   if (L < 5) return 0;
-  const int cap = precision == SV_C64 ? 12 : precision == SV_DF64 ? 10 : 9;
+  // Double-float: a chain that one tile holds stays in one block (10 sites 67 us a
+  // period, 98 in tiles of 2^9); else tiles of 2^10, eight warps each, where they
+  // leave most SMs one (21 sites 1.40 ms a period, 1.44 in tiles of 2^9, 1.58 of
+  // 2^8), and of 2^9 below (13 sites 119 us; 137 in tiles of 2^10, 123 of 2^8).
+  if (precision == SV_DF64) return std::min(L, L <= 10 || (4ll << (L - 10)) >= 3ll * num_sms ? 10 : 9);
+  // complex128: one block up to 8 sites (42 us a period, 52 in tiles of 2^7; 9 sites
+  // 70 and 61); then FP64 work against launches: 13 sites 100 us in tiles of 2^7, 105
+  // of 2^6, 115 of 2^8; 21 sites 5.03 ms of 2^8, 5.07 of 2^7, 5.21 of 2^9.
+  if (precision == SV_C128) return L <= 8 ? L : L < 15 ? 7 : 8;
   int best = 0;
   double best_t = 0;
   for (int tb = std::min(L, 6); tb <= std::min(L, kTileMaxBits); ++tb) {
-    if (tb > cap) continue;
     const double tiles = (double)(1ull << (L - tb));
     const double per_sm = (double)((int64_t)((tiles + num_sms - 1) / num_sms));
     const double amps = (double)(1ull << tb);
@@ -166,18 +173,8 @@ int tile_bits(int L, const std::vector<Gate2>& gates, int precision, int num_sms
       }
       // arithmetic of the busiest SM, and the latency of one tile's chain
       const double g = end - at;
-      double work, chain;
-      if (precision == SV_C64) {
-        work = per_sm * amps * g * 32 / 128;
-        chain = (g + 1) / 2 * 1400;
-      } else if (precision == SV_DF64) {
-        work = per_sm * amps * g * 200 / 128;
-        chain = g * 1400;
-      } else {
-        work = per_sm * amps * g * 16 / 2;
-        chain = g * 500;
-      }
-      t += std::max(work, chain) + (g == ng && L == tb ? 1500 : 4000);
+      t += std::max(per_sm * amps * g * 32 / 128, (g + 1) / 2 * 1400) +
+           (g == ng && L == tb ? 1500 : 4000);
       at = end;
     }
     if (t < 0) continue;

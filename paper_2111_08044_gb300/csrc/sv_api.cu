@@ -70,7 +70,10 @@ struct sv_ctx {
   struct TileLaunch {
     fsv::TileArgs ta;
     int grid = 0;
-    std::unique_ptr<fsv::TileTab> tab;  // complex64, fixed gates
+    // the pass's tables and rounds where its gates are fixed (double-float: at
+    // most kTileTabSlots of them)
+    std::unique_ptr<fsv::TileTab> tab;
+    std::unique_ptr<fsv::TileTabDf<fsv::kTileTabSlots>> tab_df;
   };
   std::vector<TileLaunch> tiles;
   bool tile_single = false;  // one block (or cluster) holds the chain: runs of whole
@@ -230,7 +233,7 @@ int enqueue_tile_run(sv_ctx* ctx, int64_t periods, cudaStream_t s) {
   }
   fsv::TileArgs ta = ctx->tiles[0].ta;
   ta.periods = (int)periods;
-  SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, ta, nullptr, 1, s), "tile launch");
+  SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, ta, nullptr, nullptr, 1, s), "tile launch");
   return SV_OK;
 }
 
@@ -245,7 +248,8 @@ int enqueue_tile_period(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev) {
   } else {
     for (const auto& t : ctx->tiles) {
       if (ev) SV_CUDA(cudaEventRecord(ev[k++], s), "event record");
-      SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, t.ta, t.tab.get(), t.grid, s), "tile launch");
+      SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, t.ta, t.tab.get(), t.tab_df.get(), t.grid, s),
+              "tile launch");
     }
     if (ev) SV_CUDA(cudaEventRecord(ev[k++], s), "event record");
     SV_CUDA(fsv::launch_period_reduce(ctx->d_part_evolve, ctx->part_pairs, ctx->L, ctx->d_ring,
@@ -909,8 +913,8 @@ int build_resident_chain(sv_ctx* ctx) {
 
 // The tile passes of a plain-mode period (none on chains too short for them):
 // their rounds on the device, the launch arguments, the partial pairs.
-// host_tab: the first period's complex64 tables.
-int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab) {
+// host_tab, host_df: the first period's tables (complex64, double-float).
+int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab, const std::vector<float4>& host_df) {
   const int L = ctx->L, ng = (int)ctx->gates.size();
   if (ctx->precision == SV_C64 && L >= 5 && L <= fsv::kResidentPlainMaxL) {
     int clusters = 0;
@@ -962,6 +966,16 @@ int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab) {
         t.tab->g[0][e] = fsv::PackedEntry{{g.x, g.x}, {-g.y, g.y}};
       }
       std::memcpy(t.tab->r, p.rounds.data(), sizeof(fsv::TileRound) * p.rounds.size());
+    }
+    if (ctx->precision == SV_DF64 && ta.stride == 0 && !ta.ep.rn.ring && !ctx->tile_single &&
+        ta.ngates <= fsv::kTileTabSlots && ta.nrounds <= fsv::kTileTabSlots) {
+      ta.in_params = 1;
+      t.tab_df.reset(new fsv::TileTabDf<fsv::kTileTabSlots>());
+      for (int g = 0; g < ta.ngates; ++g)
+        for (int e = 0; e < 16; ++e)
+          t.tab_df->g[g][e] =
+              fsv::df_entry(host_df[(size_t)(p.gates[0] + g) * fsv::kGateEntries + e]);
+      std::memcpy(t.tab_df->r, p.rounds.data(), sizeof(fsv::TileRound) * p.rounds.size());
     }
     for (const auto& r : p.rounds) {
       ta.any_xorder |= r.xorder[0] | r.xorder[1];
@@ -1476,7 +1490,7 @@ int sv_build_floquet(sv_ctx* ctx, const sv_floquet_params* p) {
     ctx->passes_per_period = ng;
     ctx->launches_per_period = ng + 1;
     ctx->build_bytes = ctx->d_gates_bytes;
-    const int rc = p->mode == SV_MODE_MULTIGATE ? build_multigate(ctx, mplan) : build_tiles(ctx, host_tab);
+    const int rc = p->mode == SV_MODE_MULTIGATE ? build_multigate(ctx, mplan) : build_tiles(ctx, host_tab, tab_df);
     if (rc) return rc;
   }
   ctx->built = true;

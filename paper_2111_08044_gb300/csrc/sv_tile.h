@@ -86,6 +86,29 @@ struct TileTabOf {
 };
 using TileTab = TileTabOf<kTileTabSlots>;
 
+// A double-float table entry as packed operands (df_entry): (re, re) and
+// (-im, im) leading parts, their negatives, the trailing parts negated.
+struct EntryDf {
+  uint64_t re, nre, nre_lo, im, nim, nim_lo;
+};
+// entry (re hi, re lo, im hi, im lo)
+__host__ __device__ inline EntryDf df_entry(float4 g) {
+  auto pair = [](float x, float y) {
+    union {
+      float f[2];
+      uint64_t u;
+    } p = {{x, y}};
+    return p.u;
+  };
+  return EntryDf{pair(g.x, g.x),  pair(-g.x, -g.x), pair(-g.y, -g.y),
+                 pair(-g.z, g.z), pair(g.z, -g.z),  pair(g.w, -g.w)};
+}
+template <int kSlots>
+struct TileTabDf {
+  EntryDf g[kSlots][16];
+  TileRound r[kSlots];
+};
+
 struct TileArgs {
   int L = 0, tb = 0;
   int ngates = 0, nrounds = 0;
@@ -102,7 +125,7 @@ struct TileArgs {
   uint32_t run_m[kTileRuns] = {};
   const TileRound* rounds = nullptr;  // device
   const void* gates = nullptr;        // device: the pass's first gate table
-  int in_params = 0;                  // complex64: tables and rounds in the parameters
+  int in_params = 0;                  // tables and rounds in the parameters
   int any_xorder = 0, any_epi = 0;    // over the pass's gates
   long long stride = 0;               // per-period table stride (entries; 0: one table)
   const long long* counter = nullptr;
@@ -121,9 +144,9 @@ struct TileArgs {
 // memory; opts
 // its kernel into the shared memory it needs (at build time, outside a capture)
 cudaError_t tile_grid(int precision, TileArgs* ta, const LaunchCfg& cfg, int* grid);
-// tab: the pass's tables and rounds on the host (in_params; else unused)
-cudaError_t launch_tile(int precision, void* psi, const TileArgs& ta,
-                        const TileTab* tab, int grid, cudaStream_t s);
+// tab, tab_df: the pass's tables and rounds on the host (in_params; else unused)
+cudaError_t launch_tile(int precision, void* psi, const TileArgs& ta, const TileTab* tab,
+                        const TileTabDf<kTileTabSlots>* tab_df, int grid, cudaStream_t s);
 
 // ------------------------------------------------------------ adjoint sweep
 // A pass of the reverse sweep on tiles of psi and lambda (complex64): operations
