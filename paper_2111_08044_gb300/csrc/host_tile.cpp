@@ -145,7 +145,7 @@ std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int 
   return out;
 }
 
-int tile_bits(int L, const std::vector<Gate2>& gates, int precision, int num_sms) {
+int tile_bits(int L, int precision, int num_sms) {
   if (L < 5) return 0;
   // Double-float: a chain that one tile holds stays in one block (10 sites 67 us a
   // period, 98 in tiles of 2^9); else tiles of 2^10, eight warps each, where they
@@ -156,34 +156,10 @@ int tile_bits(int L, const std::vector<Gate2>& gates, int precision, int num_sms
   // 70 and 61); then FP64 work against launches: 13 sites 100 us in tiles of 2^7, 105
   // of 2^6, 115 of 2^8; 21 sites 5.03 ms of 2^8, 5.07 of 2^7, 5.21 of 2^9.
   if (precision == SV_C128) return L <= 8 ? L : L < 15 ? 7 : 8;
-  int best = 0;
-  double best_t = 0;
-  for (int tb = std::min(L, 6); tb <= std::min(L, kTileMaxBits); ++tb) {
-    const double tiles = (double)(1ull << (L - tb));
-    const double per_sm = (double)((int64_t)((tiles + num_sms - 1) / num_sms));
-    const double amps = (double)(1ull << tb);
-    double t = 0;
-    const int ng = (int)gates.size();
-    for (int at = 0; at < ng;) {
-      uint64_t set = 0;
-      const int end = pass_end(L, gates, precision, tb, at, most_gates(precision), &set);
-      if (end == at) {
-        t = -1;
-        break;
-      }
-      // arithmetic of the busiest SM, and the latency of one tile's chain
-      const double g = end - at;
-      t += std::max(per_sm * amps * g * 32 / 128, (g + 1) / 2 * 1400) +
-           (g == ng && L == tb ? 1500 : 4000);
-      at = end;
-    }
-    if (t < 0) continue;
-    if (best == 0 || t < best_t) {
-      best = tb;
-      best_t = t;
-    }
-  }
-  return best;
+  // complex64 (chains too long for the resident form): tiles of 2^12 where they leave
+  // most SMs one (21 sites 307 us a period, 330 in tiles of 2^11; 24 sites 2.12 and
+  // 2.17 ms), of 2^11 below (16 sites 86 us, 104 in tiles of 2^12, 88 of 2^10).
+  return (4ll << L) >= 3ll * num_sms << 12 ? 12 : 11;
 }
 
 std::vector<ResidentRound> resident_rounds(const std::vector<Gate2>& gates, const ResidentShape& sh) {

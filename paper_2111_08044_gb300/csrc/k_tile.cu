@@ -529,7 +529,10 @@ const void* tile_kernel(int precision, const TileArgs& ta) {
     return ta.in_params   ? reinterpret_cast<const void*>(k_tile_df<kTileTabSlots, 3>)
            : ta.tb < ta.L ? reinterpret_cast<const void*>(k_tile_df<0, 3>)
                           : reinterpret_cast<const void*>(k_tile_df<0, 1>);
-  if (!ta.in_params) return reinterpret_cast<const void*>(k_tile_f32<0, true, true, 256, 2>);
+  if (!ta.in_params)
+    return ta.any_epi      ? reinterpret_cast<const void*>(k_tile_f32<0, true, true, 256, 2>)
+           : ta.any_xorder ? reinterpret_cast<const void*>(k_tile_f32<0, true, false, 256, 2>)
+                           : reinterpret_cast<const void*>(k_tile_f32<0, false, false, 256, 2>);
   if (ta.any_epi) return reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, true, 256, 2>);
   return ta.any_xorder ? reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, false, 256, 3>)
                        : reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, false, false, 256, 3>);

@@ -69,13 +69,16 @@ struct sv_ctx {
   // which take one launch per gate)
   struct TileLaunch {
     fsv::TileArgs ta;
-    int grid = 0;
+    int grid = 0, first_gate = 0;
     // the pass's tables and rounds where its gates are fixed (double-float: at
     // most kTileTabSlots of them)
     std::unique_ptr<fsv::TileTab> tab;
     std::unique_ptr<fsv::TileTabDf<fsv::kTileTabSlots>> tab_df;
   };
   std::vector<TileLaunch> tiles;
+  // complex64 chains with per-period tables, from kDriveMinL sites: the tables of
+  // every period on the host, whose passes are launched with them as parameters
+  std::vector<float2> drive_tab;
   bool tile_single = false;  // one block (or cluster) holds the chain: runs of whole
                              // periods in one launch
   bool resident = false;     // complex64: that launch is the resident form's
@@ -168,6 +171,7 @@ void free_build(sv_ctx* ctx) {
   ctx->d_mg = nullptr;
   ctx->mg.clear();
   ctx->tiles.clear();
+  ctx->drive_tab.clear();
   ctx->tile_single = false;
   ctx->resident = false;
   if (ctx->block) {
@@ -237,6 +241,14 @@ int enqueue_tile_run(sv_ctx* ctx, int64_t periods, cudaStream_t s) {
   return SV_OK;
 }
 
+// Tables of a pass's `n` gates as packed operands.
+void pack_tables(const float2* gates, size_t n, fsv::PackedEntry* out) {
+  for (size_t e = 0; e < n * fsv::kGateEntries; ++e) {
+    const float2 g = gates[e];
+    out[e] = fsv::PackedEntry{{g.x, g.x}, {-g.y, g.y}};
+  }
+}
+
 // One period in tile passes; ev (nullable): one event before each launch and
 // one after the last.
 int enqueue_tile_period(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev) {
@@ -248,6 +260,10 @@ int enqueue_tile_period(sv_ctx* ctx, cudaStream_t s, cudaEvent_t* ev) {
   } else {
     for (const auto& t : ctx->tiles) {
       if (ev) SV_CUDA(cudaEventRecord(ev[k++], s), "event record");
+      if (!ctx->drive_tab.empty() && t.ta.in_params)
+        pack_tables(&ctx->drive_tab[((size_t)ctx->counter * ctx->gates.size() + t.first_gate) *
+                                    fsv::kGateEntries],
+                    t.ta.ngates, t.tab->g[0]);
       SV_CUDA(fsv::launch_tile(ctx->precision, ctx->state, t.ta, t.tab.get(), t.tab_df.get(), t.grid, s),
               "tile launch");
     }
@@ -317,7 +333,7 @@ int capture_period(sv_ctx* ctx, bool last, cudaGraphExec_t* out) {
 }
 
 int ensure_graph(sv_ctx* ctx) {
-  if (ctx->tile_single) return SV_OK;  // launched directly
+  if (ctx->tile_single || !ctx->drive_tab.empty()) return SV_OK;  // launched directly
   if (!ctx->graph) {
     int rc = capture_period(ctx, false, &ctx->graph);
     if (rc) return rc;
@@ -340,6 +356,14 @@ int launch_periods(sv_ctx* ctx, int64_t count, bool last) {
       int rc = enqueue_tile_run(ctx, n, ctx->stream);
       if (rc) return rc;
       ctx->counter += n;
+    }
+    return SV_OK;
+  }
+  if (!ctx->drive_tab.empty()) {
+    for (int64_t k = 0; k < count; ++k) {
+      int rc = enqueue_tile_period(ctx, ctx->stream, nullptr);
+      if (rc) return rc;
+      ++ctx->counter;
     }
     return SV_OK;
   }
@@ -911,10 +935,15 @@ int build_resident_chain(sv_ctx* ctx) {
   return SV_OK;
 }
 
+// Per-period tables are passed as parameters from this length on, where a pass (7 us
+// and more) hides the host's packing and launch of the next (3 us): 24 sites 2.1 ms a
+// period, with the tables copied to shared memory by each block 2.7 ms.
+constexpr int kDriveMinL = 19;
+
 // The tile passes of a plain-mode period (none on chains too short for them):
 // their rounds on the device, the launch arguments, the partial pairs.
-// host_tab, host_df: the first period's tables (complex64, double-float).
-int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab, const std::vector<float4>& host_df) {
+// host_tab, host_df: every period's tables (complex64, double-float).
+int build_tiles(sv_ctx* ctx, std::vector<float2>& host_tab, const std::vector<float4>& host_df) {
   const int L = ctx->L, ng = (int)ctx->gates.size();
   if (ctx->precision == SV_C64 && L >= 5 && L <= fsv::kResidentPlainMaxL) {
     int clusters = 0;
@@ -927,7 +956,7 @@ int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab, const std::vec
     }
     if (clusters > 0) return build_resident_chain(ctx);
   }
-  const int tb = fsv::tile_bits(L, ctx->gates, ctx->precision, ctx->cfg.num_sms);
+  const int tb = fsv::tile_bits(L, ctx->precision, ctx->cfg.num_sms);
   if (tb == 0) return SV_OK;
   const auto plan = fsv::tile_plan(L, ctx->gates, ctx->precision, tb);
   if (plan.empty()) return SV_OK;
@@ -958,13 +987,11 @@ int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab, const std::vec
       ta.cx[i] = (float)ctx->obs.cx[i];
     }
     if (ta.first) ta.ep.rn = renorm_of(ctx);
-    if (ctx->precision == SV_C64 && ta.stride == 0 && !ta.ep.rn.ring) {
+    t.first_gate = p.gates[0];
+    if (ctx->precision == SV_C64 && (ta.stride == 0 || L >= kDriveMinL) && !ta.ep.rn.ring) {
       ta.in_params = 1;
       t.tab.reset(new fsv::TileTab());
-      for (size_t e = 0; e < p.gates.size() * fsv::kGateEntries; ++e) {
-        const float2 g = host_tab[(size_t)p.gates[0] * fsv::kGateEntries + e];
-        t.tab->g[0][e] = fsv::PackedEntry{{g.x, g.x}, {-g.y, g.y}};
-      }
+      pack_tables(&host_tab[(size_t)t.first_gate * fsv::kGateEntries], p.gates.size(), t.tab->g[0]);
       std::memcpy(t.tab->r, p.rounds.data(), sizeof(fsv::TileRound) * p.rounds.size());
     }
     if (ctx->precision == SV_DF64 && ta.stride == 0 && !ta.ep.rn.ring && !ctx->tile_single &&
@@ -1006,6 +1033,8 @@ int build_tiles(sv_ctx* ctx, const std::vector<float2>& host_tab, const std::vec
     round_at += p.rounds.size();
     ctx->tiles.push_back(std::move(t));
   }
+  if (ctx->precision == SV_C64 && ctx->n_period_params > 0 && L >= kDriveMinL)
+    ctx->drive_tab = std::move(host_tab);
   // the rounds behind the gate tables (allocated with them)
   const size_t bytes = rounds.size() * sizeof(fsv::TileRound);
   char* d_rounds = static_cast<char*>(ctx->d_gates) + ctx->d_gates_bytes;
@@ -1140,11 +1169,6 @@ std::vector<fsv::Gate2> adjoint_bonds(const std::vector<fsv::AdjOp>& ops) {
   return g;
 }
 
-int adjoint_tile_bits(const sv_ctx* ctx, const std::vector<fsv::AdjOp>& ops) {
-  return std::min(fsv::kAdjointTileBits,
-                  fsv::tile_bits(ctx->L, adjoint_bonds(ops), SV_C64, ctx->cfg.num_sms));
-}
-
 // The reverse sweep of sv_adjoint in tile passes (complex64): forward to
 // psi_P, lambda = (H0 / L) psi_P, then every period's operations from last to
 // first, several to a pass on tiles of both states.  tab: odag and d of every
@@ -1209,10 +1233,7 @@ int adjoint_tiles(sv_ctx* ctx, int64_t P, const std::vector<fsv::AdjOp>& ops, in
         double* part = d_part + (size_t)(k - k0) * pairs * 2;
         for (int i = 0; i < np; ++i) {
           const fsv::TilePassPlan& p = plan[i];
-          for (size_t e = 0; e < p.gates.size() * 32; ++e) {
-            const float2 g = period[(size_t)p.gates[0] * 32 + e];
-            tt->g[0][e] = fsv::PackedEntry{{g.x, g.x}, {-g.y, g.y}};
-          }
+          pack_tables(&period[(size_t)p.gates[0] * 32], p.gates.size(), tt->g[0]);
           std::memcpy(tt->r, p.rounds.data(), sizeof(fsv::TileRound) * p.rounds.size());
           SV_CUDA(fsv::launch_adjoint_tile(ctx->state, d_lam, passes[i], *tt,
                                            part + 2 * passes[i].pair_at, grids[i], ctx->stream),
@@ -1739,7 +1760,7 @@ int sv_adjoint(sv_ctx* ctx, int64_t periods, double* grad_theta, double* grad_hx
   });
   if (!tables_ok) return fail(ctx, SV_ENOMEM, "adjoint tables");
   if (!c128) {
-    const int tb = adjoint_tile_bits(ctx, ops[0]);
+    const int tb = ctx->L < 5 ? 0 : std::min(ctx->L, fsv::kAdjointTileBits);
     if (tb) return adjoint_tiles(ctx, P, ops[0], tb, tab32, grad_theta, grad_hx, energy_density);
   }
   const int grid = fsv::adjoint_grid(ctx->cfg);

@@ -19,7 +19,7 @@ TOL = {"c64": 8e-6, "df64": 2e-12, "c128": 4e-13}
 @pytest.mark.parametrize("L,K,first,drive", [
     (5, 1, 0, False), (6, 4, 1, True), (8, 2, 0, False), (9, 9, 1, False), (12, 4, 0, True),
     (10, 3, 1, False), (11, 2, 0, True), (13, 6, 1, False), (15, 2, 1, False), (16, 1, 0, False),
-    (17, 2, 0, True), (18, 1, 1, False)])
+    (17, 2, 0, True), (18, 1, 1, False), (19, 1, 1, True)])
 def test_tile_passes_match_oracle(svlib, precision, L, K, first, drive):
     from paper_2111_08044_gb300.sim import FloquetSimulator, chain_params
     P = 3
