@@ -145,7 +145,8 @@ std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int 
   return out;
 }
 
-int tile_bits(int L, int precision, int num_sms) {
+int tile_bits(int L, int precision, const LaunchCfg& cfg) {
+  const int num_sms = cfg.num_sms;
   if (L < 5) return 0;
   // Double-float: a chain that one tile holds stays in one block (10 sites 67 us a
   // period, 98 in tiles of 2^9); else tiles of 2^10, eight warps each, where they
@@ -158,8 +159,10 @@ int tile_bits(int L, int precision, int num_sms) {
   if (precision == SV_C128) return L <= 8 ? L : L < 15 ? 7 : 8;
   // complex64 (chains too long for the resident form): tiles of 2^12 where they leave
   // most SMs one (21 sites 307 us a period, 330 in tiles of 2^11; 24 sites 2.12 and
-  // 2.17 ms), of 2^11 below (16 sites 86 us, 104 in tiles of 2^12, 88 of 2^10).
-  return (4ll << L) >= 3ll * num_sms << 12 ? 12 : 11;
+  // 2.17 ms), of 2^11 below (16 sites 86 us, 104 in tiles of 2^12, 88 of 2^10) unless
+  // other chains' passes fill the rest (12 chains of 16 to 18 sites, 32 periods: 7.5 ms
+  // and 9.4 ms in tiles of 2^11).
+  return !cfg.alone() || (4ll << L) >= 3ll * num_sms << 12 ? 12 : 11;
 }
 
 std::vector<ResidentRound> resident_rounds(const std::vector<Gate2>& gates, const ResidentShape& sh) {

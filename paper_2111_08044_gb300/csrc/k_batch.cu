@@ -138,7 +138,24 @@ __global__ void __launch_bounds__(kThreads)
   for (uint32_t i = threadIdx.x; i < n; i += kThreads) ch.psi[i] = sp[i];
 }
 
+// Ring slots of periods c0 .. c0 + count - 1 of each chain, and its flag: one block
+// a chain.
+__global__ void k_gather_rings(const RingSource* __restrict__ from, long long c0, int count,
+                               int ring_len, double2* __restrict__ out, int* __restrict__ status) {
+  const RingSource src = from[blockIdx.x];
+  const double2* ring = reinterpret_cast<const double2*>(src.ring);
+  for (int q = threadIdx.x; q < count; q += blockDim.x)
+    out[(size_t)blockIdx.x * count + q] = ring[(c0 + q) % ring_len];
+  if (threadIdx.x == 0) status[blockIdx.x] = src.status ? *src.status : 0;
+}
+
 }  // namespace
+
+cudaError_t launch_gather_rings(const RingSource* from, int chains, long long c0, int count,
+                                int ring_len, double* out, int* status, cudaStream_t s) {
+  k_gather_rings<<<chains, 128, 0, s>>>(from, c0, count, ring_len, reinterpret_cast<double2*>(out), status);
+  return cudaGetLastError();
+}
 
 cudaError_t short_prepare() {
   // the carve-out of the resident form's blocks, so that both share an SM

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <map>
 
 #include "sv_block.h"
 #include "sv_device.cuh"
@@ -538,14 +539,32 @@ cudaError_t block_enqueue_period_events(BlockPlan* bp, void* psi, long long* cou
 
 // ------------------------------------------------------------ chain groups
 
+namespace {
 struct BlockGroup {
   std::vector<GroupMember> m;
   std::vector<PassArgs> ops;        // structure of each pass, ntiles over the group
   GroupChain* d_chains = nullptr;   // [passes][chains]
-  ReduceItem* d_reduce = nullptr;   // [chains]
-  double* d_part = nullptr;         // [chains][measuring slots][grid] (energy, norm) pairs
+  double* d_part = nullptr;         // [chains][measuring slots][pairs] (energy, norm) pairs
+  int pairs = 0;                    // of a slot: its CTAs, or 1 (tile sums)
+  float2* d_sums = nullptr;         // tile sums: [chains][slots][tiles of a chain][rows]
   int nt_log2 = 0;
-  int grid = 0;
+};
+struct TileSumItem {
+  const float2* sums = nullptr;
+  double* pair = nullptr;
+  long long first = 0, tiles = 0;  // the chain's tiles among the group's total
+  long long total = 0;
+  int ranges = 0;
+};
+}  // namespace
+
+struct BlockSet {
+  std::vector<BlockGroup> groups;
+  // CTAs of each group in the k-th passes of a period (0: it has fewer)
+  std::vector<std::vector<int>> share;
+  ReduceItem* d_reduce = nullptr;   // [chains]
+  TileSumItem* d_tile_sums = nullptr;  // [chains][slots] (together; else null)
+  int chains = 0, num_sms = 0, ntile_sums = 0;
 };
 
 namespace {
@@ -577,9 +596,74 @@ bool block_same_structure(const BlockPlan* a, const BlockPlan* b) {
   return true;
 }
 
-int block_group_build(const std::vector<GroupMember>& mem, int ring_len, const LaunchCfg& cfg,
-                      cudaStream_t s, BlockGroup** out, std::string* msg) {
-  *out = nullptr;
+namespace {
+
+constexpr int kGroupRows = 128;      // rows of a tile
+constexpr int kTileSumThreads = 512;
+
+// A chain's (energy, norm) of one slot from its tile sums: the group's tiles in
+// `ranges` contiguous ranges, a row's sums over a range in order, compensated, then
+// everything in FP64.
+__global__ void __launch_bounds__(kTileSumThreads) k_tile_sums(const TileSumItem* __restrict__ items) {
+  __shared__ double red[2][kTileSumThreads / 32];
+  const TileSumItem it = items[blockIdx.x];
+  const int row = threadIdx.x & (kGroupRows - 1);
+  const long long end = it.first + it.tiles;
+  double e = 0.0, n = 0.0;
+  grid_wait();
+  grid_trigger();
+  // range v holds the tiles from v total / ranges on
+  long long v = it.first * it.ranges / it.total;
+  while (v > 0 && v * it.total / it.ranges > it.first) --v;
+  while ((v + 1) * it.total / it.ranges <= it.first) ++v;
+  for (v += threadIdx.x / kGroupRows; v < it.ranges; v += kTileSumThreads / kGroupRows) {
+    long long a = v * it.total / it.ranges, b = (v + 1) * it.total / it.ranges;
+    if (a >= end) break;
+    if (a < it.first) a = it.first;
+    if (b > end) b = end;
+    float es = 0.f, ec = 0.f, ns = 0.f, nc = 0.f;
+    for (long long t = a; t < b; ++t) {
+      const float2 s = it.sums[(t - it.first) * kGroupRows + row];
+      const float ye = __fsub_rn(s.x, ec), te = __fadd_rn(es, ye);
+      ec = __fsub_rn(__fsub_rn(te, es), ye);
+      es = te;
+      const float yn = __fsub_rn(s.y, nc), tn = __fadd_rn(ns, yn);
+      nc = __fsub_rn(__fsub_rn(tn, ns), yn);
+      ns = tn;
+    }
+    e += (double)es - (double)ec;
+    n += (double)ns - (double)nc;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    e += __shfl_xor_sync(0xffffffffu, e, o);
+    n += __shfl_xor_sync(0xffffffffu, n, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = e;
+    red[1][threadIdx.x >> 5] = n;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    e = n = 0.0;
+    for (int w = 0; w < kTileSumThreads / 32; ++w) {
+      e += red[0][w];
+      n += red[1][w];
+    }
+    it.pair[0] = e;
+    it.pair[1] = n;
+  }
+}
+
+// CTAs (and ranges of tiles) of a group of `tiles` tiles by itself: one an SM, each
+// with at least kGroupMinTiles tiles.
+constexpr long long kGroupMinTiles = 4;
+int group_ranges(long long tiles, int num_sms) {
+  return (int)std::max<long long>(1, std::min<long long>(num_sms, tiles / kGroupMinTiles));
+}
+
+int group_build(const std::vector<GroupMember>& mem, int num_sms, bool tile_sums, cudaStream_t s,
+                BlockGroup* g, std::string* msg) {
   if (mem.empty()) return SV_EINVAL;
   const BlockPlan* ref = mem[0].plan;
   for (const GroupMember& x : mem) {
@@ -602,14 +686,8 @@ int block_group_build(const std::vector<GroupMember>& mem, int ring_len, const L
       return SV_EINVAL;
     }
   const size_t C = mem.size(), K = ref->args.size();
-  BlockGroup* g = new BlockGroup();
   g->m = mem;
   g->nt_log2 = lg;
-  // one CTA per SM, each with at least kGroupMinTiles tiles (a small group
-  // then leaves SMs to the others instead of paying a CTA's set-up per tile)
-  constexpr long long kGroupMinTiles = 4;
-  g->grid = (int)std::max<long long>(
-      1, std::min<long long>(cfg.num_sms, nt * (long long)C / kGroupMinTiles));
   g->ops = ref->args;
   for (PassArgs& pa : g->ops) {
     pa.ntiles = nt * (long long)C;
@@ -617,17 +695,16 @@ int block_group_build(const std::vector<GroupMember>& mem, int ring_len, const L
     pa.partial = nullptr;  // per chain
   }
   // partial sums: the chains' own buffers hold one pair per CTA of their
-  // own launches; a group launch has its own grid, so the group keeps a
-  // buffer of [chains][slots][grid] pairs (zero where a CTA meets no tile
-  // of the chain)
-  const int S = std::max(1, ref->nslots), G = g->grid;
-  const size_t part_pairs = C * (size_t)S * G;
+  // own launches; a group has its own (zero where a CTA meets no tile of the chain)
+  const int S = std::max(1, ref->nslots);
+  g->pairs = tile_sums ? 1 : group_ranges(nt * (long long)C, num_sms);
+  const size_t part_pairs = C * (size_t)S * g->pairs;
+  const size_t chain_sums = (size_t)nt * kGroupRows;
   std::vector<GroupChain> hc(K * C);
   std::vector<uint8_t> maps(block_tc_map_bytes());
-  cudaError_t e = cudaMalloc(&g->d_part, sizeof(double) * 2 * part_pairs);
-  if (e != cudaSuccess) {
+  if (cudaMalloc(&g->d_part, sizeof(double) * 2 * part_pairs) != cudaSuccess ||
+      (tile_sums && cudaMalloc(&g->d_sums, sizeof(float2) * C * S * chain_sums) != cudaSuccess)) {
     cudaGetLastError();
-    block_group_free(g);
     *msg = "group partials allocation";
     return SV_ENOMEM;
   }
@@ -636,82 +713,235 @@ int block_group_build(const std::vector<GroupMember>& mem, int ring_len, const L
       const PassArgs& pa = mem[c].plan->args[k];
       GroupChain& gc = hc[k * C + c];
       if (block_tc_make_map(pa, mem[c].psi, maps.data()) != SV_OK) {
-        block_group_free(g);
         *msg = "tensor map";
         return SV_ECUDA;
       }
       std::memcpy(gc.map_in, maps.data(), sizeof(gc.map_in));
       std::memcpy(gc.map_out, maps.data() + sizeof(gc.map_in), sizeof(gc.map_out));
       gc.W = pa.W;
-      gc.partial = pa.slot >= 0 ? g->d_part + 2 * ((c * S + pa.slot) * (size_t)G) : nullptr;
+      if (pa.slot >= 0 && tile_sums) gc.partial = g->d_sums + (c * S + pa.slot) * chain_sums;
+      else if (pa.slot >= 0) gc.partial = g->d_part + 2 * (c * S + pa.slot) * (size_t)g->pairs;
       std::memcpy(gc.cx, pa.cx, sizeof(gc.cx));
       std::memcpy(gc.diag_f, pa.diag_f, sizeof(gc.diag_f));
       std::memcpy(gc.diag_lin0, pa.diag_lin0, sizeof(gc.diag_lin0));
     }
-  std::vector<ReduceItem> red(C);
-  for (size_t c = 0; c < C; ++c) {
-    const BlockPlan* bp = mem[c].plan;
-    red[c].partials = g->d_part + 2 * (c * (size_t)S * G);
-    red[c].n = (long long)S * G;
-    red[c].ring = mem[c].ring;
-    red[c].counter = mem[c].counter;
-    red[c].L = bp->L;
-    red[c].ring_len = ring_len;
-  }
-  e = cudaMalloc(&g->d_chains, sizeof(GroupChain) * hc.size());
-  if (e == cudaSuccess) e = cudaMalloc(&g->d_reduce, sizeof(ReduceItem) * C);
+  cudaError_t e = cudaMalloc(&g->d_chains, sizeof(GroupChain) * hc.size());
   if (e == cudaSuccess) e = cudaMemsetAsync(g->d_part, 0, sizeof(double) * 2 * part_pairs, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(g->d_chains, hc.data(), sizeof(GroupChain) * hc.size(),
                         cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(g->d_reduce, red.data(), sizeof(ReduceItem) * C, cudaMemcpyHostToDevice,
-                        s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host arrays are freed below
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host array is freed below
   if (e != cudaSuccess) {
     cudaGetLastError();
-    block_group_free(g);
     *msg = "group upload";
     return SV_ECUDA;
   }
-  *out = g;
   return SV_OK;
 }
 
-int block_group_start(const BlockGroup* g) { return g->m[0].plan->start; }
-
-size_t block_group_size(const BlockGroup* g) { return g->m.size(); }
-
-namespace {
-cudaError_t group_pass(BlockGroup* g, int k, cudaStream_t s) {
-  return launch_block_tc_group(g->ops[k], g->d_chains + (size_t)k * g->m.size(), g->nt_log2,
-                               g->m[0].plan->d_status, g->grid, s);
+// CTAs of groups of t[g] tiles in one launch (0: not part of it), at most one an SM:
+// one each, then one more for the group with most tiles a CTA.
+std::vector<int> cta_shares(const std::vector<long long>& t, int num_sms) {
+  std::vector<int> n(t.size(), 0);
+  int left = num_sms;
+  for (size_t g = 0; g < t.size(); ++g)
+    if (t[g] > 0) {
+      n[g] = 1;
+      --left;
+    }
+  for (; left > 0; --left) {
+    size_t most = t.size();
+    for (size_t g = 0; g < t.size(); ++g)
+      if (t[g] > n[g] && (most == t.size() || t[g] * n[most] > t[most] * n[g])) most = g;
+    if (most == t.size()) break;  // one tile a CTA
+    ++n[most];
+  }
+  return n;
 }
+
+// One launch (or several, of kGroupsPerLaunch groups each) of op[g] of every group g with
+// CTAs in share.
+cudaError_t set_pass(BlockSet* set, const std::vector<int>& op, const std::vector<int>& share,
+                     bool overlap, cudaStream_t s) {
+  GroupPasses p;
+  int n = 0, ctas = 0;
+  auto launch = [&]() {
+    const cudaError_t e =
+        n ? launch_block_tc_groups(p, n, set->groups[0].m[0].plan->d_status, overlap, s) : cudaSuccess;
+    n = ctas = 0;
+    return e;
+  };
+  for (size_t g = 0; g < set->groups.size(); ++g) {
+    if (share[g] == 0) continue;
+    const BlockGroup& gr = set->groups[g];
+    GroupPass& q = p.g[n++];
+    q.pa = gr.ops[op[g]];
+    q.chains = gr.d_chains + (size_t)op[g] * gr.m.size();
+    q.nt_log2 = gr.nt_log2;
+    q.tile_sums = gr.d_sums != nullptr;
+    q.cta_end = ctas += share[g];
+    if (n == kGroupsPerLaunch) {
+      const cudaError_t e = launch();
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return launch();
+}
+
+// The passes seq(plan) of every group, the k-th of all of them together.
+template <typename Seq>
+cudaError_t set_sequence(BlockSet* set, const Seq& seq, bool overlap, cudaStream_t s) {
+  const size_t G = set->groups.size();
+  for (size_t k = 0;; ++k) {
+    std::vector<long long> t(G, 0);
+    std::vector<int> op(G, 0);
+    bool any = false;
+    for (size_t g = 0; g < G; ++g) {
+      const std::vector<int>& q = seq(set->groups[g].m[0].plan);
+      if (k >= q.size()) continue;
+      any = true;
+      op[g] = q[k];
+      t[g] = set->groups[g].ops[0].ntiles;
+    }
+    if (!any) return cudaSuccess;
+    const std::vector<int> share =
+        set->d_tile_sums ? cta_shares(t, set->num_sms) : std::vector<int>(1, set->groups[0].pairs);
+    const cudaError_t e = set_pass(set, op, share, overlap, s);
+    if (e != cudaSuccess) return e;
+  }
+}
+
 }  // namespace
 
-cudaError_t block_group_enqueue_entry(BlockGroup* g, cudaStream_t s) {
-  for (int k : g->m[0].plan->seq_entry) {
-    cudaError_t e = group_pass(g, k, s);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+bool block_groups_together(const std::vector<std::vector<GroupMember>>& groups, const LaunchCfg& cfg) {
+  // Below three tiles an SM in all, one launch on one tile or a few a CTA gains: 48
+  // chains of 14 sites (96 tiles) take 98 us a period, 24 of 15 to 17 sites (224)
+  // 125 us, 48 of them (448) 172 us; in launches of their own, of four tiles a CTA,
+  // 153, 165 and 185 us.  From there on these overlap better: 24 chains of 15 to 19
+  // sites (595) 190 us, together 213 us.
+  constexpr long long kTogether = 3;
+  long long tiles = 0;
+  for (const auto& g : groups) tiles += g[0].plan->args[0].ntiles * (long long)g.size();
+  return tiles < kTogether * cfg.num_sms;
 }
 
-cudaError_t block_group_enqueue_period(BlockGroup* g, cudaStream_t s, bool last) {
-  const BlockPlan* ref = g->m[0].plan;
-  for (int k : last ? ref->seq_exit : ref->seq_cyc) {
-    cudaError_t e = group_pass(g, k, s);
-    if (e != cudaSuccess) return e;
+int block_set_build(const std::vector<std::vector<GroupMember>>& groups, bool together, int ring_len,
+                    const LaunchCfg& cfg, cudaStream_t s, BlockSet** out, std::string* msg) {
+  *out = nullptr;
+  if (groups.empty() || (!together && groups.size() != 1)) return SV_EINVAL;
+  BlockSet* set = new BlockSet();
+  set->num_sms = cfg.num_sms;
+  set->groups.resize(groups.size());
+  int rc = SV_OK;
+  size_t longest = 0;
+  std::vector<ReduceItem> red;
+  std::vector<TileSumItem> sums;
+  for (size_t g = 0; g < groups.size() && rc == SV_OK; ++g) {
+    BlockGroup& gr = set->groups[g];
+    rc = group_build(groups[g], cfg.num_sms, together, s, &gr, msg);
+    if (rc) break;
+    const size_t S = std::max(1, gr.m[0].plan->nslots);
+    longest = std::max(longest, gr.m[0].plan->seq_cyc.size());
+    for (size_t c = 0; c < gr.m.size(); ++c) {
+      ReduceItem it;
+      it.partials = gr.d_part + 2 * (c * S * (size_t)gr.pairs);
+      it.n = (long long)S * gr.pairs;
+      it.ring = gr.m[c].ring;
+      it.counter = gr.m[c].counter;
+      it.L = gr.m[c].plan->L;
+      it.ring_len = ring_len;
+      red.push_back(it);
+      for (size_t k = 0; k < S && together; ++k) {
+        TileSumItem t;
+        t.tiles = 1ll << gr.nt_log2;
+        t.sums = gr.d_sums + (c * S + k) * (size_t)t.tiles * kGroupRows;
+        t.pair = gr.d_part + 2 * (c * S + k);
+        t.first = (long long)c * t.tiles;
+        t.total = gr.ops[0].ntiles;
+        t.ranges = group_ranges(t.total, cfg.num_sms);
+        sums.push_back(t);
+      }
+    }
   }
-  return launch_period_reduce_many(g->d_reduce, (int)g->m.size(), s);
+  set->chains = (int)red.size();
+  set->ntile_sums = (int)sums.size();
+  for (size_t k = 0; k < longest && rc == SV_OK; ++k) {
+    std::vector<long long> t;
+    for (const BlockGroup& gr : set->groups)
+      t.push_back(k < gr.m[0].plan->seq_cyc.size() ? gr.ops[0].ntiles : 0);
+    set->share.push_back(together ? cta_shares(t, cfg.num_sms) : std::vector<int>(1, set->groups[0].pairs));
+  }
+  if (rc == SV_OK) {
+    cudaError_t e = cudaMalloc(&set->d_reduce, sizeof(ReduceItem) * red.size());
+    if (e == cudaSuccess && together) e = cudaMalloc(&set->d_tile_sums, sizeof(TileSumItem) * sums.size());
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(set->d_reduce, red.data(), sizeof(ReduceItem) * red.size(),
+                          cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && together)
+      e = cudaMemcpyAsync(set->d_tile_sums, sums.data(), sizeof(TileSumItem) * sums.size(),
+                          cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host arrays are freed below
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      *msg = "group upload";
+      rc = SV_ECUDA;
+    }
+  }
+  if (rc != SV_OK) {
+    block_set_free(set);
+    return rc;
+  }
+  *out = set;
+  return SV_OK;
 }
 
-void block_group_free(BlockGroup* g) {
-  if (!g) return;
-  cudaFree(g->d_chains);
-  cudaFree(g->d_reduce);
-  cudaFree(g->d_part);
-  delete g;
+size_t block_set_size(const BlockSet* set) { return set->chains; }
+
+cudaError_t block_set_enqueue(BlockSet* set, int periods, bool alone, cudaStream_t s) {
+  if (periods <= 0) return cudaSuccess;
+  cudaError_t e = set_sequence(
+      set, [](const BlockPlan* p) -> const std::vector<int>& { return p->seq_entry; }, alone, s);
+  for (int k = 0; k < periods && e == cudaSuccess; ++k) {
+    const bool last = k + 1 == periods;
+    std::vector<int> op(set->groups.size(), 0);
+    for (size_t j = 0; j < set->share.size() && e == cudaSuccess; ++j) {
+      for (size_t g = 0; g < set->groups.size(); ++g) {
+        const BlockPlan* p = set->groups[g].m[0].plan;
+        if (j < p->seq_cyc.size()) op[g] = (last ? p->seq_exit : p->seq_cyc)[j];
+      }
+      e = set_pass(set, op, set->share[j], alone, s);
+    }
+    if (e == cudaSuccess && set->ntile_sums) {
+      void* args[] = {&set->d_tile_sums};
+      e = launch_overlapped(reinterpret_cast<const void*>(k_tile_sums), set->ntile_sums, kTileSumThreads,
+                            0, s, args, alone);
+    }
+    if (e == cudaSuccess) e = launch_period_reduce_many(set->d_reduce, set->chains, alone, s);
+  }
+  // the relabel steps behind the last period's passes
+  if (e == cudaSuccess) {
+    std::map<const BlockPlan*, std::vector<int>> rest;
+    for (const BlockGroup& gr : set->groups) {
+      const BlockPlan* p = gr.m[0].plan;
+      rest[p].assign(p->seq_exit.begin() + std::min(p->seq_cyc.size(), p->seq_exit.size()),
+                     p->seq_exit.end());
+    }
+    e = set_sequence(
+        set, [&](const BlockPlan* p) -> const std::vector<int>& { return rest[p]; }, alone, s);
+  }
+  return e;
+}
+
+void block_set_free(BlockSet* set) {
+  if (!set) return;
+  for (BlockGroup& g : set->groups) {
+    cudaFree(g.d_chains);
+    cudaFree(g.d_part);
+    cudaFree(g.d_sums);
+  }
+  cudaFree(set->d_reduce);
+  cudaFree(set->d_tile_sums);
+  delete set;
 }
 
 void block_free(BlockPlan* bp) {

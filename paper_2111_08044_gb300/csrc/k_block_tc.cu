@@ -67,6 +67,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "sv_block.h"
 #include "sv_device.cuh"
@@ -411,17 +412,23 @@ __device__ __forceinline__ int tile_row(const PassArgs& pa, int m) {
 // instance (kGeneric, flags read at run time), so that SMs switching between
 // their CTAs keep one kernel's code in the instruction cache.
 //
-// kGroup (with kGeneric): one launch over the tiles of a chain group.  Tile
-// g of the group is tile g mod 2^nt_log2 of chain g / 2^nt_log2; a CTA takes
-// a contiguous range of them, so it meets each chain once.  At a change of
-// chain the producer reloads the operand block once the MMAs are done with
-// the previous one (kBarWFree), and the epilogue writes the previous chain's
-// partial sums and takes the new chain's coefficients and descriptors.
+// kGroup (with kGeneric): one launch over the tiles of several chain groups, each on
+// CTAs of its own.  Tile g of a group is tile g mod 2^nt_log2 of its chain
+// g / 2^nt_log2; a CTA takes a contiguous range of them, so it meets each chain
+// once.  At a change of chain the producer reloads the operand block once the MMAs
+// are done with the previous one (kBarWFree), and the epilogue writes the previous
+// chain's partial sums and takes the new chain's coefficients and descriptors.
+//
+// A CTA's set-up, first tile and last store (about 8 us) are paid per launch, beside
+// 2.7 us a tile (its 128 KiB at the L2 cache's rate), hence the sets of groups.
+struct SinglePass {
+  CUtensorMap in, out;
+  PassArgs pa;
+};
 template <bool kGeneric, bool kX, bool kDiag, bool kGroup = false>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_block_tc(const __grid_constant__ CUtensorMap tmap_in,
-               const __grid_constant__ CUtensorMap tmap_out, PassArgs pa, int* status,
-               const GroupChain* __restrict__ grp, int nt_log2) {
+    k_block_tc(const __grid_constant__ typename std::conditional<kGroup, GroupPasses, SinglePass>::type arg,
+               int* status) {
   static_assert(!kGroup || kGeneric, "a group pass takes the generic epilogue");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
@@ -431,16 +438,34 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t mbase = sbase + kOffMisc;
   volatile uint32_t* abort = reinterpret_cast<volatile uint32_t*>(misc + kAbort);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the pass, and this CTA among its CTAs
+  int which = 0;
+  uint32_t bx = blockIdx.x, nb = gridDim.x;
+  if constexpr (kGroup) {
+    while ((int)blockIdx.x >= arg.g[which].cta_end) ++which;
+    const int first = which ? arg.g[which - 1].cta_end : 0;
+    bx -= first;
+    nb = arg.g[which].cta_end - first;
+  }
+  const PassArgs& pa = [&]() -> const PassArgs& {
+    if constexpr (kGroup) return arg.g[which].pa;
+    else return arg.pa;
+  }();
+  const GroupChain* grp = nullptr;
+  int nt_log2 = 0;
+  if constexpr (kGroup) {
+    grp = arg.g[which].chains;
+    nt_log2 = arg.g[which].nt_log2;
+  }
   const int a = pa.a;
   const long long ntiles = pa.ntiles;
   // this CTA's tiles: strided over the pass, or (group) a contiguous range
-  const long long my_first = kGroup ? (long long)blockIdx.x * ntiles / gridDim.x : 0;
-  const long long my_tiles =
-      kGroup ? ((long long)blockIdx.x + 1) * ntiles / gridDim.x - my_first
-             : (blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0);
+  const long long my_first = kGroup ? (long long)bx * ntiles / nb : 0;
+  const long long my_tiles = kGroup ? ((long long)bx + 1) * ntiles / nb - my_first
+                                    : (bx < ntiles ? (ntiles - 1 - bx) / nb + 1 : 0);
   // tile index within its chain, and the chain, of this CTA's tile i
   auto tile_of = [&](long long i) -> long long {
-    return kGroup ? ((my_first + i) & ((1ll << nt_log2) - 1)) : blockIdx.x + i * gridDim.x;
+    return kGroup ? ((my_first + i) & ((1ll << nt_log2) - 1)) : bx + i * nb;
   };
   auto chain_of = [&](long long i) -> int { return kGroup ? (int)((my_first + i) >> nt_log2) : 0; };
   // tile i starts a chain other than tile i - 1's
@@ -645,7 +670,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // per-thread energy and norm over its tiles: compensated FP32 sums
     // (Kahan), so that no FP64 instruction runs per tile
     float es_s = 0.f, es_c = 0.f, ns_s = 0.f, ns_c = 0.f;
-    // energy partials of this CTA into part[2 blockIdx.x + {0, 1}] (fixed order)
+    // energy partials of this CTA into part[2 bx + {0, 1}] (fixed order)
     auto flush = [&](double* part) {
       if (!part) return;
       double eacc = (double)es_s - (double)es_c, nacc = (double)ns_s - (double)ns_c;
@@ -661,18 +686,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       epilogue_sync();
       if (q == 0 && lane == 0) {
-        part[2 * blockIdx.x] = (red[0] + red[2]) + (red[4] + red[6]);
-        part[2 * blockIdx.x + 1] = (red[1] + red[3]) + (red[5] + red[7]);
+        part[2 * bx] = (red[0] + red[2]) + (red[4] + red[6]);
+        part[2 * bx + 1] = (red[1] + red[3]) + (red[5] + red[7]);
       }
     };
     int cur = -1;  // group: the chain whose coefficients are loaded
-    const CUtensorMap* map_out = &tmap_out;
+    bool tile_sums = false;
+    if constexpr (kGroup) tile_sums = arg.g[which].tile_sums;
+    const CUtensorMap* map_out = nullptr;
+    if constexpr (!kGroup) map_out = &arg.out;
     for (long long i = 0; i < my_tiles; ++i) {
       if constexpr (kGroup) {
         const int c = chain_of(i);
         if (c != cur) {
-          if (cur >= 0) {
-            flush(grp[cur].partial);
+          if (cur >= 0 && !tile_sums) {
+            flush(static_cast<double*>(grp[cur].partial));
             es_s = es_c = ns_s = ns_c = 0.f;
           }
           epilogue_sync();  // the previous chain's coefficients are no longer read
@@ -814,7 +842,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         ns += S;
         es += fmaf(h0, S, a_lo + a_hi);
       }
-      {
+      if (kGroup && tile_sums) {
+        if (grp[cur].partial)
+          static_cast<float2*>(grp[cur].partial)[tile_of(i) * kRows + q * 32 + lane] = make_float2(es, ns);
+      } else {
         const float ye = es - es_c, te = es_s + ye;
         es_c = (te - es_s) - ye;
         es_s = te;
@@ -861,7 +892,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the CTA's stores complete before its shared memory is released
     if (elected) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if constexpr (kGroup) {
-      if (cur >= 0) flush(grp[cur].partial);
+      if (cur >= 0 && !tile_sums) flush(static_cast<double*>(grp[cur].partial));
     } else {
       flush(pa.partial);
     }
@@ -926,7 +957,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     } else if (warp == 9 && lane == 0) {
       // load number g is box (g mod 4) of tile g / 4, into slot g mod kSlots
-      const CUtensorMap* map_in = &tmap_in;
+      const CUtensorMap* map_in = nullptr;
+      if constexpr (!kGroup) map_in = &arg.in;
       auto load_box = [&](long long g) {
         const long long t = tile_of(g >> 2);
         const int tlo = (int)(t & ((1ll << (a - kN)) - 1));
@@ -1349,32 +1381,27 @@ cudaError_t block_tc_prepare() {
 
 cudaError_t launch_block_tc(const PassArgs& pa, void* psi, const void* map, int* status,
                             int grid, cudaStream_t s, bool overlap) {
-  PassArgs p = pa;
-  p.psi = psi;
-  alignas(64) CUtensorMap maps[2];
-  std::memcpy(maps, map, sizeof(maps));
+  SinglePass p;
+  std::memcpy(&p.in, map, sizeof(p.in));
+  std::memcpy(&p.out, static_cast<const char*>(map) + sizeof(p.in), sizeof(p.out));
+  p.pa = pa;
+  p.pa.psi = psi;
   constexpr long long kMinTilesSpecialised = 32;  // tiles per CTA
-  const long long per_cta = (p.ntiles + grid - 1) / grid;
+  const long long per_cta = (pa.ntiles + grid - 1) / grid;
   const void* k = (const void*)k_block_tc<false, false, false>;
   if (per_cta < kMinTilesSpecialised) k = (const void*)k_block_tc<true, false, false>;
-  else if (p.diag && p.x_mask) k = (const void*)k_block_tc<false, true, true>;
-  else if (p.diag) k = (const void*)k_block_tc<false, false, true>;
-  else if (p.x_mask) k = (const void*)k_block_tc<false, true, false>;
-  const GroupChain* group = nullptr;
-  int nt_log2 = 0;
-  void* args[] = {&maps[0], &maps[1], &p, &status, &group, &nt_log2};
+  else if (pa.diag && pa.x_mask) k = (const void*)k_block_tc<false, true, true>;
+  else if (pa.diag) k = (const void*)k_block_tc<false, false, true>;
+  else if (pa.x_mask) k = (const void*)k_block_tc<false, true, false>;
+  void* args[] = {&p, &status};
   return launch_overlapped(k, grid, kThreads, kSmemBytes, s, args, overlap);
 }
 
-cudaError_t launch_block_tc_group(const PassArgs& pa, const GroupChain* chains, int nt_log2,
-                                  int* status, int grid, cudaStream_t s) {
-  // the kernel's descriptor parameters are unused: each chain's come from
-  // the group array
-  alignas(64) CUtensorMap unused[2];
-  std::memset(unused, 0, sizeof(unused));
-  k_block_tc<true, false, false, true><<<grid, kThreads, kSmemBytes, s>>>(
-      unused[0], unused[1], pa, status, chains, nt_log2);
-  return cudaGetLastError();
+cudaError_t launch_block_tc_groups(const GroupPasses& passes, int n, int* status, bool overlap,
+                                   cudaStream_t s) {
+  void* args[] = {const_cast<GroupPasses*>(&passes), &status};
+  return launch_overlapped((const void*)k_block_tc<true, false, false, true>, passes.g[n - 1].cta_end,
+                           kThreads, kSmemBytes, s, args, overlap);
 }
 
 }  // namespace fsv

@@ -590,9 +590,11 @@ cudaError_t launch_period_reduce(const double* partials, long long n, int L, dou
   return launch_overlapped(reinterpret_cast<const void*>(k_period_reduce), 1, 256, 0, s, args);
 }
 
-cudaError_t launch_period_reduce_many(const ReduceItem* items, int count, cudaStream_t s) {
-  k_period_reduce_many<<<count, 256, 0, s>>>(items);
-  return cudaGetLastError();
+cudaError_t launch_period_reduce_many(const ReduceItem* items, int count, bool overlap,
+                                      cudaStream_t s) {
+  void* args[] = {&items};
+  return launch_overlapped(reinterpret_cast<const void*>(k_period_reduce_many), count, 256, 0, s, args,
+                           overlap);
 }
 
 cudaError_t launch_product_state(int precision, void* psi, int L, const double* spinors,

@@ -434,8 +434,11 @@ void ctx_set_min_tiles(sv_ctx* ctx, int tiles) { ctx->cfg.min_tiles_per_cta = ti
 
 void ctx_set_cyclic(sv_ctx* ctx, bool cyclic) { ctx->cyclic = cyclic; }
 
-int ctx_read_energies(sv_ctx* ctx, int64_t c0, int64_t count, double* e, double* n) {
-  return read_ring(ctx, c0, count, e, n);
+RingSource ctx_ring(const sv_ctx* ctx) {
+  RingSource s;
+  s.ring = ctx->d_ring;
+  s.status = ctx->block ? ctx->block->d_status : nullptr;
+  return s;
 }
 
 int ctx_ring_len() { return kRing; }
@@ -956,7 +959,7 @@ int build_tiles(sv_ctx* ctx, std::vector<float2>& host_tab, const std::vector<fl
     }
     if (clusters > 0) return build_resident_chain(ctx);
   }
-  const int tb = fsv::tile_bits(L, ctx->precision, ctx->cfg.num_sms);
+  const int tb = fsv::tile_bits(L, ctx->precision, ctx->cfg);
   if (tb == 0) return SV_OK;
   const auto plan = fsv::tile_plan(L, ctx->gates, ctx->precision, tb);
   if (plan.empty()) return SV_OK;

@@ -7,9 +7,9 @@
 // 14 sites may instead run the resident form (k_resident.cu): one launch per
 // length advances them, each in the shared memory of one CTA or of a cluster.  An evolution is
 // one CUDA graph per run of M periods: the resident launch; one branch per
-// group of tensor-core chains whose plans share their structure (same L),
-// each pass of all its chains one launch over all their tiles and each
-// period's reduces one launch; and, for every other chain, its run of M
+// group of tensor-core chains whose plans share their structure (same L; one
+// branch for all groups where their tiles are few), each pass of all its chains
+// one launch over all their tiles and each period's reduces one launch; and, for every other chain, its run of M
 // periods captured from its context.  A block plan whose periods start off
 // site 0 relabels into its period layout at the start of the run and hands
 // back the natural layout at its end.
@@ -84,7 +84,12 @@ struct sv_batch {
   // of a batch whose chains all are resident: d_count[1] (run) periods
   cudaGraphExec_t gr = nullptr;
   int64_t run = 0;
-  std::vector<fsv::BlockGroup*> groups;  // chain groups the two graphs launch
+  std::vector<fsv::BlockSet*> groups;  // chain groups the two graphs launch
+  // energies of the graph-form chains: their rings, and a buffer that a run's
+  // slots are gathered into for one copy
+  fsv::RingSource* d_rings = nullptr;
+  char* d_gather = nullptr;
+  size_t gather_bytes = 0;
   int M = 16;
   int64_t counter = 0;
   std::string err;
@@ -265,10 +270,10 @@ int build_graph_form(sv_batch* b, int c, int form, int n) {
   return SV_OK;
 }
 
-// Tensor-core chains grouped by plan structure (an existing group of the
-// same structure is reused); the other chains are returned in `rest`.
+// Tensor-core chains grouped by plan structure, the groups in sets; the other chains
+// are returned in `rest`.
 int make_groups(sv_batch* b, const std::vector<int>& chains, std::vector<int>* rest,
-                std::vector<fsv::BlockGroup*>* groups) {
+                std::vector<fsv::BlockSet*>* sets) {
   std::vector<std::vector<fsv::GroupMember>> parts;
   for (int c : chains) {
     fsv::GroupMember m;
@@ -285,27 +290,31 @@ int make_groups(sv_batch* b, const std::vector<int>& chains, std::vector<int>* r
       }
     if (!placed) parts.push_back({m});
   }
-  for (auto& p : parts) {
-    fsv::BlockGroup* g = nullptr;
+  if (parts.empty()) return SV_OK;
+  const fsv::LaunchCfg& cfg = parts[0][0].plan->cfg;
+  const bool together = fsv::block_groups_together(parts, cfg);
+  for (size_t k = 0; k < (together ? 1 : parts.size()); ++k) {
+    fsv::BlockSet* set = nullptr;
     std::string msg;
-    int rc = fsv::block_group_build(p, fsv::ctx_ring_len(), p[0].plan->cfg, b->stream, &g, &msg);
-    if (rc) return bfail(b, rc, "chain group: %s", msg.c_str());
-    groups->push_back(g);
+    int rc = fsv::block_set_build(together ? parts : std::vector<std::vector<fsv::GroupMember>>{parts[k]},
+                                  together, fsv::ctx_ring_len(), cfg, b->stream, &set, &msg);
+    if (rc) return bfail(b, rc, "chain groups: %s", msg.c_str());
+    sets->push_back(set);
   }
   return SV_OK;
 }
 
-void free_groups(std::vector<fsv::BlockGroup*>* groups) {
-  for (fsv::BlockGroup* g : *groups) fsv::block_group_free(g);
-  groups->clear();
+void free_groups(std::vector<fsv::BlockSet*>* sets) {
+  for (fsv::BlockSet* s : *sets) fsv::block_set_free(s);
+  sets->clear();
 }
 
 // One graph advancing `periods` periods of the given graph-form chains and
-// of the resident set (if any); 0 (a resident set alone): d_count[1] periods.  Tensor-core chains run in groups, built on
-// the first call (groups empty) and reused by later ones; the caller frees
-// them after the graphs.
+// of the resident set (if any); 0 (a resident set alone): d_count[1] periods.
+// Tensor-core chains run in groups, built on the first call (groups empty) and
+// reused by later ones; the caller frees them after the graphs.
 int make_graph(sv_batch* b, const std::vector<int>& chains, const ResidentSet* rs, int periods,
-               cudaGraphExec_t* out, std::vector<fsv::BlockGroup*>* groups) {
+               cudaGraphExec_t* out, std::vector<fsv::BlockSet*>* groups) {
   *out = nullptr;
   cudaGraph_t g = nullptr;
   BCUDA(cudaGraphCreate(&g, 0), "graph create");
@@ -363,19 +372,17 @@ int make_graph(sv_batch* b, const std::vector<int>& chains, const ResidentSet* r
         ++grouped;
     }
     size_t members = 0;
-    for (fsv::BlockGroup* grp : *groups) members += fsv::block_group_size(grp);
+    for (const fsv::BlockSet* set : *groups) members += fsv::block_set_size(set);
     if (members != grouped)
       return fail_g(bfail(b, SV_ESTATE, "chain groups built for another set of chains"));
   }
-  for (fsv::BlockGroup* grp : *groups) {
+  for (fsv::BlockSet* set : *groups) {
+    const bool alone = groups->size() == 1 && rest.empty() && (!rs || rs->count == 0);
     cudaGraph_t pg = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeRelaxed);
     cudaError_t le = cudaSuccess;
     if (e == cudaSuccess) {
-      if (periods > 0 && fsv::block_group_start(grp) != 0)
-        le = fsv::block_group_enqueue_entry(grp, b->cap_stream);
-      for (int k = 0; k < periods && le == cudaSuccess; ++k)
-        le = fsv::block_group_enqueue_period(grp, b->cap_stream, k + 1 == periods);
+      le = fsv::block_set_enqueue(set, periods, alone, b->cap_stream);
       e = cudaStreamEndCapture(b->cap_stream, &pg);
       if (le != cudaSuccess) e = le;
     }
@@ -408,6 +415,49 @@ int make_graph(sv_batch* b, const std::vector<int>& chains, const ResidentSet* r
   return SV_OK;
 }
 
+// Energies and norms of the graph-form chains' last `count` periods (one copy for
+// all chains, rows of `periods` from column `done`).
+int read_graph_chains(sv_batch* b, const std::vector<int>& chains, int64_t count, int64_t periods,
+                      int64_t done, double* energy_out, double* norm_out) {
+  const size_t C = chains.size(), pairs = C * (size_t)count;
+  const size_t bytes = 2 * sizeof(double) * pairs + sizeof(int) * C;
+  if (!b->d_rings) {
+    std::vector<fsv::RingSource> src;
+    for (int c : chains) src.push_back(fsv::ctx_ring(b->ctx[c]));
+    BCUDA(cudaMalloc(&b->d_rings, sizeof(fsv::RingSource) * C), "ring list");
+    BCUDA(cudaMemcpyAsync(b->d_rings, src.data(), sizeof(fsv::RingSource) * C, cudaMemcpyHostToDevice,
+                          b->stream),
+          "upload ring list");
+    BCUDA(cudaStreamSynchronize(b->stream), "synchronize");
+  }
+  if (b->gather_bytes < bytes) {
+    cudaFree(b->d_gather);
+    b->d_gather = nullptr;
+    b->gather_bytes = 0;
+    BCUDA(cudaMalloc(&b->d_gather, bytes), "energy readback buffer");
+    b->gather_bytes = bytes;
+  }
+  double* out = reinterpret_cast<double*>(b->d_gather);
+  BCUDA(fsv::launch_gather_rings(b->d_rings, (int)C, b->counter, (int)count, fsv::ctx_ring_len(), out,
+                                 reinterpret_cast<int*>(out + 2 * pairs), b->stream),
+        "energy gather launch");
+  std::vector<char> host(bytes);
+  BCUDA(cudaMemcpyAsync(host.data(), b->d_gather, bytes, cudaMemcpyDeviceToHost, b->stream),
+        "energy readback");
+  BCUDA(cudaStreamSynchronize(b->stream), "synchronize");
+  const double* p = reinterpret_cast<const double*>(host.data());
+  const int* status = reinterpret_cast<const int*>(p + 2 * pairs);
+  for (size_t k = 0; k < C; ++k) {
+    if (status[k])
+      return bfail(b, SV_ETIMEOUT, "chain %d: a tensor-core block pass gave up a bounded wait", chains[k]);
+    for (int64_t q = 0; q < count; ++q, p += 2) {
+      if (energy_out) energy_out[(size_t)chains[k] * periods + done + q] = p[0];
+      if (norm_out) norm_out[(size_t)chains[k] * periods + done + q] = p[1];
+    }
+  }
+  return SV_OK;
+}
+
 int reinit(sv_batch* b, int c) {
   int rc = sv_init(b->ctx[c], b->L[c], b->spinors[c]);
   if (rc) return bfail(b, rc, "chain %d init: %s", c, sv_last_error(b->ctx[c]));
@@ -434,7 +484,7 @@ int time_forms(sv_batch* b, const std::vector<int>& sample, const std::vector<in
   }
   if (rc == SV_OK) rc = build_resident(b, res_chains, &rs);
   cudaGraphExec_t ge = nullptr;
-  std::vector<fsv::BlockGroup*> groups;
+  std::vector<fsv::BlockSet*> groups;
   if (rc == SV_OK) rc = make_graph(b, graph_chains, &rs, kPeriods, &ge, &groups);
   if (rc == SV_OK) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -530,6 +580,8 @@ void destroy(sv_batch* b) {
   if (b->gr) cudaGraphExecDestroy(b->gr);
   free_groups(&b->groups);
   b->rset.release();
+  cudaFree(b->d_rings);
+  cudaFree(b->d_gather);
   for (sv_ctx* c : b->ctx)
     if (c) sv_destroy(c);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
@@ -669,15 +721,11 @@ int sv_batch_evolve(sv_batch* b, int64_t periods, double* energy_out, double* no
     for (; b->gm && k + b->M <= chunk; k += b->M)
       BCUDA(cudaGraphLaunch(b->gm, b->stream), "graph launch");
     for (; k < chunk; ++k) BCUDA(cudaGraphLaunch(b->g1, b->stream), "graph launch");
-    for (int c : graph_chains) {
-      double* e = energy_out ? energy_out + (size_t)c * periods + done : nullptr;
-      double* n = norm_out ? norm_out + (size_t)c * periods + done : nullptr;
-      if (e || n) {
-        int rc = fsv::ctx_read_energies(b->ctx[c], b->counter, chunk, e, n);
-        if (rc) return bfail(b, rc, "chain %d: %s", c, sv_last_error(b->ctx[c]));
-      }
-      fsv::ctx_advance(b->ctx[c], chunk);
+    if (!graph_chains.empty() && (energy_out || norm_out)) {
+      int rc = read_graph_chains(b, graph_chains, chunk, periods, done, energy_out, norm_out);
+      if (rc) return rc;
     }
+    for (int c : graph_chains) fsv::ctx_advance(b->ctx[c], chunk);
     if (!b->res.empty() && (energy_out || norm_out)) {
       // the slots written, every chain's pair of a slot together
       const size_t row = 2 * b->res.size(), at = (size_t)(b->counter % ring);

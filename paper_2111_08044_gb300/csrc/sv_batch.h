@@ -83,6 +83,10 @@ cudaError_t launch_resident_batch(const ChainArgs* chains, int nchains, const Re
 cudaError_t launch_chain_short(const ChainArgs* chains, int nchains, const long long* counter,
                                int periods, int ring_len, cudaStream_t s);
 cudaError_t short_prepare();
+// (energy, norm) of `count` periods from c0 on of each chain into out[chain][count],
+// its flag into status[chain].
+cudaError_t launch_gather_rings(const RingSource* from, int chains, long long c0, int count,
+                                int ring_len, double* out, int* status, cudaStream_t s);
 cudaError_t launch_advance(long long* counter, int periods, cudaStream_t s);
 
 // The complex64 tables of a period's gates (kGateEntries each: the rounded gate

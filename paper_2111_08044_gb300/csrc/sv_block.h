@@ -66,18 +66,33 @@ struct PassArgs {
 
 // Per chain and pass of a chain group (chains whose plans share every
 // structural field: same L, windows, relabels and staging; they differ in
-// operands and measured coefficients).  The group's tensor-core pass runs
-// all chains' tiles in one launch.
+// operands and measured coefficients).
 struct alignas(64) GroupChain {
   unsigned char map_in[128];   // TMA descriptors (CUtensorMap) for this
   unsigned char map_out[128];  // chain's state
   const void* W = nullptr;     // the chain's operand block of this pass
-  double* partial = nullptr;   // the chain's (energy, norm) pairs, or null
+  void* partial = nullptr;     // the chain's (energy, norm) pairs (one a CTA, or of
+                               // FP32 one a tile and row), or null
   float cx[8] = {};
   float diag_f[5] = {};
   float diag_lin0[8] = {};
 };
 static_assert(sizeof(GroupChain) % 64 == 0, "descriptors stay 64-byte aligned in an array");
+
+// A group's pass within a launch over several groups: its structure (ntiles over
+// all its chains), chains (device array), tiles of a chain and last CTA + 1 (its
+// CTAs follow the previous group's).
+struct GroupPass {
+  PassArgs pa;
+  const GroupChain* chains = nullptr;
+  int nt_log2 = 0, cta_end = 0;
+  int tile_sums = 0;  // partial: a (energy, norm) pair of FP32 sums per tile and row
+};
+constexpr int kGroupsPerLaunch = 16;
+struct GroupPasses {
+  GroupPass g[kGroupsPerLaunch];
+};
+static_assert(sizeof(GroupPasses) <= 16 * 1024, "kernel parameters");
 
 struct BlockPlan {
   int L = 0, n = 0, R = 0, split = 0;
@@ -134,28 +149,36 @@ cudaError_t block_enqueue_period_events(BlockPlan* bp, void* psi, long long* cou
 void block_free(BlockPlan* bp);
 
 // Chain groups: tensor-core chains whose plans share every structural field
-// (same L, windows, relabels, staging orders and measured passes) run each
-// pass of all chains as one launch, and their period reduces as one.
+// (same L, windows, relabels, staging orders and measured passes).  A set of
+// groups advances together: the k-th pass of all of them is one launch, each
+// group on a share of the CTAs, and the period reduces of all their chains are
+// one.
+//
+// A chain's energy terms are summed as by CTAs of G = min(SMs, T / 4) contiguous
+// ranges of the group's T tiles (FP32, compensated, per row).  A set of one group
+// has those G CTAs.  Where CTAs are shared out over the groups (together) its passes
+// leave a sum per tile and row, and these are then added in that order.
 struct GroupMember {
   BlockPlan* plan = nullptr;
   void* psi = nullptr;           // the chain's state
   long long* counter = nullptr;  // its period counter and energy ring
   double* ring = nullptr;
 };
-struct BlockGroup;
+struct BlockSet;
 bool block_same_structure(const BlockPlan* a, const BlockPlan* b);
-// Descriptors, operands and coefficients of every chain and pass, and the
-// group's own partial sums ([chains][slots][grid] pairs, zeroed: only CTAs
-// that meet a chain write its pairs).
-int block_group_build(const std::vector<GroupMember>& members, int ring_len,
-                      const LaunchCfg& cfg, cudaStream_t s, BlockGroup** out, std::string* msg);
-// Window of the group's periods (0: the natural layout, no entry steps).
-int block_group_start(const BlockGroup* g);
-// Chains in the group.
-size_t block_group_size(const BlockGroup* g);
-cudaError_t block_group_enqueue_entry(BlockGroup* g, cudaStream_t s);
-cudaError_t block_group_enqueue_period(BlockGroup* g, cudaStream_t s, bool last);
-void block_group_free(BlockGroup* g);
+// Whether these groups (chains of one structure each) are faster as one set than as a
+// set each.
+bool block_groups_together(const std::vector<std::vector<GroupMember>>& groups, const LaunchCfg& cfg);
+// Descriptors, operands and coefficients of every chain and pass, and the set's
+// own partial sums.
+int block_set_build(const std::vector<std::vector<GroupMember>>& groups, bool together, int ring_len,
+                    const LaunchCfg& cfg, cudaStream_t s, BlockSet** out, std::string* msg);
+// Chains in the set.
+size_t block_set_size(const BlockSet* set);
+// `periods` periods from and to the natural layout; alone: no other chains' passes
+// run beside them.
+cudaError_t block_set_enqueue(BlockSet* set, int periods, bool alone, cudaStream_t s);
+void block_set_free(BlockSet* set);
 
 // Nonzero if a tensor-core pass reported a timed-out wait (synchronises s).
 int block_status(BlockPlan* bp, cudaStream_t s);
@@ -164,11 +187,10 @@ int block_status(BlockPlan* bp, cudaStream_t s);
 cudaError_t launch_block_simt(const PassArgs& pa, void* psi, int grid, cudaStream_t s);
 cudaError_t launch_block_tc(const PassArgs& pa, void* psi, const void* map, int* status,
                             int grid, cudaStream_t s, bool overlap);
-// One tensor-core pass over the tiles of a chain group: pa is the pass's
-// structure with ntiles = chains x 2^nt_log2; chains: device array, one per
-// chain.  CTA b takes the contiguous tiles [b T / grid, (b + 1) T / grid).
-cudaError_t launch_block_tc_group(const PassArgs& pa, const GroupChain* chains, int nt_log2,
-                                  int* status, int grid, cudaStream_t s);
+// One tensor-core pass of each of n <= kGroupsPerLaunch groups: CTA b of a group's G
+// takes the contiguous tiles [b T / G, (b + 1) T / G) of its T = pa.ntiles.
+cudaError_t launch_block_tc_groups(const GroupPasses& passes, int n, int* status, bool overlap,
+                                   cudaStream_t s);
 bool block_tc_supported(int L, int n);
 cudaError_t block_tc_prepare();
 size_t block_tc_map_bytes();

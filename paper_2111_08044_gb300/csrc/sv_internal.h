@@ -39,8 +39,13 @@ void ctx_set_min_tiles(sv_ctx* ctx, int tiles);
 // Whether later block builds may start their periods off site 0 (the batch
 // replays captured periods back to back and needs the natural layout).
 void ctx_set_cyclic(sv_ctx* ctx, bool cyclic);
-// (energy density, norm) of periods c0 .. c0+count-1 from the energy ring.
-int ctx_read_energies(sv_ctx* ctx, int64_t c0, int64_t count, double* e, double* n);
+// Device energy ring of (energy density, norm) pairs, and the flag of its
+// tensor-core passes (null: it has none).
+struct RingSource {
+  const double* ring = nullptr;
+  const int* status = nullptr;
+};
+RingSource ctx_ring(const sv_ctx* ctx);
 // Periods the energy ring holds.
 int ctx_ring_len();
 struct BlockPlan;

@@ -131,7 +131,8 @@ struct ReduceItem {
   int ring_len = 0;
 };
 // The period reduce of `count` chains (items: device array), counters advanced.
-cudaError_t launch_period_reduce_many(const ReduceItem* items, int count, cudaStream_t s);
+cudaError_t launch_period_reduce_many(const ReduceItem* items, int count, bool overlap,
+                                      cudaStream_t s);
 cudaError_t launch_period_reduce(const double* partials, long long n, int L,
                                  double* ring, int ring_len, long long* counter,
                                  int advance, cudaStream_t s);

@@ -67,7 +67,7 @@ struct TilePassPlan {
 std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int precision, int tb,
                                     int max_gates = 0);
 // Tile size for a chain (0: the chain is too short for tiles).
-int tile_bits(int L, int precision, int num_sms);
+int tile_bits(int L, int precision, const LaunchCfg& cfg);
 int tile_threads(int precision, int tb);
 
 // A complex64 table entry g as the operands of packed FMAs: (gx, gx) and
