@@ -9,12 +9,12 @@
 //                   ceil((L - 12) / 8) + 1 times; one identity gate pass per
 //                   pair of sites read it L / 2 times: 1160 -> 194 us.
 //   k_moments_tile  H0 psi amplitude by amplitude, for E and sigma_E (Eq. 10 and
-//                   11): partners within the tile from registers and shared
+//   k_bond_moments_tile  11): partners within the tile from registers and shared
 //                   memory, the others from the tiles whose number differs in
 //                   one bit (or, for a general bond term, two), which mostly
 //                   are in L2.  Bound by that traffic: L - 11 tiles read for one
-//                   (Ising, 1230 -> 269 us), 2 (L - 12) (general bonds, L = 24:
-//                   1085 -> 330 us).
+//                   (Ising, 1230 -> 269 us); general bonds by instructions too
+//                   (L = 24: 1090 -> 393 us).
 //   k_overlap_f32   <phi|psi> of a product state from FP64 factor tables
 //   k_factor_f32    and the state itself: the FP64 units (0.59 TFMA/s) bounded
 //                   both; products and sums are FP32 pairs here (an exact
@@ -169,155 +169,186 @@ struct MomentArgs {
   float2 h[33][16] = {};        // general: bond terms
 };
 
-// One row of a bond term: out += sum_c h[r][c] w_c, w_c the amplitude with local
-// index c; r, like the amplitudes' order, only known at run time: the row's
-// entries are selected, not indexed.
-__device__ __forceinline__ float2 row_sum(const float2 (&h)[16], int r, float2 out, float2 same,
-                                          float2 lo, float2 hi, float2 both) {
-  // column r, r ^ 1 (site b + 1 flipped), r ^ 2 (site b flipped), r ^ 3
-  float2 d = h[0], l = h[1], u = h[2], x = h[3];
-  if (r == 1) d = h[5], l = h[4], u = h[7], x = h[6];
-  if (r == 2) d = h[10], l = h[11], u = h[8], x = h[9];
-  if (r == 3) d = h[15], l = h[14], u = h[13], x = h[12];
-  out = cmac(out, d, same);
-  out = cmac(out, l, lo);
-  out = cmac(out, u, hi);
-  return cmac(out, x, both);
+// Row r of a bond term as (h[r][r], h[r][r ^ 1], h[r][r ^ 2], h[r][r ^ 3]): the entries
+// of the amplitude itself, of its partners with site b + 1, site b and both flipped.
+// In shared memory: r is only known at run time.
+struct BondRow {
+  float4 a, b;
+};
+__device__ __forceinline__ float2 row_sum(const BondRow& h, float2 out, float2 same, float2 lo,
+                                          float2 hi, float2 both) {
+  out = cmac(out, make_float2(h.a.x, h.a.y), same);
+  out = cmac(out, make_float2(h.a.z, h.a.w), lo);
+  out = cmac(out, make_float2(h.b.x, h.b.y), hi);
+  return cmac(out, make_float2(h.b.z, h.b.w), both);
 }
 
-// A thread's amplitudes: tile indices 2 tid + (0, 1) + 1024 j, j = 0..3 (bit 0 of
-// m: site 0, bits 1 and 2: sites 10 and 11), so that every read of another tile
+// A thread's kA amplitudes of a tile of 2^kB: indices 2 tid + (0, 1) + 1024 j (bit 0
+// of m: site 0, the bits above: sites 10 and on), so that every read of another tile
 // is of whole lines; sites 1..9 are thread bits, their partners in the tile.
-// General bond terms hold four arrays of partners: one block an SM.
 constexpr int kMomentThreads = 512;
-constexpr int kAmps = 8;
-
-template <bool kBonds>
-__global__ void __launch_bounds__(kMomentThreads, kBonds ? 1 : 2)
-    k_moments_tile(const float2* __restrict__ psi, const __grid_constant__ MomentArgs ma,
-                   double* __restrict__ part) {
-  extern __shared__ __align__(16) uint8_t tile[];
-  const int L = ma.L;
-  const uint32_t ntiles = 1u << (L - kBits);
-  const uint32_t tid = threadIdx.x;
-  TileDiag dg;
-  if (!kBonds) dg.init(ma.ep, L);
-  double acc[3] = {0.0, 0.0, 0.0};
-  const uint32_t e0 = 2 * tid;
-  auto set = [](float2 (&u)[kAmps], int j, float4 q) {
+template <int kA>
+struct MomentTile {
+  static constexpr int kB = kA == 8 ? 12 : 11;  // tile bits
+  uint8_t* tile;
+  const float2* psi;
+  uint32_t tid;
+  __device__ __forceinline__ void set(float2 (&u)[kA], int j, float4 q) const {
     u[2 * j] = make_float2(q.x, q.y);
     u[2 * j + 1] = make_float2(q.z, q.w);
-  };
-  auto read = [&](uint32_t from, float2 (&u)[kAmps]) {
-    const float4* p = reinterpret_cast<const float4*>(psi + ((uint64_t)from << kBits));
+  }
+  __device__ __forceinline__ void read(uint32_t from, float2 (&u)[kA]) const {
+    const float4* p = reinterpret_cast<const float4*>(psi + ((uint64_t)from << kB));
 #pragma unroll
-    for (int j = 0; j < kAmps / 2; ++j) set(u, j, __ldg(p + tid + kMomentThreads * j));
-  };
-  auto partner = [&](uint32_t flip, float2 (&u)[kAmps]) {  // flip: tile bits 1..9
+    for (int j = 0; j < kA / 2; ++j) set(u, j, __ldg(p + tid + kMomentThreads * j));
+  }
+  __device__ __forceinline__ void put(const float2 (&v)[kA]) const {
 #pragma unroll
-    for (int j = 0; j < kAmps / 2; ++j)
-      set(u, j, *reinterpret_cast<const float4*>(tile + tile_byte8((e0 ^ flip) + 1024 * j)));
-  };
-  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    float2 v[kAmps], hv[kAmps], a[kAmps];
-    read(t, v);
-#pragma unroll
-    for (int j = 0; j < kAmps / 2; ++j)
-      *reinterpret_cast<float4*>(tile + tile_byte8(e0 + 1024 * j)) =
+    for (int j = 0; j < kA / 2; ++j)
+      *reinterpret_cast<float4*>(tile + tile_byte8(2 * tid + 1024 * j)) =
           make_float4(v[2 * j].x, v[2 * j].y, v[2 * j + 1].x, v[2 * j + 1].y);
-    __syncthreads();
-    if (!kBonds) {
-      dg.tile(t);
-      auto add = [&](float c, const float2 (&u)[kAmps]) {
+  }
+  __device__ __forceinline__ void partner(uint32_t flip, float2 (&u)[kA]) const {  // flip: bits 1..9
 #pragma unroll
-        for (int m = 0; m < kAmps; ++m) {
-          hv[m].x += c * u[m].x;
-          hv[m].y += c * u[m].y;
-        }
-      };
-#pragma unroll
-      for (int m = 0; m < kAmps; ++m) {
-        const float d = dg(e0 + 1024 * (m >> 1) + (m & 1));
-        hv[m] = make_float2(d * v[m].x, d * v[m].y);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {  // sites 0, 10, 11: within the thread
-          const float c = ma.cx[k == 0 ? 0 : 9 + k];
-          hv[m].x += c * v[m ^ (1 << k)].x;
-          hv[m].y += c * v[m ^ (1 << k)].y;
-        }
-      }
-#pragma unroll
-      for (int i = 1; i < 10; ++i) {
-        partner(1u << i, a);
-        add(ma.cx[i], a);
-      }
-#pragma unroll 4
-      for (int i = kBits; i < L; ++i) {
-        read(t ^ (1u << (i - kBits)), a);
-        add(ma.cx[i], a);
-      }
-    } else {
-      float2 b[kAmps], c[kAmps];
-      // (10, 11): within the thread
-#pragma unroll
-      for (int m = 0; m < kAmps; ++m) {
-        const int r = 2 * ((m >> 1) & 1) + (m >> 2);
-        hv[m] = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          hv[m] = cmac(hv[m], ma.h[10][4 * r + q], v[(m & 1) | ((q >> 1) << 1) | ((q & 1) << 2)]);
-      }
-      // (0, 1)
-      partner(2, a);
-      const int s1 = tid & 1;
-#pragma unroll
-      for (int m = 0; m < kAmps; ++m)
-        hv[m] = row_sum(ma.h[0], 2 * (m & 1) + s1, hv[m], v[m], a[m], v[m ^ 1], a[m ^ 1]);
-      // (i, i + 1), i = 1..8: both thread bits; a holds site i's partner
-#pragma unroll 1
-      for (int i = 1; i < 9; ++i) {
-        partner(2u << i, b);
-        partner(3u << i, c);
-        const int r = 2 * (int)((tid >> (i - 1)) & 1) + (int)((tid >> i) & 1);
-#pragma unroll
-        for (int m = 0; m < kAmps; ++m) {
-          hv[m] = row_sum(ma.h[i], r, hv[m], v[m], b[m], a[m], c[m]);
-          a[m] = b[m];
-        }
-      }
-      // (9, 10)
-      const int s9 = (int)(tid >> 8);
-#pragma unroll
-      for (int m = 0; m < kAmps; ++m)
-        hv[m] = row_sum(ma.h[9], 2 * s9 + ((m >> 1) & 1), hv[m], v[m], v[m ^ 2], a[m], a[m ^ 2]);
-      // (11, 12): site 12 is the tile number's bit 0
-      read(t ^ 1u, a);
-      const int s12 = (int)(t & 1u);
-#pragma unroll
-      for (int m = 0; m < kAmps; ++m)
-        hv[m] = row_sum(ma.h[11], 2 * (m >> 2) + s12, hv[m], v[m], a[m], v[m ^ 4], a[m ^ 4]);
-#pragma unroll 1
-      for (int i = kBits; i + 1 < L; ++i) {  // a holds site i's partner
-        const uint32_t bit = 1u << (i - kBits);
-        read(t ^ (2 * bit), b);
-        read(t ^ (3 * bit), c);
-        const int r = 2 * (int)((t & bit) != 0) + (int)((t & (2 * bit)) != 0);
-#pragma unroll
-        for (int m = 0; m < kAmps; ++m) {
-          hv[m] = row_sum(ma.h[i], r, hv[m], v[m], b[m], a[m], c[m]);
-          a[m] = b[m];
-        }
-      }
-    }
+    for (int j = 0; j < kA / 2; ++j)
+      set(u, j, *reinterpret_cast<const float4*>(tile + tile_byte8(((2 * tid) ^ flip) + 1024 * j)));
+  }
+  // <psi|H0|psi>, |H0 psi|^2 and the norm
+  __device__ __forceinline__ static void sums(const float2 (&v)[kA], const float2 (&hv)[kA],
+                                              double (&acc)[3]) {
     FloatSum s[3];
 #pragma unroll
-    for (int m = 0; m < kAmps; ++m) {
+    for (int m = 0; m < kA; ++m) {
       s[0].add(v[m].x * hv[m].x + v[m].y * hv[m].y);
       s[1].add(hv[m].x * hv[m].x + hv[m].y * hv[m].y);
       s[2].add(v[m].x * v[m].x + v[m].y * v[m].y);
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) s[k].flush(acc[k]);
+  }
+};
+
+__global__ void __launch_bounds__(kMomentThreads, 2)
+    k_moments_tile(const float2* __restrict__ psi, const __grid_constant__ MomentArgs ma,
+                   double* __restrict__ part) {
+  extern __shared__ __align__(16) uint8_t tile[];
+  constexpr int kA = 8;
+  const int L = ma.L;
+  const uint32_t ntiles = 1u << (L - kBits);
+  const MomentTile<kA> mt{tile, psi, threadIdx.x};
+  const uint32_t e0 = 2 * threadIdx.x;
+  TileDiag dg;
+  dg.init(ma.ep, L);
+  double acc[3] = {0.0, 0.0, 0.0};
+  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    float2 v[kA], hv[kA], a[kA];
+    mt.read(t, v);
+    mt.put(v);
+    __syncthreads();
+    dg.tile(t);
+    auto add = [&](float c, const float2 (&u)[kA]) {
+#pragma unroll
+      for (int m = 0; m < kA; ++m) {
+        hv[m].x += c * u[m].x;
+        hv[m].y += c * u[m].y;
+      }
+    };
+#pragma unroll
+    for (int m = 0; m < kA; ++m) {
+      const float d = dg(e0 + 1024 * (m >> 1) + (m & 1));
+      hv[m] = make_float2(d * v[m].x, d * v[m].y);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {  // sites 0, 10, 11: within the thread
+        const float c = ma.cx[k == 0 ? 0 : 9 + k];
+        hv[m].x += c * v[m ^ (1 << k)].x;
+        hv[m].y += c * v[m ^ (1 << k)].y;
+      }
+    }
+#pragma unroll
+    for (int i = 1; i < 10; ++i) {
+      mt.partner(1u << i, a);
+      add(ma.cx[i], a);
+    }
+#pragma unroll 4
+    for (int i = kBits; i < L; ++i) {
+      mt.read(t ^ (1u << (i - kBits)), a);
+      add(ma.cx[i], a);
+    }
+    MomentTile<kA>::sums(v, hv, acc);
+    __syncthreads();
+  }
+  block_store_k<3>(acc, part);
+}
+
+// General bond terms hold four arrays of partners, so tiles of 2^11: 64 registers a
+// thread, two blocks an SM.  Bound by instructions: 16 FMA an amplitude and bond (L =
+// 24: 168 us at the pipe's rate) beside the partners' loads; two rows of the term come
+// from shared memory (entries selected from the parameters took as many again).
+// 393 us at L = 24; 590 us so, and in tiles of 2^12 and one block an SM 750 us.
+__global__ void __launch_bounds__(kMomentThreads, 2)
+    k_bond_moments_tile(const float2* __restrict__ psi, const __grid_constant__ MomentArgs ma,
+                        double* __restrict__ part) {
+  extern __shared__ __align__(16) uint8_t tile[];
+  __shared__ BondRow rows[33][4];
+  constexpr int kA = 4, kB = MomentTile<kA>::kB;
+  const int L = ma.L;
+  const uint32_t ntiles = 1u << (L - kB);
+  const uint32_t tid = threadIdx.x;
+  const MomentTile<kA> mt{tile, psi, tid};
+  for (uint32_t q = tid; q < 16u * (L - 1); q += kMomentThreads) {
+    const uint32_t r = (q >> 2) & 3, c = q & 3;
+    reinterpret_cast<float2*>(rows)[q] = ma.h[q >> 4][4 * r + (r ^ c)];
+  }
+  double acc[3] = {0.0, 0.0, 0.0};
+  for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    float2 v[kA], hv[kA], a[kA], b[kA], c[kA];
+    mt.read(t, v);
+    mt.put(v);
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < kA; ++m) hv[m] = make_float2(0.f, 0.f);
+    // (0, 1)
+    mt.partner(2, a);
+    const int s1 = tid & 1;
+#pragma unroll
+    for (int m = 0; m < kA; ++m)
+      hv[m] = row_sum(rows[0][2 * (m & 1) + s1], hv[m], v[m], a[m], v[m ^ 1], a[m ^ 1]);
+    // (i, i + 1), i = 1..8: both thread bits; a holds site i's partner
+#pragma unroll 1
+    for (int i = 1; i < 9; ++i) {
+      mt.partner(2u << i, b);
+      mt.partner(3u << i, c);
+      const BondRow h = rows[i][2 * ((tid >> (i - 1)) & 1) + ((tid >> i) & 1)];
+#pragma unroll
+      for (int m = 0; m < kA; ++m) {
+        hv[m] = row_sum(h, hv[m], v[m], b[m], a[m], c[m]);
+        a[m] = b[m];
+      }
+    }
+    // (9, 10)
+    const int s9 = (int)(tid >> 8);
+#pragma unroll
+    for (int m = 0; m < kA; ++m)
+      hv[m] = row_sum(rows[9][2 * s9 + (m >> 1)], hv[m], v[m], v[m ^ 2], a[m], a[m ^ 2]);
+    // (10, 11): site 11 is the tile number's bit 0
+    mt.read(t ^ 1u, a);
+    const int s11 = (int)(t & 1u);
+#pragma unroll
+    for (int m = 0; m < kA; ++m)
+      hv[m] = row_sum(rows[10][2 * (m >> 1) + s11], hv[m], v[m], a[m], v[m ^ 2], a[m ^ 2]);
+#pragma unroll 2
+    for (int i = kB; i + 1 < L; ++i) {  // a holds site i's partner
+      const uint32_t at = i - kB;
+      mt.read(t ^ (2u << at), b);
+      mt.read(t ^ (3u << at), c);
+      const BondRow h = rows[i][2 * ((t >> at) & 1) + ((t >> (at + 1)) & 1)];
+#pragma unroll
+      for (int m = 0; m < kA; ++m) {
+        hv[m] = row_sum(h, hv[m], v[m], b[m], a[m], c[m]);
+        a[m] = b[m];
+      }
+    }
+    MomentTile<kA>::sums(v, hv, acc);
     __syncthreads();
   }
   block_store_k<3>(acc, part);
@@ -468,8 +499,8 @@ cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h, const E
       ma.h[b][k] = make_float2((float)bonds[16 * b + k].real(), (float)bonds[16 * b + k].imag());
   const int grid = observe_moments_grid(L, cfg);
   const float2* p = static_cast<const float2*>(psi);
-  if (bonds) k_moments_tile<true><<<grid, kMomentThreads, kTileBytes, s>>>(p, ma, part);
-  else k_moments_tile<false><<<grid, kMomentThreads, kTileBytes, s>>>(p, ma, part);
+  if (bonds) k_bond_moments_tile<<<grid, kMomentThreads, kTileBytes / 2, s>>>(p, ma, part);
+  else k_moments_tile<<<grid, kMomentThreads, kTileBytes, s>>>(p, ma, part);
   return cudaGetLastError();
 }
 
