@@ -196,14 +196,20 @@ __device__ __forceinline__ void run_round(const ResidentRound& rd, const PackedE
   };
   if (kPlain && rd.xorder[0]) gate16<0, 1, 2, 3, true>(v, from(ga));
   else gate16<0, 1, 2, 3, false>(v, from(ga));
-  if (kPlain && rd.epi[0] && rd.sweep != 1)
-    measure16<0, 1, 2, 3>(v, ch.L, ch.cx, ch.ep, rd, 0, e0, active, esum, nsum);
+  // <X> in pairs (of a measured gate most often) has its own, shorter code
+  auto pairs = [&](int k) { return rd.egroup[k] == TILE_E_PAIR && !(rd.epi[k] & EPI_DIAG); };
+  if (kPlain && rd.epi[0] && rd.sweep != 1) {
+    if (pairs(0)) measure16_x<0, 1, 2, 3>(v, ch.cx, rd, 0, active, esum);
+    else measure16<0, 1, 2, 3>(v, ch.L, ch.cx, ch.ep, rd, 0, e0, active, esum, nsum);
+  }
   if (rd.count == 2) {
     const PackedEntry* gb = ga + kGateEntries;
     if (kPlain && rd.xorder[1]) gate16<2, 3, 0, 1, true>(v, from(gb));
     else gate16<2, 3, 0, 1, false>(v, from(gb));
-    if (kPlain && rd.epi[1] && rd.sweep != 2)
-      measure16<2, 3, 0, 1>(v, ch.L, ch.cx, ch.ep, rd, 1, e0, active, esum, nsum);
+    if (kPlain && rd.epi[1] && rd.sweep != 2) {
+      if (pairs(1)) measure16_x<2, 3, 0, 1>(v, ch.cx, rd, 1, active, esum);
+      else measure16<2, 3, 0, 1>(v, ch.L, ch.cx, ch.ep, rd, 1, e0, active, esum, nsum);
+    }
   }
   if (active) {
 #pragma unroll

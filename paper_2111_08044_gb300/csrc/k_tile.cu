@@ -9,9 +9,9 @@
 // bytes of traffic, so a pass of one gate is bound by HBM, and on a short
 // chain by its launch and the latency of its loads (2.85 us a gate at L = 12,
 // 0.55 us of it the launch).  With four to six gates a pass the FP32 pipe is
-// the bound.  A pass of four gates at L = 27 takes 588 us (467 us of FMAs at
+// the bound.  A pass of four gates at L = 27 takes 580 us (467 us of FMAs at
 // the pipe's 36.8 TFMA/s), where four passes of one gate take 1350 us; a period
-// 17.9 ms (104 gates), before 35.2 ms, at L = 20 0.18 ms for 0.39 ms.  Chains of
+// 16.6 ms (104 gates), before 35.2 ms, at L = 20 0.17 ms for 0.39 ms.  Chains of
 // up to 15 sites stay in shared memory between periods instead (k_resident.cu).
 //
 // complex64 (k_tile_f32): a thread holds 16 amplitudes (four register bits
@@ -106,9 +106,11 @@ __device__ __forceinline__ void load_packed(const TileArgs& ta, PackedEntry* gs,
 
 // kSlots > 0: tables and rounds in the parameters; 0: in device memory, copied
 // to shared memory (per-period tables, and passes that scale the first gate).
-// kXor, kEpi: the pass has gates in the order r ^ j / measured gates; passes
-// without them run less code.
-template <int kSlots, bool kXor, bool kEpi, int kThreads, int kMinBlocks>
+// kXor: the pass has gates in the order r ^ j; kEpi: measured gates (1: <X> terms
+// only); passes without them run less code.  <X> alone fits three blocks an SM as
+// unmeasured gates do: the last layer's four passes at L = 27 took 5.1 ms with one
+// instance for all measured gates (two blocks), 4.1 ms with this one.
+template <int kSlots, bool kXor, int kEpi, int kThreads, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks)
     k_tile_f32(float2* __restrict__ psi, const __grid_constant__ TileArgs ta,
                const __grid_constant__ TileTabOf<kSlots ? kSlots : 1> tab) {
@@ -166,13 +168,17 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
       };
       if (kXor && rd.xorder[0]) gate16<0, 1, 2, 3, true>(v, from(ga));
       else gate16<0, 1, 2, 3, false>(v, from(ga));
-      if (kEpi && rd.epi[0] && rd.egroup[0] != TILE_E_SWEEP)
+      if (kEpi == 1 && rd.epi[0] && rd.egroup[0] != TILE_E_SWEEP)
+        measure16_x<0, 1, 2, 3>(v, ta.cx, rd, 0, active, esum);
+      if (kEpi == 2 && rd.epi[0] && rd.egroup[0] != TILE_E_SWEEP)
         measure16<0, 1, 2, 3>(v, ta.L, ta.cx, ta.ep, rd, 0, tbase + elem_state(ta, e0), active, esum,
                               nsum);
       if (rd.count == 2) {
         if (kXor && rd.xorder[1]) gate16<2, 3, 0, 1, true>(v, from(gb));
         else gate16<2, 3, 0, 1, false>(v, from(gb));
-        if (kEpi && rd.epi[1] && rd.egroup[1] != TILE_E_SWEEP)
+        if (kEpi == 1 && rd.epi[1] && rd.egroup[1] != TILE_E_SWEEP)
+          measure16_x<2, 3, 0, 1>(v, ta.cx, rd, 1, active, esum);
+        if (kEpi == 2 && rd.epi[1] && rd.egroup[1] != TILE_E_SWEEP)
           measure16<2, 3, 0, 1>(v, ta.L, ta.cx, ta.ep, rd, 1, tbase + elem_state(ta, e0), active, esum,
                                 nsum);
       }
@@ -197,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks)
       if (kEpi) {
         const int sw = rd.egroup[1] == TILE_E_SWEEP ? 1 : rd.egroup[0] == TILE_E_SWEEP ? 0 : -1;
         if (sw >= 0) {
-          measure_sweep(tile, ta.tb, ta.L, ta.cx, ta.ep, rd.bond[sw], rd.epi[sw],
+          measure_sweep<kEpi == 2>(tile, ta.tb, ta.L, ta.cx, ta.ep, rd.bond[sw], rd.epi[sw],
                         [&](uint32_t e) { return tbase + elem_state(ta, e); }, esum, nsum);
           __syncthreads();
         }
@@ -529,13 +535,15 @@ const void* tile_kernel(int precision, const TileArgs& ta) {
     return ta.in_params   ? reinterpret_cast<const void*>(k_tile_df<kTileTabSlots, 3>)
            : ta.tb < ta.L ? reinterpret_cast<const void*>(k_tile_df<0, 3>)
                           : reinterpret_cast<const void*>(k_tile_df<0, 1>);
+  const int epi = !ta.any_epi ? 0 : (ta.any_epi & EPI_DIAG) ? 2 : 1;
   if (!ta.in_params)
-    return ta.any_epi      ? reinterpret_cast<const void*>(k_tile_f32<0, true, true, 256, 2>)
-           : ta.any_xorder ? reinterpret_cast<const void*>(k_tile_f32<0, true, false, 256, 2>)
-                           : reinterpret_cast<const void*>(k_tile_f32<0, false, false, 256, 2>);
-  if (ta.any_epi) return reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, true, 256, 2>);
-  return ta.any_xorder ? reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, false, 256, 3>)
-                       : reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, false, false, 256, 3>);
+    return epi             ? reinterpret_cast<const void*>(k_tile_f32<0, true, 2, 256, 2>)
+           : ta.any_xorder ? reinterpret_cast<const void*>(k_tile_f32<0, true, 0, 256, 2>)
+                           : reinterpret_cast<const void*>(k_tile_f32<0, false, 0, 256, 2>);
+  if (epi == 2) return reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, 2, 256, 2>);
+  if (epi == 1) return reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, 1, 256, 3>);
+  return ta.any_xorder ? reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, true, 0, 256, 3>)
+                       : reinterpret_cast<const void*>(k_tile_f32<kTileTabSlots, false, 0, 256, 3>);
 }
 
 }  // namespace

@@ -274,45 +274,72 @@ __device__ __forceinline__ void measure16(const uint64_t (&v)[16], int L, const 
   }
 }
 
+// The same of a gate that measures <X> only, in neighbouring pairs (TILE_E_PAIR): a
+// term that is not measured has the coefficient 0.
+template <int J0, int J1, int K0, int K1, typename Round>
+__device__ __forceinline__ void measure16_x(const uint64_t (&v)[16], const float* cx, const Round& rd,
+                                            int which, bool active, FloatSum& esum) {
+  const int epi = rd.epi[which], bond = rd.bond[which];
+  const float ch = (epi & EPI_X_HI) ? cx[bond] * 2.f : 0.f;
+  const float cl = (epi & EPI_X_LO) ? cx[bond + 1] * 2.f : 0.f;
+  const bool take = active && (threadIdx.x & 1);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float2 w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      w[r] = un2(v[((r >> 1) << J0) | ((r & 1) << J1) | ((k & 1) << K0) | ((k >> 1) << K1)]);
+    const float hi = cdotre(w[0], w[2]) + cdotre(w[1], w[3]);
+    const float lo = cdotre(w[0], w[1]) + cdotre(w[2], w[3]);
+    const float es = __fmaf_rn(cl, lo, __fmaf_rn(ch, hi, 0.f));
+    const float e2 = __shfl_xor_sync(0xffffffffu, es, 1);
+    const float s = __fmaf_rn(cl, lo, __fmaf_rn(ch, hi, e2));
+    if (take) esum.add(s);
+  }
+}
+
 // A measured gate on bonds 0..5 of a chain of at least 8 sites, from the tile:
 // the sums of the per-gate kernel, whose threads hold bits 0, 6 and 7.
 // state(e): state index of tile index e; 2^tb amplitudes in the tile.
-template <typename S>
+template <bool kDiag = true, typename S>
 __device__ __forceinline__ void measure_sweep(const uint8_t* tile, int tb, int L, const float* cx,
                                               const EpiParams& ep, int bond, int epi, const S& state,
                                               FloatSum& esum, FloatSum& nsum) {
   const float cxh = cx[bond], cxl = cx[bond + 1];
   Diag<float> dg;
-  if (epi & EPI_DIAG) dg.init(ep, L);
+  if (kDiag && (epi & EPI_DIAG)) dg.init(ep, L);
   const uint32_t nv = 1u << (tb - 3);
-  auto at = [&](uint32_t e) { return *reinterpret_cast<const float2*>(tile + tile_byte8(e)); };
+  // amplitudes e and e + 1 (e even)
+  auto at = [&](uint32_t e) { return *reinterpret_cast<const float4*>(tile + tile_byte8(e)); };
   for (uint32_t vt = threadIdx.x; vt < nv; vt += blockDim.x) {
     const uint32_t e0 = ((vt & 31u) << 1) | ((vt >> 5) << 8);
     float2 w[4][2];
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int k = 0; k < 2; ++k) w[c][k] = at(e0 | (c << 6) | k);
+    for (int c = 0; c < 4; ++c) {
+      const float4 q = at(e0 | (c << 6));
+      w[c][0] = make_float2(q.x, q.y);
+      w[c][1] = make_float2(q.z, q.w);
+    }
     float es = 0.f, ns = 0.f;
-    if (epi & EPI_X_HI) {
+    // sum over the thread's amplitudes of the products with site bit `flip` flipped
+    auto pairs = [&](uint32_t flip) {
       float s = 0.f;
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+      for (int c = 0; c < 4; ++c) {
+        float2 u[2] = {w[c][1], w[c][0]};
+        if (flip > 1) {
+          const float4 q = at((e0 | (c << 6)) ^ flip);
+          u[0] = make_float2(q.x, q.y);
+          u[1] = make_float2(q.z, q.w);
+        }
 #pragma unroll
-        for (int k = 0; k < 2; ++k)
-          s += cdotre(w[c][k], at((e0 | (c << 6) | k) ^ (1u << bond)));
-      es += cxh * s;
-    }
-    if (epi & EPI_X_LO) {
-      float s = 0.f;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-          s += cdotre(w[c][k], at((e0 | (c << 6) | k) ^ (2u << bond)));
-      es += cxl * s;
-    }
-    if (epi & EPI_DIAG) {
+        for (int k = 0; k < 2; ++k) s += cdotre(w[c][k], u[k]);
+      }
+      return s;
+    };
+    if (epi & EPI_X_HI) es += cxh * pairs(1u << bond);
+    if (epi & EPI_X_LO) es += cxl * pairs(2u << bond);
+    if (kDiag && (epi & EPI_DIAG)) {
       const uint64_t x0 = state(e0);
 #pragma unroll
       for (int c = 0; c < 4; ++c)
@@ -324,7 +351,7 @@ __device__ __forceinline__ void measure_sweep(const uint8_t* tile, int tb, int L
         }
     }
     esum.add(es);
-    if (epi & EPI_DIAG) nsum.add(ns);
+    if (kDiag && (epi & EPI_DIAG)) nsum.add(ns);
   }
 }
 
