@@ -93,6 +93,43 @@ struct TileDiag {
   }
 };
 
+// The same as an FP32 pair, from tables of its two counts: J (L - 1 - 2 flips), and the
+// fields' sum for nb set bits between the ends and the two end bits.  A value of 20
+// rounded to FP32 is off by up to 1e-6, the same for every amplitude of its counts,
+// which does not average out of a sum near zero.
+struct PairDiag {
+  const float2 *zz, *field;  // shared memory: 34, and 4 a count
+  int L, nb_hi, flips_hi, last;
+  uint32_t top;
+  __device__ static void fill(const H0Coef& h, int L, float2* zz, float2* field) {
+    auto pair = [](double v) {
+      const float hi = (float)v;
+      return make_float2(hi, (float)(v - (double)hi));
+    };
+    const int k = threadIdx.x;
+    if (k < L) zz[k] = pair(h.J * (L - 1 - 2 * k));
+    if (k < 4 * (L - 1)) {
+      const int nb = k >> 2;
+      field[k] = pair(h.cz[1] * (L - 2 - 2 * nb) + ((k & 2) ? -h.cz[0] : h.cz[0]) +
+                      ((k & 1) ? -h.cz[L - 1] : h.cz[L - 1]));
+    }
+  }
+  __device__ void tile(uint32_t t) {
+    const int hi = L - kBits;  // bits of the tile number, at least 1
+    flips_hi = __popc((t ^ (t >> 1)) & ((1u << (hi - 1)) - 1));
+    last = (t >> (hi - 1)) & 1;
+    nb_hi = __popc(t) - last;
+    top = (t & 1u) << kBits;
+  }
+  __device__ __forceinline__ df operator()(uint32_t e) const {
+    const uint32_t x = e | top;
+    const float2 a = zz[flips_hi + __popc((x ^ (x >> 1)) & ((1u << kBits) - 1))];
+    const float2 b = field[4 * (nb_hi + __popc(e & ~1u)) + 2 * (e & 1) + last];
+    const df s = two_sum(a.x, b.x);
+    return df(s.hi, s.lo + (a.y + b.y));
+  }
+};
+
 struct EnergyArgs {
   TileArgs ta;          // layout of the pass
   float cx[kBits] = {};  // coefficient of each tile bit's <X> (0: another pass's)
@@ -165,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 struct MomentArgs {
   int L = 0;
   float cx[34] = {};            // Ising: coefficients of X_i
-  EpiParams ep;                 // Ising: diagonal coefficients
+  H0Coef h0;                    // Ising: diagonal coefficients (cz of sites 1..L-2 equal)
   float2 h[33][16] = {};        // general: bond terms
 };
 
@@ -237,8 +274,10 @@ __global__ void __launch_bounds__(kMomentThreads, 2)
   const uint32_t ntiles = 1u << (L - kBits);
   const MomentTile<kA> mt{tile, psi, threadIdx.x};
   const uint32_t e0 = 2 * threadIdx.x;
-  TileDiag dg;
-  dg.init(ma.ep, L);
+  __shared__ float2 zz[34], field[4 * 33];
+  PairDiag::fill(ma.h0, L, zz, field);
+  PairDiag dg{zz, field, L};
+  __syncthreads();
   double acc[3] = {0.0, 0.0, 0.0};
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     float2 v[kA], hv[kA], a[kA];
@@ -255,8 +294,8 @@ __global__ void __launch_bounds__(kMomentThreads, 2)
     };
 #pragma unroll
     for (int m = 0; m < kA; ++m) {
-      const float d = dg(e0 + 1024 * (m >> 1) + (m & 1));
-      hv[m] = make_float2(d * v[m].x, d * v[m].y);
+      const df d = dg(e0 + 1024 * (m >> 1) + (m & 1));
+      hv[m] = make_float2(__fmaf_rn(d.lo, v[m].x, d.hi * v[m].x), __fmaf_rn(d.lo, v[m].y, d.hi * v[m].y));
 #pragma unroll
       for (int k = 0; k < 3; ++k) {  // sites 0, 10, 11: within the thread
         const float c = ma.cx[k == 0 ? 0 : 9 + k];
@@ -487,12 +526,11 @@ cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, const Ep
 
 int observe_moments_grid(int L, const LaunchCfg& cfg) { return grid_of(L, cfg, 2); }
 
-cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h, const EpiParams& diag,
-                                const cd* bonds, double* part, const LaunchCfg& cfg,
+cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h, const cd* bonds, double* part, const LaunchCfg& cfg,
                                 cudaStream_t s) {
   MomentArgs ma;
   ma.L = L;
-  ma.ep = diag;
+  ma.h0 = h;
   for (int i = 0; i < L; ++i) ma.cx[i] = (float)h.cx[i];
   for (int b = 0; bonds && b + 1 < L; ++b)
     for (int k = 0; k < 16; ++k)

@@ -647,7 +647,6 @@ int energy_moments(sv_ctx* ctx, double* energy, double* sigma_e, double* norm2) 
   cudaError_t e = cudaSuccess;
   if (tiles) {
     e = fsv::launch_moments_tile(ctx->state, ctx->L, h0_coef(ctx),
-                                 epi_for(ctx, ctx->obs.general ? 0 : fsv::EPI_DIAG, 0, nullptr),
                                  ctx->obs.general ? ctx->obs.h.data() : nullptr, d_part, ctx->cfg,
                                  ctx->stream);
   } else if (ctx->obs.general) {

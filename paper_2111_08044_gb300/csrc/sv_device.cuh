@@ -21,7 +21,6 @@ __device__ __forceinline__ void grid_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-
 template <typename R>
 struct CT;
 template <>

@@ -187,7 +187,7 @@ cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, const Ep
                                double* part, const LaunchCfg& cfg, cudaStream_t s);
 // bonds: general bond terms on the host ((L - 1) x 16), or NULL for the Ising chain
 int observe_moments_grid(int L, const LaunchCfg& cfg);
-cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h, const EpiParams& diag,
+cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h,
                                 const std::complex<double>* bonds, double* part,
                                 const LaunchCfg& cfg, cudaStream_t s);
 int observe_overlap_grid(int L, const LaunchCfg& cfg);

@@ -58,3 +58,21 @@ def test_pair_states_and_bond_moments_match_oracle(svlib, L):
     assert abs(E - Eo) < tol and abs(n - no) < 2e-7
     assert abs(s * s - so * so) < 2 * 3 * L * tol
     assert abs(ov - np.vdot(ref, psi)) < 1e-13
+
+
+@pytest.mark.parametrize("L,hz,ew", [(13, 0.57, 0.5), (16, 0.31, 1.0), (24, 0.57, 0.5), (25, 0.43, 1.0)])
+def test_moments_of_a_sum_near_zero(svlib, L, hz, ew):
+    """|+>^L without a transverse field: the diagonal energies, of up to L (1 + hz),
+    cancel to E = 0, and sigma_E^2 = (L - 1) J^2 + sum_i cz_i^2."""
+    from paper_2111_08044_gb300.sim import FloquetSimulator, chain_params
+    cfg = inputs.ChainConfig(L=L, J=0.93, hx=0.0, hz=hz, edge_field_weight=ew, seed=1)
+    with FloquetSimulator(L) as sim:
+        sim.init_product_state(np.tile([np.sqrt(0.5), 0.0], (L, 2)))
+        sim.build(**chain_params(cfg))
+        e, s, _ = sim.energy_moments()
+    # four roundings of 2^-24 an amplitude on terms d p, |d| <= L (1 + hz), independent
+    # over 2^L amplitudes of p = 2^-L: six standard deviations
+    tol = 6 * 4 * 2.0 ** -24 * L * (1 + hz) * 2.0 ** (-L / 2)
+    assert abs(e) < tol
+    var = (L - 1) * 0.93 ** 2 + hz ** 2 * (L - 2 + 2 * ew ** 2)
+    assert abs(s / np.sqrt(var) - 1) < 8 * 2.0 ** -24
