@@ -4,7 +4,7 @@
 One step = one Floquet period of the whole hot path: K=4 Trotter steps of
 even/odd brickwork gates plus the folded X kick, and the energy density /
 norm measurement of that period.  The tensor-core block form is the headline;
-the plain per-gate form is timed beside it.  Inputs: a seeded random product
+the plain form is timed beside it.  Inputs: a seeded random product
 state of 30 sites (8 GiB state, far larger than L2, so no flush is needed).
 
     python bench.py [--steps K] [--warmup W] [--impl ours|reference]

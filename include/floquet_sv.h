@@ -205,7 +205,7 @@ int sv_expect_energy(sv_ctx *ctx, double *energy_density, double *norm2);
  * energy itself, not per site), and norm2 = <psi|psi>; any output may be
  * NULL.  <H0^2> = |H0 psi|^2 is accumulated with H0 psi formed amplitude by
  * amplitude from each amplitude's L bit-flip neighbours: no second state is
- * held, and the state is read about L + 1 times.  Errors: SV_ESTATE,
+ * held.  Errors: SV_ESTATE,
  * SV_ECUDA.
  */
 int sv_energy_moments(sv_ctx *ctx, double *energy, double *sigma_e, double *norm2);
@@ -307,8 +307,10 @@ int sv_set_layout_policy(sv_ctx *ctx, int keep_period_layout);
 int64_t sv_period_counter(const sv_ctx *ctx);
 
 /*
- * Kernel passes over the state per period and two-qubit gates per period
- * of the built evolution (for throughput accounting).  Errors: SV_ESTATE.
+ * Kernel passes over the state and two-qubit gates per period of the built
+ * evolution, and its launches (for throughput accounting).  A pass of the plain
+ * form holds several gates; a chain that stays in shared memory counts one pass
+ * and one launch a period, of which a call runs many in one.  Errors: SV_ESTATE.
  */
 int sv_pass_info(const sv_ctx *ctx, int *passes_per_period, int *gates_per_period,
                  int *launches_per_period);
@@ -474,11 +476,11 @@ int sv_host_store_view(int L, const sv_floquet_params *p, int n, int pass, int *
 typedef struct sv_batch sv_batch;
 
 #define SV_BATCH_AUTO (-1)      /* autotune per distinct L */
-#define SV_BATCH_PLAIN 0        /* per-gate passes */
+#define SV_BATCH_PLAIN 0        /* gate by gate */
 #define SV_BATCH_BLOCK_SIMT 1   /* fused windows on CUDA cores: n = 5..7 chosen by the
                                    autotuner, n = 6 when the form is forced */
 #define SV_BATCH_BLOCK_TC 2     /* fused n = 6 windows on the tensor cores (L >= 13) */
-#define SV_BATCH_RESIDENT 3     /* state in one CTA's shared memory (L <= 14) */
+#define SV_BATCH_RESIDENT 3     /* state in shared memory (L <= 14) */
 #define SV_BATCH_MULTIGATE 4    /* many gates per pass on a shared-memory tile */
 
 /* Bytes of the state buffer for n_chains chains of sizes L[0..n_chains):

@@ -12,6 +12,8 @@
 //   k_adjoint_gate  one two-site operation on bond (b, b+1): accumulates
 //                   Re <lambda|D|psi> (D = dO O^dagger), then psi <- O^dag psi
 //                   and lambda <- O^dag lambda, in place;
+//   k_adjoint_tile  the same for several operations, on tiles of both states
+//                   (complex64 from five sites);
 //   k_grad_reduce   the partials of a range of passes, summed in a fixed
 //                   order, times 2, into one gradient entry.
 #include <cuda_runtime.h>

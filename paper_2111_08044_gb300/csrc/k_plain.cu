@@ -1,7 +1,10 @@
 // Plain form: one in-place pass over the state per two-qubit gate, the
 // contraction of Eq. 2 of arXiv 2111.08044 done as a 4x4 complex matvec per
 // group of four amplitudes, plus the product-state initialisation, the
-// per-period energy / norm reduction and the renormalisation pass.
+// per-period energy / norm reduction and the renormalisation pass.  Evolutions of
+// chains from five sites take several gates a pass (k_tile.cu) or stay in shared
+// memory (k_resident.cu), with this arithmetic; the passes here serve shorter chains
+// and measurements by identity gates.
 //
 // Layout: amplitude x = sum_i b_i 2^i, interleaved (re, im).  A complex64
 // thread works on float4 vectors (two consecutive amplitudes); a complex128
