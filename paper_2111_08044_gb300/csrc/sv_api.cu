@@ -940,7 +940,9 @@ int build_resident_chain(sv_ctx* ctx) {
 // Per-period tables are passed as parameters from this length on, where a pass (7 us
 // and more) hides the host's packing and launch of the next (3 us): 24 sites 2.1 ms a
 // period, with the tables copied to shared memory by each block 2.7 ms.
+// The host keeps every period's tables for it: at most kDriveBytes.
 constexpr int kDriveMinL = 19;
+constexpr size_t kDriveBytes = 256 << 20;
 
 // The tile passes of a plain-mode period (none on chains too short for them):
 // their rounds on the device, the launch arguments, the partial pairs.
@@ -965,6 +967,8 @@ int build_tiles(sv_ctx* ctx, std::vector<float2>& host_tab, const std::vector<fl
   std::vector<fsv::TileRound> rounds;
   for (const auto& p : plan) rounds.insert(rounds.end(), p.rounds.begin(), p.rounds.end());
   ctx->tile_single = plan.size() == 1 && tb == L;
+  const bool drive = ctx->precision == SV_C64 && ctx->n_period_params > 0 && L >= kDriveMinL &&
+                     sizeof(float2) * host_tab.size() <= kDriveBytes;
   const size_t cb = amp_bytes(ctx->precision);
   size_t round_at = 0;
   ctx->part_pairs = 0;
@@ -990,7 +994,7 @@ int build_tiles(sv_ctx* ctx, std::vector<float2>& host_tab, const std::vector<fl
     }
     if (ta.first) ta.ep.rn = renorm_of(ctx);
     t.first_gate = p.gates[0];
-    if (ctx->precision == SV_C64 && (ta.stride == 0 || L >= kDriveMinL) && !ta.ep.rn.ring) {
+    if (ctx->precision == SV_C64 && (ta.stride == 0 || drive) && !ta.ep.rn.ring) {
       ta.in_params = 1;
       t.tab.reset(new fsv::TileTab());
       pack_tables(&host_tab[(size_t)t.first_gate * fsv::kGateEntries], p.gates.size(), t.tab->g[0]);
@@ -1035,8 +1039,7 @@ int build_tiles(sv_ctx* ctx, std::vector<float2>& host_tab, const std::vector<fl
     round_at += p.rounds.size();
     ctx->tiles.push_back(std::move(t));
   }
-  if (ctx->precision == SV_C64 && ctx->n_period_params > 0 && L >= kDriveMinL)
-    ctx->drive_tab = std::move(host_tab);
+  if (drive) ctx->drive_tab = std::move(host_tab);
   // the rounds behind the gate tables (allocated with them)
   const size_t bytes = rounds.size() * sizeof(fsv::TileRound);
   char* d_rounds = static_cast<char*>(ctx->d_gates) + ctx->d_gates_bytes;

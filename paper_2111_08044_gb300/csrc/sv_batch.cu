@@ -88,8 +88,7 @@ struct sv_batch {
   // energies of the graph-form chains: their rings, and a buffer that a run's
   // slots are gathered into for one copy
   fsv::RingSource* d_rings = nullptr;
-  char* d_gather = nullptr;
-  size_t gather_bytes = 0;
+  double* d_gather = nullptr;
   int M = 16;
   int64_t counter = 0;
   std::string err;
@@ -415,34 +414,39 @@ int make_graph(sv_batch* b, const std::vector<int>& chains, const ResidentSet* r
   return SV_OK;
 }
 
+// Bytes that the energies of `count` periods of `chains` chains are gathered into,
+// and their flags behind them.
+size_t gather_bytes(size_t chains, int64_t count) {
+  return (2 * sizeof(double) * (size_t)count + sizeof(int)) * chains;
+}
+
+// The rings of the graph-form chains, and the buffer for a ring's length of periods.
+int make_gather(sv_batch* b, const std::vector<int>& chains) {
+  if (chains.empty()) return SV_OK;
+  std::vector<fsv::RingSource> src;
+  for (int c : chains) src.push_back(fsv::ctx_ring(b->ctx[c]));
+  const size_t bytes = sizeof(fsv::RingSource) * src.size();
+  if (cudaMalloc(&b->d_rings, bytes) != cudaSuccess ||
+      cudaMalloc(&b->d_gather, gather_bytes(src.size(), fsv::ctx_ring_len())) != cudaSuccess) {
+    cudaGetLastError();
+    return bfail(b, SV_ENOMEM, "energy readback buffer");
+  }
+  BCUDA(cudaMemcpyAsync(b->d_rings, src.data(), bytes, cudaMemcpyHostToDevice, b->stream),
+        "upload ring list");
+  BCUDA(cudaStreamSynchronize(b->stream), "synchronize");
+  return SV_OK;
+}
+
 // Energies and norms of the graph-form chains' last `count` periods (one copy for
 // all chains, rows of `periods` from column `done`).
 int read_graph_chains(sv_batch* b, const std::vector<int>& chains, int64_t count, int64_t periods,
                       int64_t done, double* energy_out, double* norm_out) {
   const size_t C = chains.size(), pairs = C * (size_t)count;
-  const size_t bytes = 2 * sizeof(double) * pairs + sizeof(int) * C;
-  if (!b->d_rings) {
-    std::vector<fsv::RingSource> src;
-    for (int c : chains) src.push_back(fsv::ctx_ring(b->ctx[c]));
-    BCUDA(cudaMalloc(&b->d_rings, sizeof(fsv::RingSource) * C), "ring list");
-    BCUDA(cudaMemcpyAsync(b->d_rings, src.data(), sizeof(fsv::RingSource) * C, cudaMemcpyHostToDevice,
-                          b->stream),
-          "upload ring list");
-    BCUDA(cudaStreamSynchronize(b->stream), "synchronize");
-  }
-  if (b->gather_bytes < bytes) {
-    cudaFree(b->d_gather);
-    b->d_gather = nullptr;
-    b->gather_bytes = 0;
-    BCUDA(cudaMalloc(&b->d_gather, bytes), "energy readback buffer");
-    b->gather_bytes = bytes;
-  }
-  double* out = reinterpret_cast<double*>(b->d_gather);
-  BCUDA(fsv::launch_gather_rings(b->d_rings, (int)C, b->counter, (int)count, fsv::ctx_ring_len(), out,
-                                 reinterpret_cast<int*>(out + 2 * pairs), b->stream),
+  std::vector<char> host(gather_bytes(C, count));
+  BCUDA(fsv::launch_gather_rings(b->d_rings, (int)C, b->counter, (int)count, fsv::ctx_ring_len(),
+                                 b->d_gather, reinterpret_cast<int*>(b->d_gather + 2 * pairs), b->stream),
         "energy gather launch");
-  std::vector<char> host(bytes);
-  BCUDA(cudaMemcpyAsync(host.data(), b->d_gather, bytes, cudaMemcpyDeviceToHost, b->stream),
+  BCUDA(cudaMemcpyAsync(host.data(), b->d_gather, host.size(), cudaMemcpyDeviceToHost, b->stream),
         "energy readback");
   BCUDA(cudaStreamSynchronize(b->stream), "synchronize");
   const double* p = reinterpret_cast<const double*>(host.data());
@@ -568,8 +572,11 @@ int setup(sv_batch* b) {
       int rc = build_graph_form(b, c, b->form[c],
                                 b->width[c] > 0 ? b->width[c] : kDefaultWidth);
       if (rc) return rc;
+      graph_chains.push_back(c);
     }
   }
+  int rc = make_gather(b, graph_chains);
+  if (rc) return rc;
   return build_resident(b, b->res, &b->rset);
 }
 
