@@ -1394,7 +1394,12 @@ cudaError_t launch_block_tc(const PassArgs& pa, void* psi, const void* map, int*
   else if (pa.diag) k = (const void*)k_block_tc<false, false, true>;
   else if (pa.x_mask) k = (const void*)k_block_tc<false, true, false>;
   void* args[] = {&p, &status};
-  return launch_overlapped(k, grid, kThreads, kSmemBytes, s, args, overlap);
+  // Overlapped where the state stays in L2 (21 sites 121 us a period, 133 in turn; 23
+  // sites 319 and 334): blocks that start in the order SMs become free find less of a
+  // larger one there (24 sites 640 and 626 us, 25 sites 1.27 and 1.24 ms), and from 26
+  // sites on a pass is too long for it to matter.
+  constexpr int kOverlapMaxL = 23;
+  return launch_overlapped(k, grid, kThreads, kSmemBytes, s, args, overlap && pa.L <= kOverlapMaxL);
 }
 
 cudaError_t launch_block_tc_groups(const GroupPasses& passes, int n, int* status, bool overlap,

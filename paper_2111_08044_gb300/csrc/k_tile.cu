@@ -565,7 +565,9 @@ cudaError_t tile_grid(int precision, TileArgs* ta, const LaunchCfg& cfg, int* gr
     if (tiles <= (uint64_t)cfg.num_sms * per_sm) break;  // one tile a block: nothing to prefetch
   }
   *grid = (int)std::min<uint64_t>(tiles, (uint64_t)cfg.num_sms * per_sm);
-  ta->overlap = cfg.alone();
+  // Passes of one tile a block start under the one before (20 sites 174 us a period, in
+  // turn 176); of several tiles they gain nothing (22 sites 505 and 497 us).
+  ta->overlap = cfg.alone() && tiles <= (uint64_t)cfg.num_sms * per_sm;
   ta->smem = (uint32_t)tile_smem_bytes(precision, *ta);
   if (ta->overlap) ta->smem = (uint32_t)even_smem(*grid, cfg.num_sms, ta->smem);
   return e;

@@ -88,11 +88,11 @@ struct GroupPass {
   int nt_log2 = 0, cta_end = 0;
   int tile_sums = 0;  // partial: a (energy, norm) pair of FP32 sums per tile and row
 };
-constexpr int kGroupsPerLaunch = 16;
+constexpr int kGroupsPerLaunch = 8;
 struct GroupPasses {
   GroupPass g[kGroupsPerLaunch];
 };
-static_assert(sizeof(GroupPasses) <= 16 * 1024, "kernel parameters");
+static_assert(sizeof(GroupPasses) <= 4 * 1024, "kernel parameters, copied into every node of a graph");
 
 struct BlockPlan {
   int L = 0, n = 0, R = 0, split = 0;
