@@ -1,7 +1,7 @@
 // Batch chains of two to kShortMaxL sites: one block a chain, its state in shared
 // memory for a run of periods, one group of four amplitudes a thread and gate.
 //
-// A chain that short is one or two warps at most, so that the length of a warp's
+// A chain that short is a few warps (eight of ten sites), so that the length of a warp's
 // chain of instructions per gate bounds it, not the device's rates; the resident
 // form of longer chains (two gates on 16 amplitudes a thread) takes fewer
 // instructions in all but more in a row.  Tables and coefficients in shared
@@ -21,17 +21,20 @@ namespace {
 
 using namespace dev;
 
-constexpr int kThreads = 128;
+constexpr int kThreads = 128;      // a group of four amplitudes each, up to nine sites
+constexpr int kThreadsMost = 256;  // ten sites
 
-__global__ void __launch_bounds__(kThreads)
+template <int T>
+__global__ void __launch_bounds__(T)
     k_chain_short(const ChainArgs* __restrict__ chains, const long long* __restrict__ counter,
                   int periods, int ring_len) {
-  __shared__ float2 sp[1 << kShortMaxL];
+  constexpr int kMaxL = T == kThreads ? kShortMaxL - 1 : kShortMaxL;
+  __shared__ float2 sp[1 << kMaxL];
   __shared__ __align__(16) float2 tables[kShortGates * kGateEntries];
   __shared__ int bonds[kShortGates];
   __shared__ ChainArgs ch;
-  __shared__ double se[kThreads / 32], sn[kThreads / 32];
-  for (uint32_t k = threadIdx.x; k < sizeof(ChainArgs) / 4; k += kThreads)
+  __shared__ double se[T / 32], sn[T / 32];
+  for (uint32_t k = threadIdx.x; k < sizeof(ChainArgs) / 4; k += T)
     reinterpret_cast<uint32_t*>(&ch)[k] = reinterpret_cast<const uint32_t*>(chains + blockIdx.x)[k];
   const long long p0 = counter[0];
   if (periods == 0) periods = (int)counter[1];
@@ -41,18 +44,18 @@ __global__ void __launch_bounds__(kThreads)
   // a period of more gates is read from global memory
   const bool held = ch.ngates <= kShortGates;
   if (held) {
-    for (int k = threadIdx.x; k < ch.ngates * (kGateEntries / 2); k += kThreads)
+    for (int k = threadIdx.x; k < ch.ngates * (kGateEntries / 2); k += T)
       reinterpret_cast<float4*>(tables)[k] = __ldg(reinterpret_cast<const float4*>(ch.gates) + k);
-    for (int k = threadIdx.x; k < ch.ngates; k += kThreads) bonds[k] = __ldg(ch.bonds + k);
+    for (int k = threadIdx.x; k < ch.ngates; k += T) bonds[k] = __ldg(ch.bonds + k);
   }
-  for (uint32_t i = threadIdx.x; i < n; i += kThreads) sp[i] = ch.psi[i];
+  for (uint32_t i = threadIdx.x; i < n; i += T) sp[i] = ch.psi[i];
   __syncthreads();
   // diagonal energy of the thread's amplitudes, site by site
-  constexpr int kAmps = (1 << kShortMaxL) / kThreads;
+  constexpr int kAmps = (1 << kMaxL) / T;
   float diag[kAmps];
 #pragma unroll
   for (int k = 0; k < kAmps; ++k) {
-    const uint32_t x = threadIdx.x + k * kThreads;
+    const uint32_t x = threadIdx.x + k * T;
     float d = 0.f;
     for (int i = 0; i < L; ++i) {
       const float zi = ((x >> i) & 1) ? -1.f : 1.f;
@@ -97,20 +100,40 @@ __global__ void __launch_bounds__(kThreads)
       }
       __syncthreads();
     }
-    // <H0> and the norm of the period's final state
+    // <H0> and the norm of the period's final state.  Of ten sites, as in the
+    // resident form (k_resident.cu): amplitudes that agree in sites 0..8 are added
+    // in ascending order, compensated in FP32
     double e = 0.0, nn = 0.0;
+    constexpr int kSums = 512 / T;
 #pragma unroll
-    for (int k = 0; k < kAmps; ++k) {
-      const uint32_t x = threadIdx.x + k * kThreads;
-      if (x >= n) break;
-      const float2 v = sp[x];
-      const float pr = cabs2(v);
-      float ex = 0.f;
+    for (int k = 0; k < kSums; ++k) {
+      float es = 0.f, ec = 0.f, ns = 0.f, nc = 0.f;
 #pragma unroll
-      for (int i = 0; i < kShortMaxL; ++i)
-        if (i < L && !((x >> i) & 1)) ex += 2.f * ch.cx[i] * cdotre(v, sp[x | (1u << i)]);
-      e += (double)(pr * diag[k] + ex);
-      nn += (double)pr;
+      for (int m = k; m < kAmps; m += kSums) {
+        const uint32_t x = threadIdx.x + m * T;
+        if (x >= n) break;
+        const float2 v = sp[x];
+        const float pr = cabs2(v);
+        float ex = 0.f;
+#pragma unroll
+        for (int i = 0; i < kMaxL; ++i)
+          if (i < L && !((x >> i) & 1)) ex += 2.f * ch.cx[i] * cdotre(v, sp[x | (1u << i)]);
+        if constexpr (kSums == kAmps) {
+          e += (double)(pr * diag[m] + ex);
+          nn += (double)pr;
+        } else {
+          const float ye = __fsub_rn(__fmaf_rn(pr, diag[m], ex), ec), te = __fadd_rn(es, ye);
+          ec = __fsub_rn(__fsub_rn(te, es), ye);
+          es = te;
+          const float yn = __fsub_rn(pr, nc), tn = __fadd_rn(ns, yn);
+          nc = __fsub_rn(__fsub_rn(tn, ns), yn);
+          ns = tn;
+        }
+      }
+      if constexpr (kSums != kAmps) {
+        e += (double)es - (double)ec;
+        nn += (double)ns - (double)nc;
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -123,9 +146,9 @@ __global__ void __launch_bounds__(kThreads)
       sn[w] = nn;
     }
     __syncthreads();
-    if (threadIdx.x == kThreads - 32) {  // its warp has no gates in chains below nine sites
+    if (threadIdx.x == T - 32) {  // its warp has no gates in chains below nine sites
       double te = 0.0, tn = 0.0;
-      for (int k = 0; k < kThreads / 32; ++k) {
+      for (int k = 0; k < T / 32; ++k) {
         te += se[k];
         tn += sn[k];
       }
@@ -135,7 +158,7 @@ __global__ void __launch_bounds__(kThreads)
       out[1] = tn;
     }
   }
-  for (uint32_t i = threadIdx.x; i < n; i += kThreads) ch.psi[i] = sp[i];
+  for (uint32_t i = threadIdx.x; i < n; i += T) ch.psi[i] = sp[i];
 }
 
 // Ring slots of periods c0 .. c0 + count - 1 of each chain, and its flag: one block
@@ -159,13 +182,24 @@ cudaError_t launch_gather_rings(const RingSource* from, int chains, long long c0
 
 cudaError_t short_prepare() {
   // the carve-out of the resident form's blocks, so that both share an SM
-  return cudaFuncSetAttribute(k_chain_short, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  cudaError_t e = cudaFuncSetAttribute(k_chain_short<kThreads>,
+                                       cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_chain_short<kThreadsMost>,
+                             cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  return e;
 }
 
-cudaError_t launch_chain_short(const ChainArgs* chains, int nchains, const long long* counter,
-                               int periods, int ring_len, cudaStream_t s) {
+int short_threads(int L) { return L < kShortMaxL ? kThreads : kThreadsMost; }
+
+cudaError_t launch_chain_short(const ChainArgs* chains, int nchains, int threads,
+                               const long long* counter, int periods, int ring_len, cudaStream_t s) {
   if (nchains <= 0) return cudaSuccess;
-  k_chain_short<<<nchains, kThreads, 0, s>>>(chains, counter, periods, ring_len);
+  if (threads == kThreads)
+    k_chain_short<kThreads><<<nchains, kThreads, 0, s>>>(chains, counter, periods, ring_len);
+  else
+    k_chain_short<kThreadsMost>
+        <<<nchains, kThreadsMost, 0, s>>>(chains, counter, periods, ring_len);
   return cudaGetLastError();
 }
 

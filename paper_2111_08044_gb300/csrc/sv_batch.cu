@@ -187,7 +187,12 @@ int build_resident(sv_batch* b, const std::vector<int>& chains, ResidentSet* rs)
     roff[k] = rounds.size();
     if (L <= fsv::kShortMaxL) {
       for (auto& g : pg) bonds.push_back(g.bond);
-      if (rs->classes.empty() || rs->classes.back().shape.L != 0) rs->classes.push_back({});
+      const int threads = fsv::short_threads(L);
+      if (rs->classes.empty() || rs->classes.back().shape.L != 0 ||
+          rs->classes.back().shape.threads != threads) {
+        rs->classes.push_back({});
+        rs->classes.back().shape.threads = threads;
+      }
     } else {
       const fsv::ResidentShape sh = fsv::resident_shape(false, L, blocks[L]);
       auto rr = fsv::resident_rounds(pg, sh);
@@ -337,8 +342,8 @@ int make_graph(sv_batch* b, const std::vector<int>& chains, const ResidentSet* r
           const ResidentSet::Class& c = rs->classes[k];
           le = c.shape.L ? fsv::launch_resident_batch(rs->d_res + c.first, c.count, c.shape,
                                                       c.ngates, rs->d_count, periods, ring, b->cap_stream)
-                         : fsv::launch_chain_short(rs->d_res + c.first, c.count, rs->d_count, periods,
-                                                  ring, b->cap_stream);
+                         : fsv::launch_chain_short(rs->d_res + c.first, c.count, c.shape.threads,
+                                                   rs->d_count, periods, ring, b->cap_stream);
         }
         e = cudaStreamEndCapture(b->cap_stream, &rg);
         if (le != cudaSuccess) e = le;

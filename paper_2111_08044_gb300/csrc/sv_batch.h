@@ -12,10 +12,12 @@
 namespace fsv {
 
 constexpr int kResidentMaxL = 14;       // of a batch chain
-// Batch chains of k_batch.cu.  Up to nine sites its 128 threads of four amplitudes
-// are the faster ones: 16 chains of nine sites take 14.7 us a period there and
-// 23.6 us in the resident form, of ten sites (two groups a thread) 26 and 25.5.
-constexpr int kShortMaxL = 9;
+// Batch chains of k_batch.cu.  While a thread has one group of four amplitudes (up to
+// nine sites of 128 threads, ten of 256) they are the faster ones: 16 chains of nine
+// sites take 14.7 us a period there and 23.6 us in the resident form, of ten sites
+// 20.9 and 25.7, 600 of ten sites 50 and 73 (with two groups a thread 26 against
+// 25.5); 256 threads for the shorter ones gain nothing.
+constexpr int kShortMaxL = 10;
 constexpr int kShortGates = 64;         // its gate tables held in shared memory (16 KiB)
 // Of a single chain in the plain form: with 16 blocks one of 15 sites takes 80 us a
 // period; tile passes (k_tile.cu) take 106 us at 16 sites and 98 us at 17, over all SMs.
@@ -80,8 +82,10 @@ cudaError_t launch_resident_batch(const ChainArgs* chains, int nchains, const Re
                                   int ngates, const long long* counter, int periods, int ring_len,
                                   cudaStream_t s);
 // The same for chains of up to kShortMaxL sites (any mix), one block each.
-cudaError_t launch_chain_short(const ChainArgs* chains, int nchains, const long long* counter,
-                               int periods, int ring_len, cudaStream_t s);
+// threads: short_threads of their lengths (one value a launch).
+int short_threads(int L);
+cudaError_t launch_chain_short(const ChainArgs* chains, int nchains, int threads,
+                               const long long* counter, int periods, int ring_len, cudaStream_t s);
 cudaError_t short_prepare();
 // (energy, norm) of `count` periods from c0 on of each chain into out[chain][count],
 // its flag into status[chain].

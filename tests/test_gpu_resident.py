@@ -48,9 +48,10 @@ def _chains(Ls, K):
 @pytest.mark.parametrize("Ls,K", [
     # every length, alone on the device: clusters of up to eight blocks
     ([2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14], [4] * 13),
-    # more gates than the tables held (64, 96 above nine sites), with shorter periods
+    # more gates than the tables held (64, 96 above ten sites), with shorter periods
     # of the same length beside them
     ([9, 9, 2, 12, 12, 14], [9, 2, 70, 9, 3, 8]),
+    ([10, 9, 10, 11], [8, 8, 3, 10]),
     # as many chains as SMs and more: one block a chain
     ([10] * 90 + [13] * 80 + [5, 14], [2] * 172)])
 def test_batch_matches_oracle(svlib, Ls, K):
