@@ -306,9 +306,12 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
           run_round<kPlain, true>(rd, gs, ch, tile, sbuf, sp, rank, at, s0 + lane < per, esum, nsum);
       }
       g += rd.count;
+      // read before the barrier: behind it, where the tables held are used up, a
+      // faster warp writes the next ones over rd
+      const int sweep = kPlain ? rd.sweep : 0;
       barrier(wide);
-      if (kPlain && rd.sweep) {
-        const int w = rd.sweep - 1;
+      if (sweep) {  // (rd stays until every warp has passed the barrier below)
+        const int w = sweep - 1;
         measure_sweep(tile, lb, L, ch.cx, ch.ep, rd.bond[w], rd.epi[w],
                       [&](uint32_t l) { return (uint64_t)sp.state(l, rank); }, esum, nsum);
         barrier(wide);
