@@ -200,8 +200,8 @@ std::string block_tile_layout(int L, int n, int R, int lo, int lo_next, int* a_o
 }
 
 int block_build(int L, const std::vector<Gate2>& gates, const Observable& obs, int n,
-                int split, const LaunchCfg& cfg, bool cyclic, BlockPlan** out,
-                std::string* msg) {
+                int split, const LaunchCfg& cfg, bool cyclic, cudaStream_t s,
+                BlockPlan** out, std::string* msg) {
   *out = nullptr;
   if (split != SV_SPLIT_BF16X3 && split != SV_SPLIT_FP32) {
     *msg = "unknown split";
@@ -372,11 +372,9 @@ int block_build(int L, const std::vector<Gate2>& gates, const Observable& obs, i
   }
   if (!bp->tensor_cores &&
       (cudaMalloc(&bp->d_U, sizeof(float2) * hu.size()) != cudaSuccess ||
-       cudaMemcpy(bp->d_U, hu.data(), sizeof(float2) * hu.size(), cudaMemcpyHostToDevice) !=
-           cudaSuccess ||
+       upload(bp->d_U, hu.data(), sizeof(float2) * hu.size(), s) != cudaSuccess ||
        cudaMalloc(&bp->d_Ulead, sizeof(float4) * hl.size()) != cudaSuccess ||
-       cudaMemcpy(bp->d_Ulead, hl.data(), sizeof(float4) * hl.size(), cudaMemcpyHostToDevice) !=
-           cudaSuccess)) {
+       upload(bp->d_Ulead, hl.data(), sizeof(float4) * hl.size(), s) != cudaSuccess)) {
     cudaGetLastError();
     *msg = "unitary upload failed";
     block_free(bp);
@@ -387,8 +385,7 @@ int block_build(int L, const std::vector<Gate2>& gates, const Observable& obs, i
     std::vector<uint32_t> all;
     for (int k = 0; k < NA; ++k) all.insert(all.end(), hw[k].begin(), hw[k].end());
     if (cudaMalloc(&bp->d_W, all.size() * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMemcpy(bp->d_W, all.data(), all.size() * sizeof(uint32_t),
-                   cudaMemcpyHostToDevice) != cudaSuccess) {
+        upload(bp->d_W, all.data(), all.size() * sizeof(uint32_t), s) != cudaSuccess) {
       cudaGetLastError();
       *msg = "operand upload failed";
       block_free(bp);
@@ -397,7 +394,7 @@ int block_build(int L, const std::vector<Gate2>& gates, const Observable& obs, i
   }
   const size_t pbytes = sizeof(double) * 2 * std::max(1, bp->nslots) * (size_t)bp->maxb;
   if (cudaMalloc(&bp->d_partials, pbytes) != cudaSuccess ||
-      cudaMemset(bp->d_partials, 0, pbytes) != cudaSuccess) {
+      upload_zeros(bp->d_partials, pbytes, s) != cudaSuccess) {
     cudaGetLastError();
     *msg = "partials allocation failed";
     block_free(bp);
@@ -415,7 +412,7 @@ int block_build(int L, const std::vector<Gate2>& gates, const Observable& obs, i
   }
   if (bp->tensor_cores) {
     if (block_tc_prepare() != cudaSuccess || cudaMalloc(&bp->d_status, sizeof(int)) != cudaSuccess ||
-        cudaMemset(bp->d_status, 0, sizeof(int)) != cudaSuccess) {
+        upload_zeros(bp->d_status, sizeof(int), s) != cudaSuccess) {
       cudaGetLastError();
       *msg = "tensor-core pass set-up failed";
       block_free(bp);

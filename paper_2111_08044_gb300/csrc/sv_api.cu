@@ -837,7 +837,7 @@ int build_multigate(sv_ctx* ctx, const std::vector<fsv::MultiPass>& plan) {
       ctx->d_mg = nullptr;
       return fail(ctx, SV_ENOMEM, "multi-gate plan allocation failed");
     }
-    SV_CUDA(cudaMemcpy(ctx->d_mg, idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice),
+    SV_CUDA(fsv::upload(ctx->d_mg, idx.data(), sizeof(int) * idx.size(), ctx->cap_stream),
             "upload multi-gate plan");
   }
   SV_CUDA(fsv::multigate_prepare(), "multi-gate shared-memory opt-in");
@@ -928,7 +928,7 @@ int build_resident_chain(sv_ctx* ctx) {
   ch.ep.rn = renorm_of(ctx);
   const size_t bytes = rounds.size() * sizeof(fsv::ResidentRound);
   char* d_rounds = static_cast<char*>(ctx->d_gates) + ctx->d_gates_bytes;  // behind the tables
-  SV_CUDA(cudaMemcpy(d_rounds, rounds.data(), bytes, cudaMemcpyHostToDevice), "upload rounds");
+  SV_CUDA(fsv::upload(d_rounds, rounds.data(), bytes, ctx->cap_stream), "upload rounds");
   ch.rounds = reinterpret_cast<const fsv::ResidentRound*>(d_rounds);
   ctx->tile_single = ctx->resident = true;
   ctx->passes_per_period = 1;
@@ -1043,7 +1043,7 @@ int build_tiles(sv_ctx* ctx, std::vector<float2>& host_tab, const std::vector<fl
   // the rounds behind the gate tables (allocated with them)
   const size_t bytes = rounds.size() * sizeof(fsv::TileRound);
   char* d_rounds = static_cast<char*>(ctx->d_gates) + ctx->d_gates_bytes;
-  SV_CUDA(cudaMemcpy(d_rounds, rounds.data(), bytes, cudaMemcpyHostToDevice), "upload tile plan");
+  SV_CUDA(fsv::upload(d_rounds, rounds.data(), bytes, ctx->cap_stream), "upload tile plan");
   round_at = 0;
   for (auto& t : ctx->tiles) {
     t.ta.rounds = reinterpret_cast<fsv::TileRound*>(d_rounds) + round_at;
@@ -1350,18 +1350,18 @@ int sv_create(sv_ctx** out, int device, int precision, void* cuda_stream) {
     if (precision == SV_C128) {
       double2 id[fsv::kGateEntries] = {};  // identity, zero residual
       for (int k = 0; k < 4; ++k) id[5 * k].x = 1.0;
-      ok = cudaMemcpy(ctx->d_ident, id, sizeof(id), cudaMemcpyHostToDevice) == cudaSuccess;
+      ok = fsv::upload(ctx->d_ident, id, sizeof(id), ctx->cap_stream) == cudaSuccess;
     } else if (precision == SV_DF64) {
       float4 id[fsv::kGateEntries] = {};  // (re hi, re lo, im hi, im lo)
       for (int k = 0; k < 4; ++k) id[5 * k].x = 1.0f;
-      ok = cudaMemcpy(ctx->d_ident, id, sizeof(id), cudaMemcpyHostToDevice) == cudaSuccess;
+      ok = fsv::upload(ctx->d_ident, id, sizeof(id), ctx->cap_stream) == cudaSuccess;
     } else {
       float2 id[fsv::kGateEntries] = {};
       for (int k = 0; k < 4; ++k) id[5 * k].x = 1.0f;
-      ok = cudaMemcpy(ctx->d_ident, id, sizeof(id), cudaMemcpyHostToDevice) == cudaSuccess;
+      ok = fsv::upload(ctx->d_ident, id, sizeof(id), ctx->cap_stream) == cudaSuccess;
     }
-    ok = ok && cudaMemset(ctx->d_counter, 0, sizeof(long long)) == cudaSuccess;
-    ok = ok && cudaMemset(ctx->d_ring, 0, sizeof(double) * 2 * kRing) == cudaSuccess;
+    ok = ok && fsv::upload_zeros(ctx->d_counter, sizeof(long long), ctx->cap_stream) == cudaSuccess;
+    ok = ok && fsv::upload_zeros(ctx->d_ring, sizeof(double) * 2 * kRing, ctx->cap_stream) == cudaSuccess;
   }
   if (!ok) {
     cudaGetLastError();
@@ -1468,7 +1468,7 @@ int sv_build_floquet(sv_ctx* ctx, const sv_floquet_params* p) {
     if (n > ctx->L) n = ctx->L;
     std::string msg;
     int rc = fsv::block_build(ctx->L, ctx->gates, ctx->obs, n, p->split, ctx->cfg,
-                              ctx->cyclic, &ctx->block, &msg);
+                              ctx->cyclic, ctx->cap_stream, &ctx->block, &msg);
     if (rc != SV_OK) return fail(ctx, rc, "block build: %s", msg.c_str());
     fsv::block_set_renorm(ctx->block, renorm_of(ctx));
     fsv::block_info(ctx->block, &ctx->passes_per_period, &ctx->launches_per_period);

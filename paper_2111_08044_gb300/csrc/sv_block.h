@@ -126,9 +126,10 @@ struct BlockPlan {
 // bits) goes to output tile bit sigma[q].  Empty on success, else the reason.
 std::string block_tile_layout(int L, int n, int R, int lo, int lo_next, int* a_out,
                               int8_t* sigma);
+// s: a stream of the library's for the uploads (see upload).
 int block_build(int L, const std::vector<Gate2>& gates, const Observable& obs, int n,
-                int split, const LaunchCfg& cfg, bool cyclic, BlockPlan** out,
-                std::string* msg);
+                int split, const LaunchCfg& cfg, bool cyclic, cudaStream_t s,
+                BlockPlan** out, std::string* msg);
 void block_info(const BlockPlan* bp, int* passes, int* launches);
 // Fold the periodic renormalisation into the period's first pass.
 void block_set_renorm(BlockPlan* bp, const Renorm& rn);

@@ -100,6 +100,18 @@ inline size_t even_smem(int grid, int num_sms, size_t need) {
 }
 constexpr int kEvenSmemMax = 116 * 1024;  // its largest padding (one block an SM)
 
+// A host array to the device, there when the call returns (a copy on the default stream
+// may still be on its way then, and another stream does not wait for it).  s: a stream
+// of the library's, without work of the caller's.
+inline cudaError_t upload(void* to, const void* from, size_t bytes, cudaStream_t s) {
+  const cudaError_t e = cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, s);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+inline cudaError_t upload_zeros(void* to, size_t bytes, cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(to, 0, bytes, s);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+
 // Grid (blocks of 256 threads) used by the plain gate pass for this L and
 // bond; it is also the number of partial pairs the pass writes.
 int plain_gate_grid(int L, int bond, int precision, const LaunchCfg& cfg);
