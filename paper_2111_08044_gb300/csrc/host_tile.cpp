@@ -162,7 +162,10 @@ int tile_bits(int L, int precision, const LaunchCfg& cfg) {
   // 2.17 ms), of 2^11 below (16 sites 86 us, 104 in tiles of 2^12, 88 of 2^10) unless
   // other chains' passes fill the rest (12 chains of 16 to 18 sites, 32 periods: 7.5 ms
   // and 9.4 ms in tiles of 2^11).
-  return !cfg.alone() || (4ll << L) >= 3ll * num_sms << 12 ? 12 : 11;
+  // A chain that the tile would hold (where the resident form finds no room on the
+  // device) takes one launch a gate: complex64 passes run one period.
+  const int tb = !cfg.alone() || (4ll << L) >= 3ll * num_sms << 12 ? 12 : 11;
+  return L > tb ? tb : 0;
 }
 
 std::vector<ResidentRound> resident_rounds(const std::vector<Gate2>& gates, const ResidentShape& sh) {

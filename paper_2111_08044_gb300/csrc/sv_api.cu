@@ -914,6 +914,7 @@ bool tile_runs(int L, const fsv::TilePassPlan& p, fsv::TileArgs* ta) {
 int build_resident_chain(sv_ctx* ctx) {
   const int L = ctx->L;
   const auto rounds = fsv::resident_rounds(ctx->gates, ctx->shape);
+  if (rounds.empty()) return fail(ctx, SV_EINVAL, "no plan for a chain in shared memory");
   fsv::ChainArgs& ch = ctx->chain;
   ch = fsv::ChainArgs();
   ch.L = L;

@@ -196,6 +196,7 @@ int build_resident(sv_batch* b, const std::vector<int>& chains, ResidentSet* rs)
     } else {
       const fsv::ResidentShape sh = fsv::resident_shape(false, L, blocks[L]);
       auto rr = fsv::resident_rounds(pg, sh);
+      if (rr.empty()) return bfail(b, SV_EINVAL, "chain %d: no plan for a chain in shared memory", c);
       r.nrounds = (int)rr.size();
       rounds.insert(rounds.end(), rr.begin(), rr.end());
       if (rs->classes.empty() || rs->classes.back().shape.L != L) {
