@@ -120,6 +120,7 @@ int fail(sv_ctx* c, int code, const char* fmt, ...) {
 }
 
 int cuda_fail(sv_ctx* c, cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here, not again by the next call's launches
   return fail(c, SV_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 

@@ -112,6 +112,7 @@ int bfail(sv_batch* b, int code, const char* fmt, ...) {
     va_end(ap);
     b->err = buf;
   }
+  if (code == SV_ECUDA) cudaGetLastError();  // reported here, not again by the next call
   return code;
 }
 

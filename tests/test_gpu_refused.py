@@ -1,0 +1,51 @@
+"""Calls that are refused while their stream is captured: an error status, nothing
+advanced, and the calls after them as if they had not been made."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2111_08044_gb300 import capi, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+class _Capture:
+    """The stream's work goes to a graph that is thrown away."""
+
+    def __init__(self, stream):
+        self.rt = ctypes.CDLL("libcudart.so.13")
+        self.s = ctypes.c_void_p(stream.cuda_stream)
+
+    def __enter__(self):
+        assert self.rt.cudaStreamBeginCapture(self.s, 2) == 0  # relaxed
+
+    def __exit__(self, *exc):
+        g = ctypes.c_void_p()
+        self.rt.cudaStreamEndCapture(self.s, ctypes.byref(g))
+        if g.value:
+            self.rt.cudaGraphDestroy(g)
+        self.rt.cudaGetLastError()
+
+
+def _sim(L, stream, precision="c64", drive=False, **form):
+    from paper_2111_08044_gb300.sim import FloquetSimulator, chain_params
+    cfg = inputs.ChainConfig(L=L, seed=L)
+    if drive:
+        cfg.theta_p, cfg.hx_p = np.linspace(0.2, 0.4, 8), np.linspace(0.7, 0.9, 8)
+    sim = FloquetSimulator(L, precision=precision, stream=stream)
+    sim.init_product_state(cfg.spinors())
+    sim.build(**chain_params(cfg, **form))
+    return sim
+
+
+def test_refused_call_leaves_no_error_behind(svlib):
+    import torch
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        sim = _sim(14, s, mode=capi.SV_MODE_BLOCK, block_n=6)
+        sim.evolve(1)
+        with _Capture(s):
+            assert svlib.sv_evolve(sim._ctx, 1, None, None) == capi.SV_ECUDA
+        sim.init_product_state(inputs.ChainConfig(L=14).spinors())  # raised here
+        sim.close()
