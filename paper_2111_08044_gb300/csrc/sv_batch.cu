@@ -717,6 +717,13 @@ int sv_batch_evolve(sv_batch* b, int64_t periods, double* energy_out, double* no
   const int ring = fsv::ctx_ring_len();
   int64_t done = 0;
   std::vector<double> rbuf;
+  // a call that ends early may not have run the copy of its run length
+  struct Forget {
+    int64_t* run;
+    ~Forget() {
+      if (run) *run = 0;
+    }
+  } forget{&b->run};
   while (done < periods) {
     const int64_t chunk = std::min<int64_t>(periods - done, ring);
     int64_t k = 0;
@@ -766,6 +773,7 @@ int sv_batch_evolve(sv_batch* b, int64_t periods, double* energy_out, double* no
     done += chunk;
   }
   BCUDA(cudaStreamSynchronize(b->stream), "synchronize");
+  forget.run = nullptr;
   return SV_OK;
 }
 

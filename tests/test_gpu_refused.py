@@ -49,3 +49,23 @@ def test_refused_call_leaves_no_error_behind(svlib):
             assert svlib.sv_evolve(sim._ctx, 1, None, None) == capi.SV_ECUDA
         sim.init_product_state(inputs.ChainConfig(L=14).spinors())  # raised here
         sim.close()
+
+
+def test_refused_batch_run_changes_nothing(svlib):
+    """A run of another length after a refused one is of its own length."""
+    import torch
+    from paper_2111_08044_gb300.sim import FloquetBatch
+    chains = [inputs.ChainConfig(L=L, seed=L) for L in (6, 12, 13)]
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        out = []
+        for refuse in (False, True):
+            with FloquetBatch(chains, form=capi.SV_BATCH_RESIDENT, stream=s) as b:
+                parts = [b.evolve(8)]
+                if refuse:
+                    with _Capture(s):
+                        assert svlib.sv_batch_evolve(b._b, 3, None, None) == capi.SV_ECUDA
+                parts.append(b.evolve(3))
+                out.append([x for p in parts for x in p] + [b.chain_state(c) for c in range(3)])
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
