@@ -179,7 +179,8 @@ int sv_build_floquet(sv_ctx *ctx, const sv_floquet_params *p);
  * parameters the period counter must stay below n_period_params.
  * Errors: SV_EINVAL, SV_ESTATE, SV_ECUDA, SV_ETIMEOUT (a tensor-core pass
  * gave up a bounded wait; reported when the call synchronises, i.e. when
- * energy_out or norm_out is given).
+ * energy_out or norm_out is given).  On a stream under capture: SV_ECUDA, with
+ * nothing advanced.
  */
 int sv_evolve(sv_ctx *ctx, int64_t periods, double *energy_out, double *norm_out);
 

@@ -349,6 +349,13 @@ int ensure_graph(sv_ctx* ctx) {
 int launch_periods(sv_ctx* ctx, int64_t count, bool last) {
   const bool off = off_natural(ctx);
   if (count <= 0) return SV_OK;
+  // Refused under a capture, before anything is enqueued, in every form: the runtime
+  // refuses the graph launches only, and periods launched directly (or a relabel before
+  // a graph) would be counted here and run at a replay, with a drive's tables of then.
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  SV_CUDA(cudaStreamIsCapturing(ctx->stream, &st), "evolve");
+  if (st != cudaStreamCaptureStatusNone)
+    return cuda_fail(ctx, cudaErrorStreamCaptureUnsupported, "evolve");
   if (ctx->tile_single) {
     // runs of at most 2^15 gates a launch (tens of milliseconds)
     const int64_t most = std::max<int64_t>(1, 32768 / (int64_t)ctx->gates.size());

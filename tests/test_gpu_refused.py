@@ -69,3 +69,29 @@ def test_refused_batch_run_changes_nothing(svlib):
                 out.append([x for p in parts for x in p] + [b.chain_state(c) for c in range(3)])
     for x, y in zip(*out):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("L,kw", [
+    (4, {}), (6, {}), (12, {}), (15, {}), (17, {}), (12, dict(drive=True)), (17, dict(drive=True)),
+    (19, dict(drive=True)), (9, dict(precision="df64")), (13, dict(precision="df64")),
+    (7, dict(precision="c128")), (14, dict(mode=capi.SV_MODE_BLOCK, block_n=6)),
+    (14, dict(mode=capi.SV_MODE_MULTIGATE))])
+def test_refused_evolution_changes_nothing(svlib, L, kw):
+    """An evolution under a capture is refused in every form: the periods of a replay
+    would not be those that were captured."""
+    import torch
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        out = []
+        for refuse in (False, True):
+            sim = _sim(L, s, **kw)
+            sim.evolve(2)
+            if refuse:
+                with _Capture(s):
+                    assert svlib.sv_evolve(sim._ctx, 2, None, None) == capi.SV_ECUDA
+                assert sim.period == 2
+            e, n = sim.evolve(3)
+            out.append((e, n, sim.host_state()))
+            sim.close()
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
