@@ -360,7 +360,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       }
       const long long slot = (c0 + p) % ring_len;
       double* const out = ch.ring + 2 * slot * ch.ring_stride;
-      out[0] = n > 0.0 ? e / ((double)L * n) : 0.0;
+      // plain: as the period reduce writes it; batch: as the shorter chains' (NaN where
+      // the norm is NaN or zero)
+      out[0] = !kPlain || n > 0.0 ? e / ((double)L * n) : 0.0;
       out[1] = n;
       if (scaled) __threadfence();
     }
