@@ -685,7 +685,8 @@ int energy_moments(sv_ctx* ctx, double* energy, double* sigma_e, double* norm2) 
     s2 += part[3 * b + 1];
     sn += part[3 * b + 2];
   }
-  if (!(sn > 0.0)) return fail(ctx, SV_ESTATE, "the state has zero norm");
+  if (!(sn > 0.0) || !std::isfinite(sn))
+    return fail(ctx, SV_ESTATE, "the state has zero or non-finite norm");
   const double E = s1 / sn, var = s2 / sn - E * E;
   if (energy) *energy = E;
   if (sigma_e) *sigma_e = std::sqrt(std::max(var, 0.0));

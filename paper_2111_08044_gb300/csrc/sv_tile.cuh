@@ -82,8 +82,9 @@ struct FloatSum {
     hi = s.hi;
     lo = __fadd_rn(lo, s.lo);
   }
+  // (an infinite hi is the sum, its rounding errors are NaN)
   __device__ __forceinline__ void flush(double& acc) {
-    acc += (double)hi + (double)lo;
+    acc += (double)hi + (lo == lo ? (double)lo : 0.0);
     hi = lo = 0.f;
   }
 };
