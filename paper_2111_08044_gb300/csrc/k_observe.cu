@@ -63,40 +63,10 @@ __device__ void block_store_k(double (&v)[K], double* out) {
   }
 }
 
-// The diagonal part of H0 over a thread's amplitudes of one contiguous tile:
-// the tile number's share once, the low bits' per amplitude.
-struct TileDiag {
-  float J, cz_bulk, cz_first, cz_last, czsum;
-  int L, nb_hi, flips_hi, last;
-  uint32_t top;  // bit 0 of the tile number at the place above the tile's bits
-  __device__ void init(const EpiParams& ep, int L_) {
-    L = L_;
-    J = (float)ep.J;
-    cz_bulk = (float)ep.cz_bulk;
-    cz_first = (float)ep.cz_first;
-    cz_last = (float)ep.cz_last;
-    czsum = (float)(ep.cz_bulk * (L_ - 2) + ep.cz_first + ep.cz_last);
-  }
-  __device__ void tile(uint32_t t) {
-    const int hi = L - kBits;  // bits of the tile number, at least 1
-    flips_hi = __popc((t ^ (t >> 1)) & ((1u << (hi - 1)) - 1));
-    last = (t >> (hi - 1)) & 1;
-    nb_hi = __popc(t) - last;
-    top = (t & 1u) << kBits;
-  }
-  __device__ __forceinline__ float operator()(uint32_t e) const {
-    const uint32_t x = e | top;
-    const int flips = flips_hi + __popc((x ^ (x >> 1)) & ((1u << kBits) - 1));
-    const int nb = nb_hi + __popc(e & ~1u);
-    const float up = cz_bulk * (float)nb + ((e & 1) ? cz_first : 0.f) + (last ? cz_last : 0.f);
-    return J * (float)(L - 1 - 2 * flips) + czsum - 2.f * up;
-  }
-};
-
-// The same as an FP32 pair, from tables of its two counts: J (L - 1 - 2 flips), and the
-// fields' sum for nb set bits between the ends and the two end bits.  A value of 20
-// rounded to FP32 is off by up to 1e-6, the same for every amplitude of its counts,
-// which does not average out of a sum near zero.
+// The diagonal part of H0 over the amplitudes of one contiguous tile as an FP32 pair,
+// from tables of its two counts: J (L - 1 - 2 flips), and the fields' sum for nb set
+// bits between the ends and the two end bits.  A value of 20 rounded to FP32 is off by
+// up to 1e-6, the same for every amplitude of its counts, which does not average out.
 struct PairDiag {
   const float2 *zz, *field;  // shared memory: 34, and 4 a count
   int L, nb_hi, flips_hi, last;
@@ -132,6 +102,7 @@ struct PairDiag {
 
 struct EnergyArgs {
   TileArgs ta;          // layout of the pass
+  H0Coef h0;            // of the diagonal part
   float cx[kBits] = {};  // coefficient of each tile bit's <X> (0: another pass's)
   int low = 0;          // tile bits 0..3 measured too
   int diag = 0;
@@ -156,8 +127,9 @@ __global__ void __launch_bounds__(kThreads, 4)
   const uint32_t ntiles = 1u << (ta.L - kBits);
   const uint32_t tid = threadIdx.x;
   const TileIo io = tile_io(ta);
-  TileDiag dg;
-  if (ea.diag) dg.init(ta.ep, ta.L);
+  __shared__ float2 zz[34], field[4 * 33];
+  if (ea.diag) PairDiag::fill(ea.h0, ta.L, zz, field);
+  PairDiag dg{zz, field, ta.L};
   double acc[2] = {0.0, 0.0};
   for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     load_tile(ta, io, sbuf, psi + tile_base(ta, t));
@@ -180,15 +152,25 @@ __global__ void __launch_bounds__(kThreads, 4)
       es.add(ea.cx[q + 2] * pair_sum<2>(v));
       es.add(ea.cx[q + 3] * pair_sum<3>(v));
       if (q == 8 && ea.diag) {
-        float d = 0.f, n = 0.f;
+        // The norm amplitude by amplitude, the diagonal energies four to a sum, their
+        // trailing parts apart.  (With sixteen to a sum and the energies in FP32 the
+        // norm was off by 4 to 12e-9 at 13..18 sites and the density by 1.6e-8, and L =
+        // 25 took 222 us a call; now 0.8 to 3e-9, 2e-9 and 236 us.)
+        float dl = 0.f;
 #pragma unroll
-        for (int m = 0; m < 16; ++m) {
-          const float p = cabs2(v[m]);
-          n += p;
-          d += p * dg(e0 | ((uint32_t)m << q));
+        for (int g = 0; g < 16; g += 4) {
+          float d = 0.f;
+#pragma unroll
+          for (int m = g; m < g + 4; ++m) {
+            const float p = cabs2(v[m]);
+            const df c = dg(e0 | ((uint32_t)m << q));
+            ns.add(p);
+            d = __fmaf_rn(p, c.hi, d);
+            dl = __fmaf_rn(p, c.lo, dl);
+          }
+          es.add(d);
         }
-        es.add(d);
-        ns.add(n);
+        es.add(dl);
       }
     }
     es.flush(acc[0]);
@@ -487,8 +469,8 @@ int observe_energy_pairs(int L, const LaunchCfg& cfg) {
   return ((L - kBits + 7) / 8 + 1) * grid_of(L, cfg, 4);
 }
 
-cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, const EpiParams& diag,
-                               double* part, const LaunchCfg& cfg, cudaStream_t s) {
+cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, double* part,
+                               const LaunchCfg& cfg, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   const int grid = grid_of(L, cfg, 4);
   // the 12 lowest sites; then 8 at a time beside the lowest 4 state bits
@@ -497,7 +479,7 @@ cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, const Ep
     TileArgs& ta = ea.ta;
     ta.L = L;
     ta.tb = kBits;
-    ta.ep = diag;
+    ea.h0 = h;
     ea.low = ea.diag = first == 0;
     const int win = first == 0 ? 0 : std::min(first, L - 8);  // first window site
     if (first == 0) {

@@ -583,8 +583,8 @@ int measure(sv_ctx* ctx, double* e_out, double* n_out) {
   const int L = ctx->L;
   if (fsv::observe_supported(ctx->precision, L)) {
     const int pairs = fsv::observe_energy_pairs(L, ctx->cfg);
-    SV_CUDA(fsv::launch_energy_tile(ctx->state, L, h0_coef(ctx), epi_for(ctx, fsv::EPI_DIAG, 0, nullptr),
-                                    ctx->d_part_meas, ctx->cfg, ctx->stream),
+    SV_CUDA(fsv::launch_energy_tile(ctx->state, L, h0_coef(ctx), ctx->d_part_meas, ctx->cfg,
+                                    ctx->stream),
             "measurement launch");
     return read_measurement(ctx, pairs, e_out, n_out);
   }

@@ -195,8 +195,8 @@ cudaError_t launch_product_overlap(int precision, const void* psi, int L, int m,
 bool observe_supported(int precision, int L);
 // (energy, norm) partial pairs that launch_energy_tile writes
 int observe_energy_pairs(int L, const LaunchCfg& cfg);
-cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, const EpiParams& diag,
-                               double* part, const LaunchCfg& cfg, cudaStream_t s);
+cudaError_t launch_energy_tile(const void* psi, int L, const H0Coef& h, double* part,
+                               const LaunchCfg& cfg, cudaStream_t s);
 // bonds: general bond terms on the host ((L - 1) x 16), or NULL for the Ising chain
 int observe_moments_grid(int L, const LaunchCfg& cfg);
 cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h,

@@ -102,15 +102,14 @@ extern "C" int sv_energy_noalloc(const void* psi_dev, int L, int precision,
   if (fsv::observe_supported(precision, L)) {
     // the same passes as sv_expect_energy (at most four, four blocks an SM)
     fsv::H0Coef h;
-    fsv::EpiParams ep;
-    ep.J = p->J;
-    ep.cz_first = p->hz * fsv::site_field_share(L, 0, ew);
-    ep.cz_last = p->hz * fsv::site_field_share(L, L - 1, ew);
-    ep.cz_bulk = p->hz * fsv::site_field_share(L, 1, ew);
-    for (int i = 0; i < L; ++i) h.cx[i] = p->hx * fsv::site_field_share(L, i, ew);
+    h.J = p->J;
+    for (int i = 0; i < L; ++i) {
+      h.cx[i] = p->hx * fsv::site_field_share(L, i, ew);
+      h.cz[i] = p->hz * fsv::site_field_share(L, i, ew);
+    }
     const int pairs = fsv::observe_energy_pairs(L, cfg);
     if (pairs > kMaxPasses * kMaxBlocks) return SV_EINVAL;
-    cudaError_t e = fsv::launch_energy_tile(psi_dev, L, h, ep, sym.scratch, cfg, s);
+    cudaError_t e = fsv::launch_energy_tile(psi_dev, L, h, sym.scratch, cfg, s);
     if (e == cudaSuccess)
       e = fsv::launch_period_reduce(sym.scratch, pairs, L, out_dev, 1, sym.counter, /*advance=*/0, s);
     return e == cudaSuccess ? SV_OK : SV_ECUDA;
