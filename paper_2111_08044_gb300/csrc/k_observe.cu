@@ -17,9 +17,9 @@
 //                   (L = 24: 1090 -> 393 us).
 //   k_overlap_f32   <phi|psi> of a product state from FP64 factor tables
 //   k_factor_f32    and the state itself: the FP64 units (0.59 TFMA/s) bounded
-//                   both; products and sums are FP32 pairs here (an exact
-//                   product and its error, Dekker and Knuth), moved to FP64
-//                   every 16 amplitudes: 741 -> 92 us; L = 24: 188 -> 30 us.
+//                   both; products and sums are FP32 triples and pairs here (an
+//                   exact product and its error, Dekker and Knuth): 741 -> 149
+//                   us; L = 24: 188 -> 55 us.
 // Partial sums: FP32 within a thread's tile, FP32 pairs across its terms, FP64
 // across tiles, threads and blocks, in a fixed order.
 #include <cuda_runtime.h>
@@ -381,48 +381,132 @@ __device__ __forceinline__ float4 split_pair(double2 v) {
   const float xr = (float)v.x, xi = (float)v.y;
   return make_float4(xr, (float)(v.x - (double)xr), xi, (float)(v.y - (double)xi));
 }
-// (s, c) += (g.hi + g.lo) v: exact leading product, every error term in c
-__device__ __forceinline__ void add_product(float gh, float gl, float v, float& s, float& c) {
-  const float p = __fmul_rn(gh, v);
-  float e = __fmaf_rn(gh, v, -p);
-  e = __fmaf_rn(gl, v, e);
-  const df t = two_sum(s, p);
-  s = t.hi;
-  c = __fadd_rn(c, __fadd_rn(t.lo, e));
-}
+// A packed sum of products (re, im) in three FP32 parts s + c + d, each addition exact
+// in the leading two.  A factor x as packed operands: leading part and its negative, the
+// middle one's, the trailing one's negative (24 + 24 + 5 bits: all of an FP64 value).
+struct TripleFactor {
+  uint64_t x, nx, m, nm, nt;
+};
+struct TripleSum {
+  uint64_t s = 0, c = 0, d = 0;
+  __device__ __forceinline__ void add(const TripleFactor& g, uint64_t v) {
+    const uint64_t p = mul2(g.x, v), pe = fma2(g.nx, v, p);  // pe, qe: errors, negated
+    const uint64_t q = mul2(g.m, v), qe = fma2(g.nt, v, fma2(g.nm, v, q));
+    uint64_t t, e1, e2, e3;
+    s = two_sum2(s, p, t);
+    c = two_sum2(c, t, e1);
+    const uint64_t r = sub2(c, pe), b = sub2(r, c);  // c - pe and its error
+    e2 = sub2(sub2(c, sub2(r, b)), add2(pe, b));
+    c = two_sum2(r, q, e3);
+    d = add2(d, sub2(add2(add2(e1, e2), e3), qe));
+  }
+};
 
-__global__ void __launch_bounds__(kThreads, 2)
+// <phi|psi> = sum_m conj(lo[m]) sum_k conj(hi[k]) psi[k, m]: a thread keeps the inner
+// sums of eight amplitudes of each chunk, so that FP64 is left for their last step.
+//
+// Bound by the FP32 pipe: 66 packed operations an amplitude, 117 us at L = 25 at the
+// pipe's rate, measured 149 us; 84 us at L = 24, 22 us at L = 20.  In two FP32 parts (44
+// scalar operations) 92, 57 and 24 us, but an overlap was off by 6 to 9e-14 of its
+// value (rms, 13 to 20 sites) where it is by 1 to 2e-15 now and was by 1 to 4e-15 in FP64 (741
+// us), and what lies below FP32's range was lost.
+//
+// Where an inner sum is so small that FP32 parts of its terms may have been lost
+// (below 2^-126 each, against 2^-70), or not finite, the thread takes it again in FP64.
+constexpr int kOverlapThreads = 512;
+// (double)f of a normal number or zero, without the FP64 unit; subnormal: zero
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t u = __float_as_uint(f);
+  const bool z = (u & 0x7f800000u) == 0;
+  const uint32_t hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+  return __hiloint2double(z ? 0 : (int)hi, z ? 0 : (int)(u << 29));
+}
+__global__ void __launch_bounds__(kOverlapThreads, 1)
     k_overlap_f32(const float2* __restrict__ psi, int L, const double2* __restrict__ lo,
                   const double2* __restrict__ hi, double* __restrict__ part) {
-  // the thread's 16 entries of the low table: 2 tid + (0, 1) + 512 j
-  float4 g[16];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) g[m] = split_pair(lo[2 * threadIdx.x + 512 * (m >> 1) + (m & 1)]);
-  const uint32_t chunks = 1u << (L - kBits);
-  double acc[2] = {0.0, 0.0};
-  for (uint32_t k = blockIdx.x; k < chunks; k += gridDim.x) {
+  const uint32_t chunks = 1u << (L - kBits), tid = threadIdx.x, lane = tid & 31;
+  auto read = [&](uint32_t k, float4 (&u)[4]) {
     const float4* p = reinterpret_cast<const float4*>(psi + ((uint64_t)k << kBits));
-    float4 u[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) u[j] = __ldg(p + threadIdx.x + kThreads * j);
-    float rs = 0.f, rc = 0.f, is = 0.f, ic = 0.f;
+    for (int j = 0; j < 4; ++j) u[j] = __ldg(p + tid + kOverlapThreads * j);
+  };
+  TripleSum sum[8];
+  float vmax = 0.f, hmax = 0.f;
+  uint32_t any = 0;  // bit m: an amplitude other than zero
+  float4 next[4];
+  if (blockIdx.x < chunks) read(blockIdx.x, next);
+  for (uint32_t k0 = blockIdx.x; k0 < chunks; k0 += 32 * gridDim.x) {
+    // a lane splits the factor of one of the next 32 chunks
+    float part3[2][3] = {};
+    if (k0 + lane * gridDim.x < chunks) {
+      const double2 h = hi[k0 + lane * gridDim.x];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      float2 v[2];
-      unpack(u[j], v);
+      for (int i = 0; i < 2; ++i) {
+        double r = i ? h.y : h.x;
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const float4 f = g[2 * j + q];
-        add_product(f.x, f.y, v[q].x, rs, rc);
-        add_product(f.z, f.w, v[q].y, rs, rc);
-        add_product(f.x, f.y, v[q].y, is, ic);
-        add_product(-f.z, -f.w, v[q].x, is, ic);
+        for (int j = 0; j < 3; ++j) {
+          part3[i][j] = (float)r;
+          r -= (double)part3[i][j];
+        }
+      }
+      hmax = fmaxf(hmax, (h.x != 0.0 || h.y != 0.0) ? 1.f : 0.f);
+    }
+#pragma unroll 1
+    for (uint32_t q = 0; q < 32; ++q) {
+      const uint32_t k = k0 + q * gridDim.x;
+      if (k >= chunks) break;
+      TripleFactor g[2];  // (re, re) and (im, -im)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        float f[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) f[j] = __shfl_sync(0xffffffffu, part3[i][j], q);
+        const float sg = i ? -1.f : 1.f;
+        g[i] = TripleFactor{pk2(f[0], sg * f[0]), pk2(-f[0], -sg * f[0]), pk2(f[1], sg * f[1]),
+                            pk2(-f[1], -sg * f[1]), pk2(-f[2], -sg * f[2])};
+      }
+      float4 u[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) u[j] = next[j];
+      if (k + gridDim.x < chunks) read(k + gridDim.x, next);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        vmax = fmaxf(vmax, fmaxf(fmaxf(fabsf(u[j].x), fabsf(u[j].y)), fmaxf(fabsf(u[j].z), fabsf(u[j].w))));
+        any |= (u[j].x != 0.f || u[j].y != 0.f) ? 1u << 2 * j : 0u;
+        any |= (u[j].z != 0.f || u[j].w != 0.f) ? 2u << 2 * j : 0u;
+        sum[2 * j].add(g[0], pk2(u[j].x, u[j].y));
+        sum[2 * j].add(g[1], pk2(u[j].y, u[j].x));
+        sum[2 * j + 1].add(g[0], pk2(u[j].z, u[j].w));
+        sum[2 * j + 1].add(g[1], pk2(u[j].w, u[j].z));
       }
     }
-    const double re = (double)rs + (double)rc, im = (double)is + (double)ic;
-    const double2 h = hi[k];
-    acc[0] += h.x * re + h.y * im;
-    acc[1] += h.x * im - h.y * re;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) hmax = fmaxf(hmax, __shfl_xor_sync(0xffffffffu, hmax, o));
+  double acc[2] = {0.0, 0.0};
+  const float least = 0x1p-70f * fmaxf(vmax, 1.f);
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    const uint32_t at = 2 * tid + 2 * kOverlapThreads * (m >> 1) + (m & 1);
+    const double2 g = lo[at];
+    const float2 s = un2(sum[m].s), c = un2(sum[m].c), d = un2(sum[m].d);
+    double re = widen(s.x) + (widen(c.x) + widen(d.x));
+    double im = widen(s.y) + (widen(c.y) + widen(d.y));
+    const float size = fabsf(s.x) + fabsf(s.y);
+    // (not where every term is zero; vmax passes over NaN, size does not)
+    if (!(size >= least && size <= 3e38f) && hmax != 0.f && (g.x != 0.0 || g.y != 0.0) &&
+        ((any >> m) & 1)) {
+      re = im = 0.0;
+#pragma unroll 1
+      for (uint32_t k = blockIdx.x; k < chunks; k += gridDim.x) {
+        const float2 v = __ldg(psi + ((uint64_t)k << kBits) + at);
+        const double2 h = hi[k];
+        re += h.x * (double)v.x + h.y * (double)v.y;
+        im += h.x * (double)v.y - h.y * (double)v.x;
+      }
+    }
+    acc[0] += g.x * re + g.y * im;
+    acc[1] += g.x * im - g.y * re;
   }
   block_store_k<2>(acc, part);
 }
@@ -524,11 +608,11 @@ cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h, const c
   return cudaGetLastError();
 }
 
-int observe_overlap_grid(int L, const LaunchCfg& cfg) { return grid_of(L, cfg, 2); }
+int observe_overlap_grid(int L, const LaunchCfg& cfg) { return grid_of(L, cfg, 1); }
 
 cudaError_t launch_overlap_f32(const void* psi, int L, const void* lo, const void* hi, double* part,
                                const LaunchCfg& cfg, cudaStream_t s) {
-  k_overlap_f32<<<observe_overlap_grid(L, cfg), kThreads, 0, s>>>(
+  k_overlap_f32<<<observe_overlap_grid(L, cfg), kOverlapThreads, 0, s>>>(
       static_cast<const float2*>(psi), L, static_cast<const double2*>(lo),
       static_cast<const double2*>(hi), part);
   return cudaGetLastError();

@@ -248,12 +248,6 @@ __device__ __forceinline__ uint64_t swap2(uint64_t v) {
   const float2 t = un2(v);
   return pk2(t.y, t.x);
 }
-// leading part of a + b and its error
-__device__ __forceinline__ uint64_t two_sum2(uint64_t a, uint64_t b, uint64_t& err) {
-  const uint64_t s = add2(a, b), bb = sub2(s, a);
-  err = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
-  return s;
-}
 // acc + g v (s: v swapped): dot2_acc of both components, operation by operation,
 // the errors of the products negated.  kFirst: acc is zero.
 template <bool kFirst>
