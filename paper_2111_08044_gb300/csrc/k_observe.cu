@@ -517,6 +517,15 @@ __device__ __forceinline__ float mul_sub(float ah, float al, float bh, float bl,
   return dot2_acc(df(0.f, 0.f), df(ah, al), df(bh, bl), df(-ch, -cl), df(dh, dl)).hi;
 }
 
+// The thread's amplitudes in `small` again, in FP64 (a call: kept out of the others' way).
+__device__ __noinline__ void factor_small(float2* chunk, const double2* lo, double2 h, uint32_t small) {
+  for (; small; small &= small - 1) {
+    const uint32_t m = __ffs(small) - 1, at = 2 * threadIdx.x + 512 * (m >> 1) + (m & 1);
+    const double2 g = lo[at];
+    chunk[at] = make_float2((float)(g.x * h.x - g.y * h.y), (float)(g.x * h.y + g.y * h.x));
+  }
+}
+
 __global__ void __launch_bounds__(kThreads, 2)
     k_factor_f32(float2* __restrict__ psi, int L, const double2* __restrict__ lo,
                  const double2* __restrict__ hi) {
@@ -526,6 +535,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   const uint32_t chunks = 1u << (L - kBits);
   for (uint32_t k = blockIdx.x; k < chunks; k += gridDim.x) {
     const float4 h = split_pair(hi[k]);
+    uint32_t small = 0;  // bit 2 j + q
     float4* p = reinterpret_cast<float4*>(psi + ((uint64_t)k << kBits));
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -535,9 +545,14 @@ __global__ void __launch_bounds__(kThreads, 2)
         const float4 f = g[2 * j + q];
         o[2 * q] = mul_sub(f.x, f.y, h.x, h.y, f.z, f.w, h.z, h.w);
         o[2 * q + 1] = mul_sub(f.x, f.y, h.z, h.w, -f.z, -f.w, h.x, h.y);
+        // trailing parts or errors of the products below FP32's range
+        small |= (fmaxf(fabsf(o[2 * q]), fabsf(o[2 * q + 1])) < 0x1p-98f && (f.x != 0.f || f.z != 0.f))
+                     ? 1u << (2 * j + q)
+                     : 0u;
       }
       p[threadIdx.x + kThreads * j] = make_float4(o[0], o[1], o[2], o[3]);
     }
+    if (small && (h.x != 0.f || h.z != 0.f)) factor_small(psi + ((uint64_t)k << kBits), lo, hi[k], small);
   }
 }
 

@@ -91,3 +91,23 @@ def test_overlap_of_non_finite_amplitudes(svlib, L):
         sp = np.tile([1.0, 0.0, 1.0, 0.0], (L, 1))
         want = np.float64(np.float32(3e38)) * 2.0 ** (L / 2)
         assert abs(sim.overlap_product(sp).real / want - 1) < 4 * L * EPS
+
+
+@pytest.mark.parametrize("L,eps", [(14, 1.0), (16, 1e-2), (16, 1e-3), (18, 1e-4), (24, 0.03)])
+def test_small_amplitudes_of_pair_states(svlib, L, eps):
+    """Each component rounded once to FP32 (2^-24 of it, 2^-150 where that is subnormal)
+    from FP64 products, off by L + 4 roundings of the amplitude."""
+    from paper_2111_08044_gb300.sim import FloquetSimulator
+    rng = np.random.default_rng(L)
+    pairs = (rng.normal(size=(L // 2, 4)) + 1j * rng.normal(size=(L // 2, 4))) * np.array([1, eps, eps, eps ** 2])
+    pairs[0, 1] = 0
+    with FloquetSimulator(L) as sim:
+        sim.init_pairs(pairs)
+        psi = sim.host_state()
+    want = np.ones(1, dtype=np.clongdouble)
+    for p in pairs:
+        f = p.astype(np.clongdouble) / np.sqrt((np.abs(p.astype(np.clongdouble)) ** 2).sum())
+        want = (f[[0, 2, 1, 3]][:, None] * want[None, :]).reshape(-1)  # memory order 2 b_1 + b_0
+    bound = (L + 4) * EPS * np.abs(want) + 2.0 ** -150
+    for got, x in ((psi.real, want.real), (psi.imag, want.imag)):
+        assert np.all(np.abs(got - x) <= 2.0 ** -24 * np.abs(x) * (1 + 1e-6) + bound)
