@@ -90,7 +90,7 @@ struct FloatSum {
   }
   // (an infinite hi is the sum, its rounding errors are NaN)
   __device__ __forceinline__ void flush(double& acc) {
-    acc += (double)hi + (lo == lo ? (double)lo : 0.0);
+    acc += (double)hi + (double)(lo == lo ? lo : 0.f);
     hi = lo = 0.f;
   }
 };
