@@ -40,6 +40,7 @@ namespace cg = cooperative_groups;
 
 constexpr int kMaxThreads = 256;
 constexpr int kMaxWarps = kMaxThreads / 32;
+static_assert(kShortMaxL == 10, "batch chains here have at least 11 sites");
 constexpr int kMaxDynamic = 224 * 1024;  // of 227 KiB a block, beside the static arrays
 
 __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
@@ -76,7 +77,8 @@ struct Spread {
 template <int kNa>
 __device__ __forceinline__ void measure_final(const ChainArgs& ch, const uint8_t* tile, uint32_t sbuf,
                                               const Spread& sp, uint32_t rank, double& e, double& n) {
-  const int L = ch.L, low = L < 9 ? L : 9;    // sites that tell sums apart
+  constexpr int low = 9;                      // sites that tell sums apart
+  const int L = ch.L;
   const int lt = low - sp.kbits;              // of them in the block's part (rank: pos .. 8)
   const int nk = L - low;                     // sites summed over
   constexpr int kM = 1 << kNa;
@@ -320,11 +322,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     // the period's sums: over the block, then over the cluster in rank 0
     double e = 0.0, n = 0.0;
     if (!kPlain) {
-      switch (L < 9 ? 0 : L - 9) {
-        case 0: measure_final<0>(ch, tile, sbuf, sp, rank, e, n); break;
-        case 1: measure_final<1>(ch, tile, sbuf, sp, rank, e, n); break;
-        case 2: measure_final<2>(ch, tile, sbuf, sp, rank, e, n); break;
-        case 3: measure_final<3>(ch, tile, sbuf, sp, rank, e, n); break;
+      switch (L) {  // more than kShortMaxL sites
+        case 11: measure_final<2>(ch, tile, sbuf, sp, rank, e, n); break;
+        case 12: measure_final<3>(ch, tile, sbuf, sp, rank, e, n); break;
         default: measure_final<4>(ch, tile, sbuf, sp, rank, e, n);
       }
     } else {

@@ -34,7 +34,7 @@ struct sv_ctx {
   int device = 0;
   int precision = SV_C64;
   cudaStream_t stream = nullptr;      // caller's stream
-  cudaStream_t cap_stream = nullptr;  // internal stream used only for capture
+  cudaStream_t cap_stream = nullptr;  // internal stream for captures and for uploads at build time
   fsv::LaunchCfg cfg;
 
   void* state = nullptr;

@@ -62,7 +62,7 @@ struct TilePassPlan {
 
 // The passes of a period in tiles of 2^tb amplitudes (tb >= 4, tb <= L).
 // Gates are taken in the order given; a pass ends where the next gate's
-// sites no longer fit beside the pass's.  pairs: two gates a round.
+// sites no longer fit beside the pass's.  complex64: up to two gates a round.
 // max_gates: gates of a pass (0: the type's).
 std::vector<TilePassPlan> tile_plan(int L, const std::vector<Gate2>& gates, int precision, int tb,
                                     int max_gates = 0);
