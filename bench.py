@@ -28,6 +28,8 @@ if ROOT not in sys.path:
 METRIC = "Floquet periods/s at L=30 c64 (plain vs tensor-core block form), % of roofline"
 UNIT = "periods/s"
 L_BENCH = 30
+# SV_BATCH_* forms
+_FORM_NAMES = {0: "plain", 1: "block_simt", 2: "block_tc", 3: "resident", 4: "multigate"}
 
 
 def _workload(L: int) -> str:
@@ -323,11 +325,10 @@ def _batch(args, local):
     hbm_gbs = _peaks()[0]
     bound_ms = _batch_hbm_bound_ms(chains, forms, widths, hbm_gbs)
     ms_period = ms / args.batch_periods
-    names = {0: "plain", 1: "block_simt", 2: "block_tc", 3: "resident", 4: "multigate"}
     by_L = {}
     for L in sorted(set(Ls.tolist())):
         c = int(np.nonzero(Ls == L)[0][0])
-        by_L[str(L)] = names[int(forms[c])] + (f" n={int(widths[c])}" if widths[c] else "")
+        by_L[str(L)] = _FORM_NAMES[int(forms[c])] + (f" n={int(widths[c])}" if widths[c] else "")
     return {
         "workload": "512 chains, L uniform 14..22, J~U[0.8,1.2] hx~U[0.6,1.0] hz~U[0.2,0.6] "
                     "theta~U[0.1,0.5], random product states (seed 2), complex64",
@@ -336,7 +337,7 @@ def _batch(args, local):
         "ms": ms,
         "create_and_autotune_s": t_create,
         "amplitudes": amps,
-        "forms": {names[k]: int((forms == k).sum()) for k in range(5) if (forms == k).any()},
+        "forms": {_FORM_NAMES[k]: int((forms == k).sum()) for k in range(5) if (forms == k).any()},
         "form_by_L": by_L,
         "norm_max_dev": float(np.abs(n - 1.0).max()),
         "ms_per_period": ms_period,
@@ -432,7 +433,7 @@ FP32_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
 
 def _mg_fp32_tflops(L, form):
-    """Algorithmic FP32 rate of the multi-gate form: each gate costs 32 FMA
+    """Algorithmic FP32 rate of the plain and multi-gate forms: each gate costs 32 FMA
     per amplitude (the FP32 table and its residual), 4(L-1) gates a period."""
     flops = 2.0 * 32 * (1 << L) * form["gates_per_period"]
     return flops * form["periods_per_s"] / 1e12
@@ -493,8 +494,8 @@ def _config(args, world):
 
 def run_batch_breakdown(args):
     """Each L group of the 512-chain preset run alone in the form the full
-    batch gives it (resident at L <= 14, tensor-core groups above): ms per
-    period of the group against its HBM bound, one JSON line per L."""
+    batch gives it (the autotuner's choice for that L): ms per period of the
+    group against its HBM bound, one JSON line per L."""
     import numpy as np
     import torch
 
@@ -506,8 +507,7 @@ def run_batch_breakdown(args):
     periods = 64
     for L in sorted({c.L for c in chains}):
         group = [c for c in chains if c.L == L]
-        form = capi.SV_BATCH_RESIDENT if L <= 14 else capi.SV_BATCH_BLOCK_TC
-        b = FloquetBatch(group, form=form)
+        b = FloquetBatch(group)
         b.evolve(16)
         torch.cuda.synchronize()
         start = torch.cuda.Event(enable_timing=True)
@@ -523,7 +523,7 @@ def run_batch_breakdown(args):
         torch.cuda.empty_cache()
         bound = _batch_hbm_bound_ms(group, forms, widths, hbm_gbs)
         print(json.dumps({"batch_breakdown": True, "L": L, "chains": len(group),
-                          "form": "resident" if form == capi.SV_BATCH_RESIDENT else "block_tc group",
+                          "form": _FORM_NAMES[int(forms[0])],
                           "ms_per_period": ms, "hbm_bound_ms_per_period": bound,
                           "hbm_bound_frac": bound / ms if bound else None}), flush=True)
     return 0
@@ -566,7 +566,7 @@ def run_ours(args):
     plain = _time_form(args, "plain", plain_steps, rank, world, local)
     multigate = _time_form(args, "multigate", mg_steps, rank, world, local)
     ck = clocks.stop()
-    plain.pop("pass_ms_each", None)  # 116 gate passes: the mean is enough
+    plain.pop("pass_ms_each", None)  # 27 tile passes: the mean is enough
     t_block = _max_over_ranks(block["elapsed_ms"], world)
     t_plain = _max_over_ranks(plain["elapsed_ms"], world)
     value = world * args.steps / (t_block / 1e3)
@@ -607,8 +607,11 @@ def run_ours(args):
         "block": {k: block[k] for k in ("periods_per_s", "passes_per_period",
                                         "gates_per_period", "avg_pass_ms", "pass_gbs",
                                         "pass_share", "energy_last", "pass_ms_each")},
+        # its passes hold several gates: the FP32 pipe is their bound, not HBM
         "plain": dict(plain, periods_per_s=plain_value, steps=plain_steps,
-                      roofline_frac=plain["pass_gbs"] / hbm_peak),
+                      hbm_frac=plain["pass_gbs"] / hbm_peak,
+                      fp32_tflops=_mg_fp32_tflops(args.L, plain),
+                      roofline_frac=_mg_fp32_tflops(args.L, plain) / FP32_TFLOPS),
         "multigate": dict(multigate, steps=mg_steps,
                           periods_per_s=world * mg_steps / (
                               _max_over_ranks(multigate["elapsed_ms"], world) / 1e3),
