@@ -7,21 +7,21 @@
 //                   bits of a tile, and the diagonal part.  A pass covers the
 //                   12 lowest sites or 8 further ones, so the state is read
 //                   ceil((L - 12) / 8) + 1 times; one identity gate pass per
-//                   pair of sites read it L / 2 times: 1160 -> 194 us.
+//                   pair of sites read it L / 2 times: 1217 -> 236 us a call.
 //   k_moments_tile  H0 psi amplitude by amplitude, for E and sigma_E (Eq. 10 and
 //   k_bond_moments_tile  11): partners within the tile from registers and shared
 //                   memory, the others from the tiles whose number differs in
 //                   one bit (or, for a general bond term, two), which mostly
 //                   are in L2.  Bound by that traffic: L - 11 tiles read for one
-//                   (Ising, 1230 -> 269 us); general bonds by instructions too
-//                   (L = 24: 1090 -> 393 us).
+//                   (Ising, 1230 -> 285 us); general bonds by instructions too
+//                   (L = 24: 1080 -> 386 us).
 //   k_overlap_f32   <phi|psi> of a product state from FP64 factor tables
 //   k_factor_f32    and the state itself: the FP64 units (0.59 TFMA/s) bounded
 //                   both; products and sums are FP32 triples and pairs here (an
 //                   exact product and its error, Dekker and Knuth): 741 -> 149
-//                   us; L = 24: 188 -> 55 us.
-// Partial sums: FP32 within a thread's tile, FP32 pairs across its terms, FP64
-// across tiles, threads and blocks, in a fixed order.
+//                   us; L = 24: 188 -> 57 us.
+// Partial sums: FP32 over at most eight terms, FP32 pairs (overlaps: triples) across a
+// thread's terms, FP64 across tiles, threads and blocks, in a fixed order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
