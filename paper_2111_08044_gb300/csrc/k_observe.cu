@@ -18,7 +18,7 @@
 //   k_overlap_f32   <phi|psi> of a product state from FP64 factor tables
 //   k_factor_f32    and the state itself: the FP64 units (0.59 TFMA/s) bounded
 //                   both; products and sums are FP32 triples and pairs here (an
-//                   exact product and its error, Dekker and Knuth): 741 -> 149
+//                   exact product and its error, Dekker and Knuth): 741 -> 142
 //                   us; L = 24: 188 -> 57 us.
 // Partial sums: FP32 over at most eight terms, FP32 pairs (overlaps: triples) across a
 // thread's terms, FP64 across tiles, threads and blocks, in a fixed order.
@@ -400,16 +400,26 @@ struct TripleSum {
     c = two_sum2(r, q, e3);
     d = add2(d, sub2(add2(add2(e1, e2), e3), qe));
   }
+  __device__ __forceinline__ void add(const TripleSum& o) {
+    uint64_t t, e1, e2;
+    s = two_sum2(s, o.s, t);
+    c = two_sum2(c, o.c, e1);
+    c = two_sum2(c, t, e2);
+    d = add2(add2(d, o.d), add2(e1, e2));
+  }
 };
 
-// <phi|psi> = sum_m conj(lo[m]) sum_k conj(hi[k]) psi[k, m]: a thread keeps the inner
-// sums of eight amplitudes of each chunk, so that FP64 is left for their last step.
+// <phi|psi> = sum_m conj(lo[m]) sum_k conj(hi[k]) psi[k, m]: a block keeps the inner
+// sums of a quarter of the low indices m, a thread two of them in four parts, over its
+// chunks k.  So FP64 is left for two products a thread (with eight low indices a
+// thread a call at 13 to 18 sites took 60 us, now 50).
 //
 // Bound by the FP32 pipe: 66 packed operations an amplitude, 117 us at L = 25 at the
-// pipe's rate, measured 149 us; 84 us at L = 24, 22 us at L = 20.  In two FP32 parts (44
+// pipe's rate, measured 142 us; 76 us at L = 24, 13 us at L = 20.  In two FP32 parts (44
 // scalar operations) 92, 57 and 24 us, but an overlap was off by 6 to 9e-14 of its
 // value (rms, 13 to 20 sites) where it is by 1 to 2e-15 now and was by 1 to 4e-15 in FP64 (741
-// us), and what lies below FP32's range was lost.
+// us), and what lies below FP32's range was lost.  (A fourth of the sums in FP64 beside
+// them: 130 us, but sparse states then take the sums again.)
 //
 // Where an inner sum is so small that FP32 parts of its terms may have been lost
 // (below 2^-126 each, against 2^-70), or not finite, the thread takes it again in FP64.
@@ -425,21 +435,25 @@ __global__ void __launch_bounds__(kOverlapThreads, 1)
     k_overlap_f32(const float2* __restrict__ psi, int L, const double2* __restrict__ lo,
                   const double2* __restrict__ hi, double* __restrict__ part) {
   const uint32_t chunks = 1u << (L - kBits), tid = threadIdx.x, lane = tid & 31;
-  auto read = [&](uint32_t k, float4 (&u)[4]) {
-    const float4* p = reinterpret_cast<const float4*>(psi + ((uint64_t)k << kBits));
+  const uint32_t slice = blockIdx.x & 3, first = blockIdx.x >> 2, step = gridDim.x >> 2;
+  const uint32_t n = first < chunks ? (chunks - first + step - 1) / step : 0;  // chunks of the block
+  const uint32_t at0 = 2 * kOverlapThreads * slice + 2 * tid;  // the thread's first m
+  auto read = [&](uint32_t i, float4 (&u)[4]) {  // of chunks i .. i + 3 of the block's
 #pragma unroll
-    for (int j = 0; j < 4; ++j) u[j] = __ldg(p + tid + kOverlapThreads * j);
+    for (int j = 0; j < 4; ++j)
+      if (i + j < n)
+        u[j] = __ldg(reinterpret_cast<const float4*>(psi + ((uint64_t)(first + (i + j) * step) << kBits) + at0));
   };
-  TripleSum sum[8];
+  TripleSum sum[4][2];
   float vmax = 0.f, hmax = 0.f;
   uint32_t any = 0;  // bit m: an amplitude other than zero
   float4 next[4];
-  if (blockIdx.x < chunks) read(blockIdx.x, next);
-  for (uint32_t k0 = blockIdx.x; k0 < chunks; k0 += 32 * gridDim.x) {
+  read(0, next);
+  for (uint32_t i0 = 0; i0 < n; i0 += 32) {
     // a lane splits the factor of one of the next 32 chunks
     float part3[2][3] = {};
-    if (k0 + lane * gridDim.x < chunks) {
-      const double2 h = hi[k0 + lane * gridDim.x];
+    if (i0 + lane < n) {
+      const double2 h = hi[first + (i0 + lane) * step];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         double r = i ? h.y : h.x;
@@ -452,32 +466,31 @@ __global__ void __launch_bounds__(kOverlapThreads, 1)
       hmax = fmaxf(hmax, (h.x != 0.0 || h.y != 0.0) ? 1.f : 0.f);
     }
 #pragma unroll 1
-    for (uint32_t q = 0; q < 32; ++q) {
-      const uint32_t k = k0 + q * gridDim.x;
-      if (k >= chunks) break;
-      TripleFactor g[2];  // (re, re) and (im, -im)
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        float f[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) f[j] = __shfl_sync(0xffffffffu, part3[i][j], q);
-        const float sg = i ? -1.f : 1.f;
-        g[i] = TripleFactor{pk2(f[0], sg * f[0]), pk2(-f[0], -sg * f[0]), pk2(f[1], sg * f[1]),
-                            pk2(-f[1], -sg * f[1]), pk2(-f[2], -sg * f[2])};
-      }
+    for (uint32_t i = i0; i < n && i < i0 + 32; i += 4) {
       float4 u[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) u[j] = next[j];
-      if (k + gridDim.x < chunks) read(k + gridDim.x, next);
+      read(i + 4, next);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
+        if (i + j >= n) break;
+        TripleFactor g[2];  // (re, re) and (im, -im)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          float f[3];
+#pragma unroll
+          for (int q = 0; q < 3; ++q) f[q] = __shfl_sync(0xffffffffu, part3[k][q], i - i0 + j);
+          const float sg = k ? -1.f : 1.f;
+          g[k] = TripleFactor{pk2(f[0], sg * f[0]), pk2(-f[0], -sg * f[0]), pk2(f[1], sg * f[1]),
+                              pk2(-f[1], -sg * f[1]), pk2(-f[2], -sg * f[2])};
+        }
         vmax = fmaxf(vmax, fmaxf(fmaxf(fabsf(u[j].x), fabsf(u[j].y)), fmaxf(fabsf(u[j].z), fabsf(u[j].w))));
-        any |= (u[j].x != 0.f || u[j].y != 0.f) ? 1u << 2 * j : 0u;
-        any |= (u[j].z != 0.f || u[j].w != 0.f) ? 2u << 2 * j : 0u;
-        sum[2 * j].add(g[0], pk2(u[j].x, u[j].y));
-        sum[2 * j].add(g[1], pk2(u[j].y, u[j].x));
-        sum[2 * j + 1].add(g[0], pk2(u[j].z, u[j].w));
-        sum[2 * j + 1].add(g[1], pk2(u[j].w, u[j].z));
+        any |= (u[j].x != 0.f || u[j].y != 0.f) ? 1u : 0u;
+        any |= (u[j].z != 0.f || u[j].w != 0.f) ? 2u : 0u;
+        sum[j][0].add(g[0], pk2(u[j].x, u[j].y));
+        sum[j][0].add(g[1], pk2(u[j].y, u[j].x));
+        sum[j][1].add(g[0], pk2(u[j].z, u[j].w));
+        sum[j][1].add(g[1], pk2(u[j].w, u[j].z));
       }
     }
   }
@@ -486,10 +499,13 @@ __global__ void __launch_bounds__(kOverlapThreads, 1)
   double acc[2] = {0.0, 0.0};
   const float least = 0x1p-70f * fmaxf(vmax, 1.f);
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    const uint32_t at = 2 * tid + 2 * kOverlapThreads * (m >> 1) + (m & 1);
+  for (int m = 0; m < 2; ++m) {
+    const uint32_t at = at0 + m;
     const double2 g = lo[at];
-    const float2 s = un2(sum[m].s), c = un2(sum[m].c), d = un2(sum[m].d);
+    sum[0][m].add(sum[1][m]);
+    sum[2][m].add(sum[3][m]);
+    sum[0][m].add(sum[2][m]);
+    const float2 s = un2(sum[0][m].s), c = un2(sum[0][m].c), d = un2(sum[0][m].d);
     double re = widen(s.x) + (widen(c.x) + widen(d.x));
     double im = widen(s.y) + (widen(c.y) + widen(d.y));
     const float size = fabsf(s.x) + fabsf(s.y);
@@ -498,7 +514,7 @@ __global__ void __launch_bounds__(kOverlapThreads, 1)
         ((any >> m) & 1)) {
       re = im = 0.0;
 #pragma unroll 1
-      for (uint32_t k = blockIdx.x; k < chunks; k += gridDim.x) {
+      for (uint32_t k = first; k < chunks; k += step) {
         const float2 v = __ldg(psi + ((uint64_t)k << kBits) + at);
         const double2 h = hi[k];
         re += h.x * (double)v.x + h.y * (double)v.y;
@@ -623,7 +639,10 @@ cudaError_t launch_moments_tile(const void* psi, int L, const H0Coef& h, const c
   return cudaGetLastError();
 }
 
-int observe_overlap_grid(int L, const LaunchCfg& cfg) { return grid_of(L, cfg, 1); }
+int observe_overlap_grid(int L, const LaunchCfg& cfg) {
+  // four quarters of the low indices
+  return 4 * (int)std::min<uint64_t>(1ull << (L - kBits), (uint64_t)std::max(1, cfg.num_sms / 4));
+}
 
 cudaError_t launch_overlap_f32(const void* psi, int L, const void* lo, const void* hi, double* part,
                                const LaunchCfg& cfg, cudaStream_t s) {
