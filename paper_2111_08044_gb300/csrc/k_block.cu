@@ -394,7 +394,7 @@ int block_build(int L, const std::vector<Gate2>& gates, const Observable& obs, i
   }
   const size_t pbytes = sizeof(double) * 2 * std::max(1, bp->nslots) * (size_t)bp->maxb;
   if (cudaMalloc(&bp->d_partials, pbytes) != cudaSuccess ||
-      upload_zeros(bp->d_partials, pbytes, s) != cudaSuccess) {
+      cudaMemsetAsync(bp->d_partials, 0, pbytes, s) != cudaSuccess) {
     cudaGetLastError();
     *msg = "partials allocation failed";
     block_free(bp);
@@ -412,16 +412,16 @@ int block_build(int L, const std::vector<Gate2>& gates, const Observable& obs, i
   }
   if (bp->tensor_cores) {
     if (block_tc_prepare() != cudaSuccess || cudaMalloc(&bp->d_status, sizeof(int)) != cudaSuccess ||
-        upload_zeros(bp->d_status, sizeof(int), s) != cudaSuccess) {
+        cudaMemsetAsync(bp->d_status, 0, sizeof(int), s) != cudaSuccess) {
       cudaGetLastError();
       *msg = "tensor-core pass set-up failed";
       block_free(bp);
       return SV_ECUDA;
     }
   }
-  if (prepare_simt(n) != cudaSuccess) {
+  if (prepare_simt(n) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
     cudaGetLastError();
-    *msg = "shared-memory opt-in failed";
+    *msg = "shared-memory opt-in or upload failed";
     block_free(bp);
     return SV_ECUDA;
   }

@@ -1356,6 +1356,9 @@ int sv_create(sv_ctx** out, int device, int precision, void* cuda_stream) {
   ok = ok && cudaMalloc(&ctx->d_ident, 16 * fsv::kGateEntries) == cudaSuccess;
   ok = ok && cudaMalloc(&ctx->d_part_meas, sizeof(double) * 2 * ctx->maxb *
                                                ctx->part_slots_meas) == cudaSuccess;
+  // (the upload behind them waits for both)
+  ok = ok && cudaMemsetAsync(ctx->d_counter, 0, sizeof(long long), ctx->cap_stream) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(ctx->d_ring, 0, sizeof(double) * 2 * kRing, ctx->cap_stream) == cudaSuccess;
   if (ok) {
     if (precision == SV_C128) {
       double2 id[fsv::kGateEntries] = {};  // identity, zero residual
@@ -1370,8 +1373,6 @@ int sv_create(sv_ctx** out, int device, int precision, void* cuda_stream) {
       for (int k = 0; k < 4; ++k) id[5 * k].x = 1.0f;
       ok = fsv::upload(ctx->d_ident, id, sizeof(id), ctx->cap_stream) == cudaSuccess;
     }
-    ok = ok && fsv::upload_zeros(ctx->d_counter, sizeof(long long), ctx->cap_stream) == cudaSuccess;
-    ok = ok && fsv::upload_zeros(ctx->d_ring, sizeof(double) * 2 * kRing, ctx->cap_stream) == cudaSuccess;
   }
   if (!ok) {
     cudaGetLastError();

@@ -107,10 +107,6 @@ inline cudaError_t upload(void* to, const void* from, size_t bytes, cudaStream_t
   const cudaError_t e = cudaMemcpyAsync(to, from, bytes, cudaMemcpyHostToDevice, s);
   return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
-inline cudaError_t upload_zeros(void* to, size_t bytes, cudaStream_t s) {
-  const cudaError_t e = cudaMemsetAsync(to, 0, bytes, s);
-  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
-}
 
 // Grid (blocks of 256 threads) used by the plain gate pass for this L and
 // bond; it is also the number of partial pairs the pass writes.
